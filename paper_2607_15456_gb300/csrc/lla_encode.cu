@@ -329,7 +329,7 @@ lla_status launch_encode_layers(const EncodeArgs *a, int L, cudaStream_t stream)
     if (L <= 0 || a[0].N == 0) return LLA_OK;
     const EncodeArgs &a0 = a[0];
     // prompts take the tensor-core kernel layer by layer; decode batches share one launch
-    if (encode_tc_supported(a0) || a0.dense || L > kMaxEncodeLayers) {
+    if (encode_tc_layers(a0) || a0.dense || L > kMaxEncodeLayers) {
         for (int l = 0; l < L; ++l) {
             const lla_status st = launch_encode(a[l], stream);
             if (st != LLA_OK) return st;

@@ -4,12 +4,13 @@
 // A unit is (head h, tile of 128 tokens, column group g of one axis):
 //   C[128 x R] = X[128 x T*d] W_down[T*d x R] - mu W_down,
 // with X the stacked loop vectors of the tile's tokens (row n, column t*d + e = x_t[n][h][e]).
-// An axis of rank r is cut into equal column groups of at most 192 columns (320 = 2 x 160).
-// Units are numbered head-major, then tile, then group (K groups first): one CTA per SM takes an
-// equal contiguous range of them, so the groups of a tile follow one another on the same SM and
-// the second read of a tile's x_v hits L2, and a CTA meets few heads (the bias mu W_down is
-// computed once per head it meets).  bf16 operands, fp32 accumulation in TMEM, latents rounded
-// to bf16 and scattered to each token's slot.  Warp roles:
+// LLA-2D is the case of one head of width H*d.  An axis of rank r is cut into ceil(r / 192) column
+// groups of equal width (a multiple of 16; the columns of the last group past r read as zeros and
+// are not stored).  Units are numbered head-major, then tile, then group (K groups first): one CTA
+// per SM takes an equal contiguous range of them, so the groups of a tile follow one another on the
+// same SM and the second read of a tile's x_v hits L2, and a CTA meets few heads (the bias
+// mu W_down of a group is computed once per head the CTA meets).  bf16 operands, fp32 accumulation
+// in TMEM, latents rounded to bf16 and scattered to each token's slot.  Warp roles:
 //   warp 0     x producer: per slab of 64 reduction rows, a TMA tensor load with 128-byte swizzle
 //              of the x tile (one box of 128 tokens x 64 elements: a K-major operand) into its
 //              own ring, which runs on across units
@@ -22,6 +23,23 @@
 //   warps 2-5  epilogue: one token row per thread, TMEM -> bias -> bf16 -> the paged cache (V-plane
 //              rows pass through a per-warp staging buffer, so a store writes 8 rows of 64 bytes)
 // Tokens past N read as zeros (tensor-map fill) and are not stored.
+//
+// Few units with a long reduction (LLA-2D prompts: T*H*d = 8192 rows, N/128 tiles) are split over
+// clusters of up to 8 CTAs: each CTA reduces its share of the rows, then writes its accumulators,
+// column range by column range, into the shared memory of the CTA that owns the range (the rings
+// are idle by then), which adds the parts in rank order and stores.
+//
+// Rows of W_down that are not a multiple of 16 bytes (r = 18, 30) have no tensor map: with WRES the
+// epilogue warps copy the head's whole W_down of an axis (ranks up to 64, T*d up to 512) into
+// shared memory, zero-padded to a multiple of 32 columns, in the layout the boxes would have, when
+// the CTA first meets that head and axis.
+//
+// Bound: HBM for per-head prompts (x is read once; 41.7 us of bytes for 7208 tokens at (72, 120)),
+// the L2 -> shared memory stream for LLA-2D (a 128 x 192 unit moves 40 KB per 64 rows).  Measured
+// against the CUDA-core kernel, which these shapes took before: 7208 tokens at (72, 120) with mu
+// 1690 -> 60.6 us; 8000 tokens at (18, 30) 516 -> 62 us (150 tokens: 17.4 -> 7.9 us); LLA-2D
+// (288, 480), 1500 tokens 4864 -> 32 us, 16 tokens 63 -> 16 us; and the bias in slices, 8000 tokens
+// at (96, 160) with mu 188 -> 73 us (63 us without).
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -36,7 +54,10 @@ constexpr int kEM = 128;             // tokens per tile
 constexpr int kES = 64;              // reduction rows per slab
 constexpr int kEThreads = 224;
 constexpr int kMaxGroup = 192;       // columns of a group
-constexpr int kMaxGroups = 6;        // groups of both axes (ranks up to 512: at most 3 each)
+constexpr int kMaxGroups = 20;       // groups of both axes (LLA-2D (1152, 1920): 6 + 10)
+constexpr int kMaxSplit = 8;         // CTAs that share one unit's reduction
+constexpr int kLongReduction = 4096; // reduction rows from which small batches take this kernel too
+constexpr int kResSlabs = 8;         // WRES: most slabs (T*d = 512 rows) kept resident
 constexpr int kASlab = kEM * kES * 2;   // x slab (16 KB)
 constexpr int kBAtom = kES * 128;       // one W_down atom of 64 columns (8 KB)
 constexpr int kWStage = 3 * kBAtom;          // 24 KB
@@ -45,18 +66,25 @@ constexpr int kWStages = 5;                 // W_down slabs in flight (from L2)
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSlotCols = 256;  // accumulator slot s at column s * 256
 constexpr int oW = kXStages * kASlab;
-constexpr int oBias = oW + kWStages * kWStage;
-constexpr int oStg = oBias + kMaxGroups * kMaxGroup * 4;   // V-plane store staging: 4 warps x 32 rows x 80 B
-constexpr int oBar = oStg + 4 * 32 * 80;
-constexpr int kNumBars = 2 * kXStages + 2 * kWStages + 4 + 1;
-constexpr int kSmem = 1024 + oBar + kNumBars * 8 + 16;  // + alignment slack, abort flag, TMEM slot
-static_assert(kSmem <= 227 * 1024, "shared memory");
+template <bool WRES>
+struct EL {  // shared-memory plan: x ring, W_down (ring or resident), biases, V staging, barriers
+    static constexpr int GROUPS = WRES ? 2 : kMaxGroups;
+    static constexpr int oBias = oW + (WRES ? 2 * kResSlabs * kBAtom : kWStages * kWStage);
+    static constexpr int oStg = oBias + GROUPS * kMaxGroup * 4;  // 4 warps x 32 rows x 80 B
+    static constexpr int oBar = oStg + 4 * 32 * 80;
+    static constexpr int NBAR = 2 * kXStages + 2 * kWStages + 4 + 1;
+    static constexpr int SMEM = 1024 + oBar + NBAR * 8 + 16;  // + alignment slack, abort flag, TMEM slot
+    static_assert(SMEM <= 227 * 1024, "shared memory");
+};
+// split units: parts of one column range, [rank][column / 4][row] float4 (over the idle rings)
+static_assert(kMaxSplit * kEM * 32 * 4 <= EL<false>::oBias && 2 * kEM * 96 * 4 <= EL<false>::oBias, "exchange area");
 
 struct ETParams {
     int T, H, d, N;
     int r_k, r_v;
     int nk, nv;      // column groups of each axis
-    int gk, gv;      // columns per group of each axis
+    int gk, gv;      // columns per group of each axis (the last group of an axis may hold fewer)
+    int split;       // CTAs per unit (a cluster); 1: no split
     int tiles;       // ceil(N / 128)
     int64_t units;   // H * tiles * (nk + nv)
     const float *mu_k, *mu_v;           // [H][T*d] or NULL
@@ -64,12 +92,13 @@ struct ETParams {
     char *pool;
     int64_t num_blocks, block_bytes;
     int head_page_bytes, kplane_bytes;
+    int gran;        // bytes of a K-plane granule: 16, or 4 when a K row is not whole 16-byte words
     const int64_t *slot_mapping;
     unsigned *err;
 };
 
 struct Unit {
-    int h, n0, axis, col0, R;
+    int h, n0, axis, col0, R, cols, g;  // R: columns of the product, cols: columns that exist
 };
 
 __device__ __forceinline__ Unit unit_of(const ETParams &p, int64_t u) {
@@ -78,24 +107,107 @@ __device__ __forceinline__ Unit unit_of(const ETParams &p, int64_t u) {
     Unit U;
     U.h = static_cast<int>(u / per_head);
     const int rem = static_cast<int>(u - U.h * per_head);
-    const int tile = rem / G, g = rem - tile * G;
+    const int tile = rem / G;
+    U.g = rem - tile * G;
     U.n0 = tile * kEM;
-    U.axis = g < p.nk ? 0 : 1;
-    const int ga = U.axis ? g - p.nk : g;
-    U.R = U.axis ? p.gv : p.gk;
-    U.col0 = ga * U.R;
+    U.axis = U.g < p.nk ? 0 : 1;
+    const int ga = U.axis ? U.g - p.nk : U.g;
+    const int w = U.axis ? p.gv : p.gk;
+    U.col0 = ga * w;
+    U.cols = min(w, (U.axis ? p.r_v : p.r_k) - U.col0);
+    U.R = (U.cols + 15) & ~15;
     return U;
 }
 
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster_f4(uint32_t local_addr, uint32_t rank, float4 v) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, %1;\n\t"
+        "st.shared::cluster.v4.f32 [ra], {%2, %3, %4, %5};\n\t}" ::"r"(local_addr),
+        "r"(rank), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+        : "memory");
+}
+
+// mu W_down over reduction rows [k0, k1) for the columns of unit U, into bs[0 .. cols): EPL columns
+// (8, or 2 when the rows of W_down are not whole 16-byte words) per thread and the rows cut into as
+// many slices as the 128 epilogue threads allow, sixteen rows' loads in flight each (one thread per
+// eight columns over all rows took tens of microseconds).  scr: at least 128 * EPL floats.
+template <int EPL>
+__device__ void group_bias(const uint16_t *W, const float *mu, int r, const Unit &U, int k0, int k1, int et,
+                           float *scr, float *bs) {
+    const int nch = (U.cols + EPL - 1) / EPL;  // at most 24 (EPL = 8), 32 (EPL = 2)
+    const int nsl = 128 / nch;
+    const int ch = et % nch, sl = et / nch;
+    float acc[EPL];
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) acc[i] = 0.f;
+    if (sl < nsl) {
+        const uint16_t *Wc = W + U.col0 + ch * EPL;
+#pragma unroll 16
+        for (int k = k0 + sl; k < k1; k += nsl) {
+            const float mk = mu[k];
+            uint32_t w[EPL / 2];
+            if constexpr (EPL == 8) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(Wc + static_cast<int64_t>(k) * r);
+                w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+            } else {
+                w[0] = *reinterpret_cast<const uint32_t *>(Wc + static_cast<int64_t>(k) * r);
+            }
+#pragma unroll
+            for (int i = 0; i < EPL / 2; ++i) {
+                const float2 f = bf2_to_f2(w[i]);
+                acc[2 * i] = fmaf(mk, f.x, acc[2 * i]);
+                acc[2 * i + 1] = fmaf(mk, f.y, acc[2 * i + 1]);
+            }
+        }
+    }
+    named_bar_sync(1, 128);  // scr and bs are free
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) scr[et * EPL + i] = acc[i];
+    named_bar_sync(1, 128);
+    for (int c = et; c < U.cols; c += 128) {
+        float v = 0.f;
+        for (int q = 0; q < nsl; ++q) v += scr[(q * nch + c / EPL) * EPL + c % EPL];
+        bs[c] = v;
+    }
+    named_bar_sync(1, 128);
+}
+
+// Where token row `row` of unit U goes: its K-plane row or V-plane row in the page of its slot (NULL:
+// past N, skipped, or outside the pool).
+__device__ __forceinline__ char *row_dst(const ETParams &p, const Unit &U, int row, bool flag) {
+    const int n = U.n0 + row;
+    if (n >= p.N) return nullptr;
+    const int64_t slot_id = p.slot_mapping[n];
+    if (slot_id < 0) return nullptr;
+    const int64_t blk = slot_id / kBlockTokens;
+    const int r_in = static_cast<int>(slot_id % kBlockTokens);
+    if (blk >= p.num_blocks) {
+        if (flag) atomicOr(p.err, LLA_DEVERR_SLOT);
+        return nullptr;
+    }
+    char *page = p.pool + blk * p.block_bytes + static_cast<int64_t>(U.h) * p.head_page_bytes;
+    return U.axis == 0 ? page + r_in * p.gran : page + p.kplane_bytes + static_cast<int64_t>(r_in) * p.r_v * 2;
+}
+
+template <bool WRES>
 __global__ void __launch_bounds__(kEThreads, 1)
     encode_tc_kernel(const __grid_constant__ CUtensorMap txk, const __grid_constant__ CUtensorMap txv,
                      const __grid_constant__ CUtensorMap twk, const __grid_constant__ CUtensorMap twv,
                      const ETParams p) {
+    using L = EL<WRES>;
     extern __shared__ __align__(1024) char sm_raw[];
     // 128-byte swizzle atoms need a 1024-byte aligned base
     char *sm = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    float *bias = reinterpret_cast<float *>(sm + oBias);  // [group][192] of the current head
-    uint64_t *full = reinterpret_cast<uint64_t *>(sm + oBar);
+    float *bias = reinterpret_cast<float *>(sm + L::oBias);  // [group][192] of the current head
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + L::oBar);
     uint64_t *empty = full + kXStages;
     uint64_t *wfull = empty + kXStages;
     uint64_t *wempty = wfull + kWStages;
@@ -105,10 +217,14 @@ __global__ void __launch_bounds__(kEThreads, 1)
     volatile int *abort_flag = reinterpret_cast<volatile int *>(done + 1);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1) + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t u0 = static_cast<int64_t>(blockIdx.x) * p.units / gridDim.x;
-    const int64_t u1 = static_cast<int64_t>(blockIdx.x + 1) * p.units / gridDim.x;
+    const bool split = p.split > 1;
+    const int64_t u0 = split ? blockIdx.x / p.split : static_cast<int64_t>(blockIdx.x) * p.units / gridDim.x;
+    const int64_t u1 = split ? u0 + 1 : static_cast<int64_t>(blockIdx.x + 1) * p.units / gridDim.x;
     const int Td = p.T * p.d;
-    const int NS = Td / kES;
+    // slabs of the reduction of this CTA
+    const int crank = split ? static_cast<int>(cluster_rank()) : 0;
+    const int S0 = crank * (Td / kES) / p.split, S1 = (crank + 1) * (Td / kES) / p.split;
+    const int NS = S1 - S0;
 
     if (tid == 0) {
         for (int s = 0; s < kXStages; ++s) {
@@ -116,7 +232,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
             mbar_init(&empty[s], 1);
         }
         for (int s = 0; s < kWStages; ++s) {
-            mbar_init(&wfull[s], 1);
+            mbar_init(&wfull[s], WRES ? 128 : 1);  // resident: the epilogue warps' copy (one per axis)
             mbar_init(&wempty[s], 1);
         }
         for (int s = 0; s < 2; ++s) {
@@ -128,13 +244,17 @@ __global__ void __launch_bounds__(kEThreads, 1)
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tslot, kTmemCols);
+    if constexpr (WRES) {  // the padding columns of the resident W_down
+        for (int i = tid; i < 2 * kResSlabs * kBAtom / 16; i += kEThreads)
+            reinterpret_cast<uint4 *>(sm + oW)[i] = make_uint4(0, 0, 0, 0);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
     pdl_wait();  // x, slots and the pool may come from the previous kernel
 
-    if (warp == 0 || warp == 6) {
+    if (warp == 0 || (warp == 6 && !WRES)) {
         // ------------------------------------------------------------ producers: x (0), W (6)
         const bool isx = warp == 0;
         const int NST = isx ? kXStages : kWStages;
@@ -144,7 +264,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
         bool stop = false;
         for (int64_t u = u0; u < u1 && !stop; ++u) {
             const Unit U = unit_of(p, u);
-            const int atoms = (U.R + 63) / 64;
+            const int atoms = (U.cols + 63) / 64;
             const CUtensorMap *tx = U.axis ? &txv : &txk;
             const CUtensorMap *tw = U.axis ? &twv : &twk;
             for (int s = 0; s < NS; ++s) {
@@ -160,7 +280,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
                     break;
                 }
                 __syncwarp();
-                const int k0 = s * kES, t = k0 / p.d, e0 = k0 - t * p.d;
+                const int k0 = (S0 + s) * kES, t = k0 / p.d, e0 = k0 - t * p.d;
                 if (isx) {
                     if (lane == 0) tma_load_4d(sm + st * kASlab, tx, e0, U.h, U.n0, t, &F[st]);
                 } else {
@@ -178,9 +298,21 @@ __global__ void __launch_bounds__(kEThreads, 1)
         // ------------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t base = smem_addr(sm);
-            int q = 0, j = 0;
+            int q = 0, j = 0, head = -1;
+            int nres[2] = {0, 0};               // WRES: copies of each axis's W_down seen
+            bool wax[2] = {false, false};
             for (int64_t u = u0; u < u1; ++u, ++j) {
                 const Unit U = unit_of(p, u);
+                if constexpr (WRES) {  // the head's W_down of this axis is in shared memory
+                    if (U.h != head) {
+                        head = U.h;
+                        wax[0] = wax[1] = false;
+                    }
+                    if (!wax[U.axis]) {
+                        wax[U.axis] = true;
+                        if (!mbar_wait(&wfull[U.axis], nres[U.axis]++ & 1, abort_flag, p.err)) break;
+                    }
+                }
                 const uint32_t idesc = umma_idesc_bf16(128, U.R, 0, 1);
                 const int slot = j & 1;
                 // the epilogue has read this slot's previous unit (j - 2)
@@ -192,18 +324,18 @@ __global__ void __launch_bounds__(kEThreads, 1)
                 for (int s = 0; s < NS; ++s, ++q) {
                     const int st = q % kXStages, sw = q % kWStages;
                     if (!mbar_wait(&full[st], (q / kXStages) & 1, abort_flag, p.err) ||
-                        !mbar_wait(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err)) {
+                        (!WRES && !mbar_wait(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err))) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t a = base + st * kASlab, b = base + oW + sw * kWStage;
+                    const uint32_t a = base + st * kASlab, b = base + oW + (WRES ? (U.axis * kResSlabs + s) * kBAtom : sw * kWStage);
 #pragma unroll
                     for (int ks = 0; ks < kES / 16; ++ks)
                         umma_bf16(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
                                   idesc, s > 0 || ks > 0);
                     umma_commit(&empty[st]);
-                    umma_commit(&wempty[sw]);
+                    if (!WRES) umma_commit(&wempty[sw]);
                 }
                 if (!ok) break;
                 umma_commit(&accfull[slot]);
@@ -219,70 +351,105 @@ __global__ void __launch_bounds__(kEThreads, 1)
         const int et = tid - 64;  // 0..127
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
-        int bias_head = -1;
+        int head = -1;
+        uint32_t have = 0;  // groups whose bias of this head is in `bias`
+        bool wax[2] = {false, false};  // WRES: axes whose W_down of this head is resident
         int j = 0;
         for (int64_t u = u0; u < u1; ++u, ++j) {
             const Unit U = unit_of(p, u);
             const int slot = j & 1;
-            const int g = (U.axis ? p.nk : 0) + U.col0 / U.R;
-            if ((p.mu_k || p.mu_v) && U.h != bias_head) {
-                // mu W_down of every group of this head, eight columns per thread at a time
-                named_bar_sync(1, 128);  // the previous head's biases are no longer read
-                for (int ax = 0; ax < 2; ++ax) {
-                    const float *mu = ax ? p.mu_v : p.mu_k;
-                    const int r = ax ? p.r_v : p.r_k, R = ax ? p.gv : p.gk, gbase = ax ? p.nk : 0;
-                    const uint16_t *W = static_cast<const uint16_t *>(ax ? p.w_down_v : p.w_down_k) +
-                                        static_cast<int64_t>(U.h) * Td * r;
-                    for (int c8 = et; c8 < r / 8; c8 += 128) {
-                        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                        if (mu) {
-                            const float *m = mu + static_cast<int64_t>(U.h) * Td;
-#pragma unroll 4
-                            for (int k = 0; k < Td; ++k) {
-                                const uint4 w = *reinterpret_cast<const uint4 *>(W + static_cast<int64_t>(k) * r + c8 * 8);
-                                const float mk = m[k];
-                                const float2 w0 = bf2_to_f2(w.x), w1 = bf2_to_f2(w.y), w2 = bf2_to_f2(w.z), w3 = bf2_to_f2(w.w);
-                                acc[0] = fmaf(mk, w0.x, acc[0]); acc[1] = fmaf(mk, w0.y, acc[1]);
-                                acc[2] = fmaf(mk, w1.x, acc[2]); acc[3] = fmaf(mk, w1.y, acc[3]);
-                                acc[4] = fmaf(mk, w2.x, acc[4]); acc[5] = fmaf(mk, w2.y, acc[5]);
-                                acc[6] = fmaf(mk, w3.x, acc[6]); acc[7] = fmaf(mk, w3.y, acc[7]);
-                            }
-                        }
-                        for (int i = 0; i < 8; ++i) {
-                            const int c = c8 * 8 + i;
-                            bias[(gbase + c / R) * kMaxGroup + c % R] = acc[i];
+            if (U.h != head) {
+                head = U.h;
+                have = 0;
+                wax[0] = wax[1] = false;
+            }
+            if (WRES && !wax[U.axis]) {
+                // this axis's W_down of the head, pairs of columns (zeros past r from the start): slab s at
+                // s * kBAtom, row k % 64 of 128 bytes, 16-byte chunk c at c ^ (k % 8).  Every product
+                // of the previous head has completed: its last accumulator has been read.
+                wax[U.axis] = true;
+                const int r = U.axis ? p.r_v : p.r_k, hp = r / 2;
+                // 16-byte loads of the contiguous rows, up to sixteen in flight per thread, and four
+                // 4-byte stores each (4-byte loads of padded rows took 8 us a head: 15 -> 8 us a call)
+                const uint4 *W = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(U.axis ? p.w_down_v : p.w_down_k) +
+                                                                 static_cast<int64_t>(U.h) * Td * r);
+                char *dst = sm + oW + U.axis * (kResSlabs * kBAtom);
+                const uint32_t inv = (1u << 20) / hp + 1;  // q / hp = q * inv >> 20 below 512 rows of 32 pairs
+                for (int i0 = et; i0 < Td * r / 8; i0 += 128 * 16) {
+                    uint4 v[16];
+#pragma unroll
+                    for (int b = 0; b < 16; ++b)
+                        if (i0 + b * 128 < Td * r / 8) v[b] = W[i0 + b * 128];
+#pragma unroll
+                    for (int b = 0; b < 16; ++b) {
+                        if (i0 + b * 128 >= Td * r / 8) break;
+                        const uint32_t wd[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const uint32_t q = (i0 + b * 128) * 4 + e;  // pair q: row q / hp
+                            const uint32_t k = static_cast<uint32_t>((static_cast<uint64_t>(q) * inv) >> 20), c = q - k * hp;
+                            *reinterpret_cast<uint32_t *>(dst + k * 128 + (((c >> 2) ^ (k & 7)) << 4) + (c & 3) * 4) = wd[e];
                         }
                     }
                 }
-                named_bar_sync(1, 128);
-                bias_head = U.h;
+                fence_proxy_async_smem();
+                mbar_arrive(&wfull[U.axis]);
             }
-            const float *bs = bias + g * kMaxGroup;
-            const bool use_bias = (U.axis ? p.mu_v : p.mu_k) != nullptr;
-            const int n = U.n0 + row;
-            char *dst = nullptr;
-            if (n < p.N) {
-                const int64_t slot_id = p.slot_mapping[n];
-                if (slot_id >= 0) {
-                    const int64_t blk = slot_id / kBlockTokens;
-                    const int r_in = static_cast<int>(slot_id % kBlockTokens);
-                    if (blk >= p.num_blocks) {
-                        if (g == 0) atomicOr(p.err, LLA_DEVERR_SLOT);
-                    } else {
-                        char *page = p.pool + blk * p.block_bytes + static_cast<int64_t>(U.h) * p.head_page_bytes;
-                        dst = U.axis == 0 ? page + r_in * 16
-                                          : page + p.kplane_bytes + static_cast<int64_t>(r_in) * p.r_v * 2;
-                    }
-                }
+            char *stg = sm + L::oStg + quarter * (32 * 80);
+            float *bs = bias + U.g * kMaxGroup;
+            const float *mu = U.axis ? p.mu_v : p.mu_k;
+            if (mu && !(have >> U.g & 1u)) {
+                have |= 1u << U.g;
+                const int r = U.axis ? p.r_v : p.r_k;
+                const uint16_t *W = static_cast<const uint16_t *>(U.axis ? p.w_down_v : p.w_down_k) +
+                                    static_cast<int64_t>(U.h) * Td * r;
+                group_bias<WRES ? 2 : 8>(W, mu + static_cast<int64_t>(U.h) * Td, r, U, S0 * kES, S1 * kES, et,
+                                         reinterpret_cast<float *>(sm + L::oStg), bs);
             }
+            const bool use_bias = mu != nullptr;
+            if (split) break;  // the parts meet below
+            char *dst = row_dst(p, U, row, U.g == 0);
             mbar_wait(&accfull[slot], (j >> 1) & 1, abort_flag, p.err);
             tc_fence_after();
             const uint32_t tl = tmem + slot * kSlotCols + (static_cast<uint32_t>(quarter * 32) << 16);
-            char *stg = sm + oStg + quarter * (32 * 80);
 #pragma unroll 1
-            for (int c0 = 0; c0 < U.R; c0 += 32) {
+            for (int c0 = 0; c0 < U.cols; c0 += 32) {
                 float v[32];
                 tmem_ld32(tl + c0, v);  // warp-collective: every lane loads, valid rows store
+                if constexpr (WRES) {
+                    // rows that are not whole 16-byte words: pairs of columns.  K: consecutive rows
+                    // are consecutive granules.  V: the warp's 32 rows through the staging buffer, so
+                    // that a store writes neighbouring pairs.
+                    const int np = min(32, U.cols - c0) / 2;
+                    uint32_t w[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const int c = c0 + 2 * k;
+                        w[k] = use_bias ? pack_bf16(v[2 * k] - bs[c], v[2 * k + 1] - bs[c + 1]) : pack_bf16(v[2 * k], v[2 * k + 1]);
+                    }
+                    if (U.axis == 0) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const int c = c0 + 2 * k;
+                            if (dst && k < np)
+                                *reinterpret_cast<uint32_t *>(dst + (p.gran == 16 ? (c >> 3) * (kBlockTokens * 16) + (c & 7) * 2
+                                                                                  : (c >> 1) * (kBlockTokens * 4))) = w[k];
+                        }
+                    } else {
+                        uint32_t *sw = reinterpret_cast<uint32_t *>(stg);  // 17 words a row
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) sw[lane * 17 + k] = w[k];
+                        __syncwarp();
+                        const uint32_t inv = 65536u / np + 1;  // i / np for i < 512
+                        for (int i = lane; i < 32 * np; i += 32) {
+                            const int rr = static_cast<int>(i * inv >> 16), c = i - rr * np;
+                            char *d = reinterpret_cast<char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), rr));
+                            if (d) *reinterpret_cast<uint32_t *>(d + (c0 + 2 * c) * 2) = sw[rr * 17 + c];
+                        }
+                        __syncwarp();
+                    }
+                    continue;
+                }
                 if (U.axis == 1) {
                     // V-plane rows are r_v * 2 bytes apart: stage the warp's 32 rows x 64 bytes and
                     // store 8 rows of 64 contiguous bytes per instruction
@@ -304,13 +471,14 @@ __global__ void __launch_bounds__(kEThreads, 1)
                         const int rr = 8 * i + (lane >> 2), cc = lane & 3;
                         char *d = reinterpret_cast<char *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), rr));
                         const uint4 val = *reinterpret_cast<const uint4 *>(stg + rr * 80 + cc * 16);
-                        if (d) *reinterpret_cast<uint4 *>(d + (U.col0 + c0 + cc * 8) * 2) = val;
+                        if (d && c0 + cc * 8 < U.cols) *reinterpret_cast<uint4 *>(d + (U.col0 + c0 + cc * 8) * 2) = val;
                     }
                     __syncwarp();
                 } else if (dst) {
 #pragma unroll
                     for (int k = 0; k < 32; k += 8) {
                         const int c = c0 + k, jc = U.col0 + c;  // column in the group, in the axis
+                        if (c >= U.cols) break;
                         float b8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                         if (use_bias) {
 #pragma unroll
@@ -321,8 +489,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
                                                    pack_bf16(v[k + 4] - b8[4], v[k + 5] - b8[5]),
                                                    pack_bf16(v[k + 6] - b8[6], v[k + 7] - b8[7]));
                         // K-plane: granule jc/8 of 16 bytes at (jc/8) * 64 * 16 + row * 16
-                        char *o = U.axis == 0 ? dst + (jc / 8) * (kBlockTokens * 16) : dst + jc * 2;
-                        *reinterpret_cast<uint4 *>(o) = w;
+                        *reinterpret_cast<uint4 *>(dst + (jc / 8) * (kBlockTokens * 16)) = w;
                     }
                 }
             }
@@ -333,6 +500,54 @@ __global__ void __launch_bounds__(kEThreads, 1)
         }
     }
     pdl_trigger();
+    if (split) {
+        // every CTA of the cluster has finished its products: the rings may take the parts
+        __syncthreads();
+        cluster_sync();
+        const Unit U = unit_of(p, u0);
+        const int own = ((U.cols + p.split - 1) / p.split + 7) & ~7;  // columns each rank stores
+        const bool ep = warp >= 2 && warp <= 5;
+        const int quarter = warp & 3, row = quarter * 32 + lane;
+        const float *bs = bias + U.g * kMaxGroup;
+        const bool use_bias = (U.axis ? p.mu_v : p.mu_k) != nullptr;
+        if (ep) {
+            mbar_wait(&accfull[0], 0, abort_flag, p.err);
+            tc_fence_after();
+            const uint32_t tl = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+#pragma unroll 1
+            for (int c0 = 0; c0 < U.cols; c0 += 8) {
+                float v[8];
+                tmem_ld8(tl + c0, v);
+                if (use_bias) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v[i] -= bs[c0 + i];
+                }
+                const uint32_t to = c0 / own;
+                const uint32_t at = smem_addr(sm) + ((crank * (own / 4) + (c0 - to * own) / 4) * kEM + row) * 16;
+                st_cluster_f4(at, to, make_float4(v[0], v[1], v[2], v[3]));
+                st_cluster_f4(at + kEM * 16, to, make_float4(v[4], v[5], v[6], v[7]));
+            }
+            tc_fence_before();
+        }
+        cluster_sync();
+        if (ep) {
+            char *dst = row_dst(p, U, row, U.g == 0 && crank == 0);
+            for (int c0 = crank * own; c0 < min(U.cols, (crank + 1) * own); c0 += 8) {
+                float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int q = 0; q < p.split; ++q) {
+                    const float4 *src = reinterpret_cast<const float4 *>(sm) + (q * (own / 4) + (c0 - crank * own) / 4) * kEM + row;
+                    const float4 a = src[0], b = src[kEM];
+                    v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+                    v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+                }
+                if (dst) {
+                    const int jc = U.col0 + c0;
+                    *reinterpret_cast<uint4 *>(U.axis == 0 ? dst + (jc / 8) * (kBlockTokens * 16) : dst + jc * 2) =
+                        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+                }
+            }
+        }
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -341,7 +556,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
     }
 }
 
-bool make_maps(const EncodeArgs &a, int axis, CUtensorMap *tx, CUtensorMap *tw) {
+bool make_maps(const EncodeArgs &a, int axis, bool wres, CUtensorMap *tx, CUtensorMap *tw) {
     const int Td = a.T * a.d;
     const int r = axis ? a.r_v : a.r_k;
     const void *x = axis ? a.x_v : a.x_k;
@@ -354,28 +569,68 @@ bool make_maps(const EncodeArgs &a, int axis, CUtensorMap *tx, CUtensorMap *tw) 
         const uint32_t box[4] = {kES, 1, kEM, 1};
         if (!encode_tmap_bf16(tx, x, 4, dims, strides, box, true)) return false;
     }
+    if (wres) {  // W_down goes through registers: the map is never used
+        *tw = *tx;
+        return true;
+    }
     const uint64_t dims[3] = {static_cast<uint64_t>(r), static_cast<uint64_t>(Td), static_cast<uint64_t>(a.H)};
     const uint64_t strides[2] = {static_cast<uint64_t>(r) * 2, static_cast<uint64_t>(Td) * r * 2};
     const uint32_t box[3] = {64, kES, 1};
     return encode_tmap_bf16(tw, w, 3, dims, strides, box, true);
 }
 
-// Column groups of an axis of rank r: n equal groups of at most 192 columns, each a multiple of
-// 32 (0 groups when r has no such split).
+// Column groups of an axis of rank r: ceil(r / 192) groups of `width` columns (a multiple of 16).
 int axis_groups(int r, int *width) {
     const int n = (r + kMaxGroup - 1) / kMaxGroup;
-    if (r % n != 0 || (r / n) % 32 != 0) return 0;
-    *width = r / n;
-    return n;
+    *width = ((r + n - 1) / n + 15) & ~15;
+    return (r + *width - 1) / *width;
+}
+
+// W_down rows of whole 16-byte words travel by tensor map; others (even ranks) only resident.
+bool wide_rows(const EncodeArgs &a) { return a.r_k % 8 == 0 && a.r_v % 8 == 0; }
+bool fits_resident(const EncodeArgs &a) { return a.r_k <= 64 && a.r_v <= 64 && a.T * a.d <= kResSlabs * kES; }
+
+template <bool WRES>
+lla_status launch_tc(const EncodeArgs &a, const ETParams &p, int grid, cudaStream_t stream) {
+    CUtensorMap txk, txv, twk, twv;
+    if (!make_maps(a, 0, WRES, &txk, &twk) || !make_maps(a, 1, WRES, &txv, &twv)) return LLA_ERR_CUDA;
+    static DeviceOnce configured;
+    if (raise_smem_limit(encode_tc_kernel<WRES>, EL<WRES>::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(kEThreads);
+    cfg.dynamicSmemBytes = EL<WRES>::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(p.split);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.split > 1 ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, encode_tc_kernel<WRES>, txk, txv, twk, twv, p) != cudaSuccess) return LLA_ERR_CUDA;
+    return LLA_OK;
 }
 
 }  // namespace
 
 bool encode_tc_supported(const EncodeArgs &a) {
     int w = 0;
-    return a.storage_bf16 && a.x_bf16 && !a.dense && a.d % kES == 0 && a.N >= kEM &&
-           (a.T * a.d) % kES == 0 && axis_groups(a.r_k, &w) && axis_groups(a.r_v, &w) &&
-           axis_groups(a.r_k, &w) + axis_groups(a.r_v, &w) <= kMaxGroups;
+    // From one tile of tokens on: 130 tokens at (72, 120) take 7.5 us here and 34 us on the CUDA
+    // cores, 100 tokens at (96, 160) 28 us there.  With a long reduction (LLA-2D) always: the CUDA-core
+    // kernel holds only 96 KB / (4 T*d) tokens per CTA and reads all of W_down again for each such
+    // tile (one token at 8192 rows: 59 us there, 16 us here; at 4096 rows 35 and 16 us).
+    return a.storage_bf16 && a.x_bf16 && !a.dense && a.d % kES == 0 && (a.N >= kEM || a.T * a.d >= kLongReduction) &&
+           (wide_rows(a) ? axis_groups(a.r_k, &w) + axis_groups(a.r_v, &w) <= kMaxGroups : fits_resident(a));
+}
+
+// Layer by layer on this kernel, or all layers in one launch of the CUDA-core kernel: with the
+// resident W_down a layer's launch costs about 9 us however few its tokens (128 tokens, 48 layers,
+// (18, 30): 440 us here, 400 us there, which grows with the tokens).
+bool encode_tc_layers(const EncodeArgs &a) {
+    return encode_tc_supported(a) && (wide_rows(a) || a.N >= kEM + kEM / 2);
 }
 
 lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream) {
@@ -395,26 +650,17 @@ lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream) {
     p.head_page_bytes = static_cast<int>(head_page_bytes(a.r_k, a.r_v, 2));
     p.block_bytes = static_cast<int64_t>(p.head_page_bytes) * a.H;
     p.kplane_bytes = LLA_BLOCK_TOKENS * a.r_k * 2;
+    p.gran = granule_bytes(a.r_k, 2);
     p.slot_mapping = a.slot_mapping;
     p.err = err;
-    CUtensorMap txk, txv, twk, twv;
-    if (!make_maps(a, 0, &txk, &twk) || !make_maps(a, 1, &txv, &twv)) return LLA_ERR_CUDA;
-    static DeviceOnce configured;
-    if (raise_smem_limit(encode_tc_kernel, kSmem, configured) != LLA_OK) return LLA_ERR_CUDA;
     const int sms = num_sms();
     if (sms <= 0) return LLA_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.units < sms ? p.units : sms));
-    cfg.blockDim = dim3(kEThreads);
-    cfg.dynamicSmemBytes = kSmem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, encode_tc_kernel, txk, txv, twk, twv, p) != cudaSuccess) return LLA_ERR_CUDA;
-    return LLA_OK;
+    // split the reduction while the clusters fit the SMs and each CTA keeps at least 8 slabs
+    p.split = 1;
+    const int slabs = a.T * a.d / kES;
+    while (wide_rows(a) && p.split < kMaxSplit && p.units * p.split * 2 <= sms && slabs / (p.split * 2) >= 8) p.split *= 2;
+    const int grid = static_cast<int>(p.split > 1 ? p.units * p.split : p.units < sms ? p.units : sms);
+    return wide_rows(a) ? launch_tc<false>(a, p, grid, stream) : launch_tc<true>(a, p, grid, stream);
 }
 
 }  // namespace lla

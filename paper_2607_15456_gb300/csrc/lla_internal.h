@@ -105,8 +105,10 @@ lla_status launch_encode(const EncodeArgs &a, cudaStream_t stream);
 // The same encode for L layers (one launch for decode batches).
 constexpr int kMaxEncodeLayers = 64;
 lla_status launch_encode_layers(const EncodeArgs *a, int L, cudaStream_t stream);
-// Tensor-core encode for prompts (bf16 x and storage, N >= 128, instantiated ranks).
+// Tensor-core encode (bf16 x and storage; prompts, and long reductions at any N); encode_tc_layers:
+// whether several layers go through it one by one.
 bool encode_tc_supported(const EncodeArgs &a);
+bool encode_tc_layers(const EncodeArgs &a);
 lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream);
 lla_status launch_prefill(const PrefillArgs &a, cudaStream_t stream);
 // Prefill with rotary positions after reconstruction: keys rebuilt and rotated into the

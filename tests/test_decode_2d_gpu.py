@@ -294,3 +294,36 @@ def test_large_latents_split_across_ctas(lla, lens):
     sc.append_token()
     _check(sc, 2, pass1=False)
     assert lla.lla_get_device_error() == 0
+
+
+@pytest.mark.parametrize("H,r_k,r_v,lens,with_mu", [
+    (16, 288, 480, (130, 3), True),    # two tiles, the reduction of 8192 rows split over clusters
+    (16, 288, 480, (1,), False),       # one token: clusters of eight
+    (16, 288, 480, (2000,), True),     # 16 tiles: two CTAs per unit
+    (16, 288, 480, (4100,), True),     # more units than SMs: no split, several groups' biases per CTA
+    (8, 1152, 1920, (70,), True),      # sixteen column groups
+    (8, 40, 200, (150,), True),        # groups of 48, 112 and 88 columns: padding columns
+])
+def test_encode_2d_on_tensor_cores(lla, H, r_k, r_v, lens, with_mu):
+    s = Scene2D(lla, H=H, r_k=r_k, r_v=r_v, io="bf16", lens=lens, seed=21, with_mu=with_mu) \
+        if r_k != 40 else None
+    if s is None:  # ranks without a decode kernel: encode only
+        from paper_2607_15456_gb300 import workloads as W
+        geom = lla.Geometry(4, H, 128, r_k, r_v)
+        cod = W.codec_tensors_2d(4, H, 128, r_k, r_v, 21, 0, device=DEV, with_mu=with_mu)
+        pt = W.page_table(list(lens), 21, extra_tokens=1)
+        pool = torch.full((pt.num_blocks * lla.lla_cache_2d_block_bytes(geom),), 0xFF, dtype=torch.uint8, device=DEV)
+        x = [W.normal((4, sum(lens), H, 128), 21, 40 + i, device=DEV) for i in range(2)]
+        lla.lla_encode_2d(geom, lla.Codec(**cod), lla.Cache(pool, pt.num_blocks, pt.block_table.to(DEV), pt.max_blocks),
+                          x[0], x[1], pt.slots(0, range(lens[0])).to(DEV))
+        got = unpack_head(pool.cpu(), 1, r_k, r_v, "bf16", pt.block_table[0], lens[0], 0)
+        want = [oracle.encode_2d(f64(x[i]), f64(cod["mu_" + a]), f64(cod["w_down_" + a])) for i, a in enumerate("kv")]
+        for g, w in zip(got, want):
+            assert_parity(g, w, "bf16", "2D latents")
+        return
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    for b in range(len(lens)):
+        gk, gv = s.gpu_latents(b)
+        assert_parity(gk, s.ck[b], "bf16", f"c_k {b}")
+        assert_parity(gv, s.cv[b], "bf16", f"c_v {b}")

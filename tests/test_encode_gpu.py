@@ -135,3 +135,18 @@ def test_encode_layers_equals_per_layer_calls(lla, N, storage):
     assert lla.lla_get_device_error() == 0
     for l in range(L):
         assert torch.equal(caches_a[l].pool, caches_b[l].pool), l
+
+
+@pytest.mark.parametrize("r_k,r_v,with_mu", [(72, 120, True), (72, 120, False), (8, 200, True), (104, 136, False),
+                                             (18, 30, True), (18, 30, False), (24, 62, True), (2, 64, True)])
+def test_encode_prompt_any_rank_on_tensor_cores(lla, r_k, r_v, with_mu):
+    # ranks that are not multiples of 32 (the last columns of a group are padding), an axis in two
+    # uneven groups (200 = 112 + 88), and rows of W_down that are not whole 16-byte words (resident
+    # W_down, 4-byte granules of the K-plane or 16-byte ones); 3 heads, a ragged third tile
+    _encode_and_compare(lla, 4, 3, 128, r_k, r_v, "bf16", "bf16", [128, 129, 13], with_mu, 11)
+
+
+@pytest.mark.parametrize("r_k,r_v", [(72, 120), (18, 30)])
+def test_encode_prompt_any_rank_many_units_per_cta(lla, r_k, r_v):
+    # 33 tiles of 8 heads with mu: several units per CTA and a head boundary inside a CTA's range
+    _encode_and_compare(lla, 4, 8, 128, r_k, r_v, "bf16", "bf16", [2000, 1500, 700], True, 12)

@@ -14,6 +14,10 @@
 // (x - mu) into shared memory as fp32.  At a decode step (N = batch) a launch therefore costs
 // about one memory round trip.  256 threads are 16 column pairs x 4 groups of 4 tokens x 4
 // slices of the reduction axis; the 4 partial sums per output meet in shared memory.
+//
+// bf16 x and storage go to the tensor cores instead: a decode step's tokens to lla_encode_step.cu,
+// prompts and LLA-2D to lla_encode_tc.cu.  This kernel takes fp32 x or storage and head widths that
+// are not multiples of 32.
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -328,8 +332,9 @@ lla_status set_smem() {
 lla_status launch_encode_layers(const EncodeArgs *a, int L, cudaStream_t stream) {
     if (L <= 0 || a[0].N == 0) return LLA_OK;
     const EncodeArgs &a0 = a[0];
-    // prompts take the tensor-core kernel layer by layer; decode batches share one launch
-    if (encode_tc_layers(a0) || a0.dense || L > kMaxEncodeLayers) {
+    // decode batches share one launch; prompts take the tensor-core kernel layer by layer
+    if (encode_step_supported(a0) && static_cast<int64_t>(a0.H) * L <= 65535) return launch_encode_step(a, L, stream);
+    if (encode_tc_supported(a0) || a0.dense || L > kMaxEncodeLayers) {
         for (int l = 0; l < L; ++l) {
             const lla_status st = launch_encode(a[l], stream);
             if (st != LLA_OK) return st;
@@ -382,6 +387,7 @@ lla_status launch_encode_layers(const EncodeArgs *a, int L, cudaStream_t stream)
 
 lla_status launch_encode(const EncodeArgs &a, cudaStream_t stream) {
     if (a.N == 0) return LLA_OK;
+    if (encode_step_supported(a)) return launch_encode_step(&a, 1, stream);
     if (encode_tc_supported(a)) return launch_encode_tc(a, stream);
     const int es = a.storage_bf16 ? 2 : 4;
     lla_status st = LLA_OK;

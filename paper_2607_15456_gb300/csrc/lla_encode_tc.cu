@@ -57,6 +57,7 @@ constexpr int kMaxGroup = 192;       // columns of a group
 constexpr int kMaxGroups = 20;       // groups of both axes (LLA-2D (1152, 1920): 6 + 10)
 constexpr int kMaxSplit = 8;         // CTAs that share one unit's reduction
 constexpr int kLongReduction = 4096; // reduction rows from which small batches take this kernel too
+constexpr int kLongestStack = 24576; // T*d of one fp32 token in 96 KB
 constexpr int kResSlabs = 8;         // WRES: most slabs (T*d = 512 rows) kept resident
 constexpr int kASlab = kEM * kES * 2;   // x slab (16 KB)
 constexpr int kBAtom = kES * 128;       // one W_down atom of 64 columns (8 KB)
@@ -586,6 +587,12 @@ int axis_groups(int r, int *width) {
     return (r + *width - 1) / *width;
 }
 
+// Equal groups of a multiple of 32 columns, at most 192 (7: r has no such split).
+int groups_of_32(int r) {
+    const int n = (r + kMaxGroup - 1) / kMaxGroup;
+    return r % n == 0 && (r / n) % 32 == 0 ? n : 7;
+}
+
 // W_down rows of whole 16-byte words travel by tensor map; others (even ranks) only resident.
 bool wide_rows(const EncodeArgs &a) { return a.r_k % 8 == 0 && a.r_v % 8 == 0; }
 bool fits_resident(const EncodeArgs &a) { return a.r_k <= 64 && a.r_v <= 64 && a.T * a.d <= kResSlabs * kES; }
@@ -618,19 +625,14 @@ lla_status launch_tc(const EncodeArgs &a, const ETParams &p, int grid, cudaStrea
 
 bool encode_tc_supported(const EncodeArgs &a) {
     int w = 0;
-    // From one tile of tokens on: 130 tokens at (72, 120) take 7.5 us here and 34 us on the CUDA
+    // stacks that no token tile of the CUDA-core kernel holds are taken where they always were
+    if (a.T * a.d > kLongestStack && !(a.N >= kEM && groups_of_32(a.r_k) + groups_of_32(a.r_v) <= 6)) return false;
+    // From half a tile of tokens on (what encode_step_kernel leaves): 130 tokens at (72, 120) take 7.5 us here and 34 us on the CUDA
     // cores, 100 tokens at (96, 160) 28 us there.  With a long reduction (LLA-2D) always: the CUDA-core
     // kernel holds only 96 KB / (4 T*d) tokens per CTA and reads all of W_down again for each such
     // tile (one token at 8192 rows: 59 us there, 16 us here; at 4096 rows 35 and 16 us).
-    return a.storage_bf16 && a.x_bf16 && !a.dense && a.d % kES == 0 && (a.N >= kEM || a.T * a.d >= kLongReduction) &&
+    return a.storage_bf16 && a.x_bf16 && !a.dense && a.d % kES == 0 && (a.N > kEM / 2 || a.T * a.d >= kLongReduction) &&
            (wide_rows(a) ? axis_groups(a.r_k, &w) + axis_groups(a.r_v, &w) <= kMaxGroups : fits_resident(a));
-}
-
-// Layer by layer on this kernel, or all layers in one launch of the CUDA-core kernel: with the
-// resident W_down a layer's launch costs about 9 us however few its tokens (128 tokens, 48 layers,
-// (18, 30): 440 us here, 400 us there, which grows with the tokens).
-bool encode_tc_layers(const EncodeArgs &a) {
-    return encode_tc_supported(a) && (wide_rows(a) || a.N >= kEM + kEM / 2);
 }
 
 lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream) {

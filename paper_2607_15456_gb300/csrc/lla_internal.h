@@ -105,11 +105,13 @@ lla_status launch_encode(const EncodeArgs &a, cudaStream_t stream);
 // The same encode for L layers (one launch for decode batches).
 constexpr int kMaxEncodeLayers = 64;
 lla_status launch_encode_layers(const EncodeArgs *a, int L, cudaStream_t stream);
-// Tensor-core encode (bf16 x and storage; prompts, and long reductions at any N); encode_tc_layers:
-// whether several layers go through it one by one.
+// Tensor-core encode (bf16 x and storage; prompts, and long reductions at any N).
 bool encode_tc_supported(const EncodeArgs &a);
-bool encode_tc_layers(const EncodeArgs &a);
 lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream);
+// Encode of a decode step's tokens straight from W_down to the tensor cores, L <= kMaxEncodeLayers layers
+// in one launch (bf16 x and storage).
+bool encode_step_supported(const EncodeArgs &a);
+lla_status launch_encode_step(const EncodeArgs *a, int L, cudaStream_t stream);
 lla_status launch_prefill(const PrefillArgs &a, cudaStream_t stream);
 // Prefill with rotary positions after reconstruction: keys rebuilt and rotated into the
 // workspace, then the tensor-core attention over them (bf16 storage, d = 128, the prefill ranks).

@@ -137,16 +137,31 @@ def test_encode_layers_equals_per_layer_calls(lla, N, storage):
         assert torch.equal(caches_a[l].pool, caches_b[l].pool), l
 
 
-@pytest.mark.parametrize("r_k,r_v,with_mu", [(72, 120, True), (72, 120, False), (8, 200, True), (104, 136, False),
+@pytest.mark.parametrize("r_k,r_v,with_mu", [(72, 120, True), (8, 200, True), (104, 136, False),
                                              (18, 30, True), (18, 30, False), (24, 62, True), (2, 64, True)])
 def test_encode_prompt_any_rank_on_tensor_cores(lla, r_k, r_v, with_mu):
     # ranks that are not multiples of 32 (the last columns of a group are padding), an axis in two
     # uneven groups (200 = 112 + 88), and rows of W_down that are not whole 16-byte words (resident
     # W_down, 4-byte granules of the K-plane or 16-byte ones); 3 heads, a ragged third tile
-    _encode_and_compare(lla, 4, 3, 128, r_k, r_v, "bf16", "bf16", [128, 129, 13], with_mu, 11)
+    _encode_and_compare(lla, 4, 3, 128, r_k, r_v, "bf16", "bf16", [128, 129, 33], with_mu, 11)
 
 
 @pytest.mark.parametrize("r_k,r_v", [(72, 120), (18, 30)])
 def test_encode_prompt_any_rank_many_units_per_cta(lla, r_k, r_v):
     # 33 tiles of 8 heads with mu: several units per CTA and a head boundary inside a CTA's range
     _encode_and_compare(lla, 4, 8, 128, r_k, r_v, "bf16", "bf16", [2000, 1500, 700], True, 12)
+
+
+@pytest.mark.parametrize("N", [1, 7, 16, 17, 33, 127, 256])
+@pytest.mark.parametrize("r_k,r_v,with_mu", [(96, 160, True), (72, 120, False), (8, 136, True), (128, 192, False),
+                                             (18, 30, True), (24, 70, False)])
+def test_encode_step_tokens_and_rank_edges(lla, N, r_k, r_v, with_mu):
+    # token tiles of 16 and 32 with every kind of remainder; column groups of 1 to 8 chunks of 8
+    # columns, or of up to 16 pairs when a row of W_down is not whole 16-byte words
+    _encode_and_compare(lla, 4, 2, 128, r_k, r_v, "bf16", "bf16", [N], with_mu, 13)
+
+
+@pytest.mark.parametrize("T,d", [(1, 32), (3, 96), (16, 128), (4, 64)])
+def test_encode_step_reduction_lengths(lla, T, d):
+    # fewer blocks of 32 rows than warps, blocks that do not divide by the warps, a long reduction
+    _encode_and_compare(lla, T, 2, d, 40, 72, "bf16", "bf16", [21], True, 14)

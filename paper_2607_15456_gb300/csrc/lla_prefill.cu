@@ -7,32 +7,46 @@
 //   s_ij = scale * q~_i . c_k,j,   p_i = softmax_j<=i(s_i)
 //   o_i  = W_up,t^V (sum_j p_ij c_v,j) + mu^V_t
 //
-// Tensor-core path (bf16 storage, d = 128, r_k and r_v multiples of 32): one CTA per
-// (128-query tile, sequence, head) and four warp roles.
-//   warp 0      K producer: W_up,t^K into shared memory (cp.async), then per page of 64 keys
-//               the K-plane (one bulk copy: its granule-interleaved layout is already the
-//               core-matrix layout of a K-major MMA operand), and W_up,t^V for the epilogue;
-//               the V-plane of each page comes as one TMA tensor load with 128-byte swizzle per
-//               64 latent columns (an MN-major operand)
-//   warp 2      V producer (one thread), decoupled from the K-planes so that neither ring
-//               waits on the other
-//   warp 1      Q~ and S issuer (one thread) and TMEM owner:
+// Tensor-core path (bf16 storage, d = 128, the ranks of launch_prefill): one CTA per (one or two
+// 128-query tiles, sequence, head), four warps that move data and issue products, and two softmax
+// groups of four warps with a thread per query row:
+//   warp 0      K producer: W_up,t^K by TMA, then per page of 64 keys the K-plane (one bulk copy: its
+//               granule-interleaved layout is already the core-matrix layout of a K-major MMA operand),
+//               and W_up,t^V for the epilogue (TMA; into room of its own or, at (192, 320), over q~ and
+//               the K ring once the last score product has read them)
+//   warp 2      V producer, decoupled from the K-planes so that neither ring waits on the other: one TMA
+//               load with 128-byte swizzle per 64 latent columns of a page (an MN-major operand)
+//   warp 1      Q~ and S issuer and TMEM owner:
 //                 Q~ = Q W_up,t^K             M=128, N=r_k, K=d
-//                 S_j = Q~ C_k,j^T            M=128, N=64,  K=r_k   (double-buffered in TMEM)
-//   warp 3      PV and output issuer (one thread), so that neither MMA stream waits behind the
-//               other's barriers:
-//                 O += P_j C_v,j              M=128, N=r_v (split at 256), K=64
-//                 out = (O/l) W_up,t^V^T      M=128, N=d,   K=r_v
-//   warps 4-11  two threads per query row, each with 32 keys of every page (warps w and w + 4
-//               share TMEM lanes): Q and Q~ into bf16 operands, causal mask on diagonal pages,
-//               online softmax in the exp2 domain with the row maximum exchanged through shared
-//               memory, P into a bf16 operand, O rescaled in TMEM only when a row maximum grows
-//               by more than 2^8, V rows past the prompt zeroed on its last page, then the
-//               epilogue.
-// Accumulators are fp32 in TMEM; operands are bf16 (q~ carries scale * log2 e).
+//                 S_j = Q~ C_k,j^T            M=128, N=64,  K=r_k
+//   warp 3      PV and output issuer, so that neither MMA stream waits behind the other's barriers:
+//                 O += P_j C_v,j              M=128, N=r_v (split at 256), K=64, P_j in TMEM
+//                 out = (O/l) W_up,t^V^T      M=128, N=2 x 64, K=r_v, O/l as hi + lo in TMEM
+//               The issuing warps run converged, one elected thread per product, on uniform values
+//               (page counts broadcast from one lane, TMEM address 0): issued from a one-thread branch a
+//               product cost that thread about 80 cycles, more than the product itself
+//   warps 4-11  the softmax groups: Q and Q~ into bf16 operands, causal mask on diagonal pages, online
+//               softmax in the exp2 domain, P to TMEM as packed bf16 (no shared memory, no proxy fence),
+//               O rescaled in TMEM only when a row maximum grows by more than 2^8, V rows past the
+//               prompt zeroed on its last page, then the epilogue.
+// With two tiles per CTA each group owns one.  With one tile the groups take its pages in turn, so that
+// one's softmax (about 1000 cycles from scores to weights) runs beside the other's: the running maximum
+// goes from page to page through shared memory and a named barrier per warp pair, each group keeps its
+// own row sums, and they meet after the last page.
+// Accumulators are fp32 in TMEM; operands are bf16 (q~ carries scale * log2 e).  At (72, 120) q~ and P
+// are sums of two bf16 parts (16 significant bits; twice the products): that shape was served in fp32
+// by the CUDA cores, and its bf16 outputs stay as exact as their rounding.
 //
-// CUDA-core path (fp32 storage, other ranks, d != 128): one CTA per (query, sequence, head),
-// fp32 throughout.
+// Bound by the tensor pipe and the shared memory that feeds it: a (192, 320) page takes 640 cycles of PV
+// products and 576 of score products (a 128 x 64 x 16 product reads 6 KB, 48 cycles of shared memory for
+// 32 of arithmetic).  Measured, 16 heads: 4 x 8192 tokens at (192, 320) 1920 -> 1640 us (1385 TFLOP/s; the
+// clock falls under the power limit), at (96, 160) 1445 -> 944 us, at (128, 128) 1445 -> 1016 us; a tile of
+// 2 pages from launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the
+// last page, and the hi and lo projections followed each other through shared memory); (72, 120), 300
+// tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8341 us before.
+//
+// CUDA-core path (fp32 storage, other ranks, d != 128, fp32 inputs at (72, 120)): one CTA per (query,
+// sequence, head), fp32 throughout.
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -45,25 +59,23 @@ namespace {
 
 constexpr int kBM = 128;         // queries per tile
 constexpr int kPT = 64;          // keys per page
-constexpr int kSWarps = 8;       // softmax warps: two threads per query row
-constexpr int kSWarp0 = 4;       // K producer, S issuer, V producer, PV issuer, then softmax
-constexpr int kPThreads = (kSWarp0 + kSWarps) * 32;
-constexpr int kSThreads = kSWarps * 32;
+constexpr int kGroup = 128;      // threads of a softmax group: one per query row of a tile
+constexpr int kSWarp0 = 4;       // K producer, S issuer, V producer, PV issuer, then the two groups
+constexpr int kPThreads = kSWarp0 * 32 + 2 * kGroup;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleLog2 = 8.f;  // rescale O only when a row maximum grows by more
 
 struct PParams {
     int T, H, loop, io_bf16;
     float scale_log2;
-    const void *w_up_k, *w_up_v;
     const float *mu_v;
     const char *pool;
-    int64_t num_blocks, block_bytes;
+    int64_t num_blocks;
     int head_page_bytes;
     const int32_t *block_table;
     int max_blocks;
     const int32_t *cu_seqlens;
-    int B, max_len;
+    int max_len;
     const void *q;
     void *out;
     unsigned *err;
@@ -75,78 +87,98 @@ struct PParams {
     int64_t qrows;  // rows of the rotated-query buffer (B * max_len)
 };
 
-// Shared-memory plan of the tensor-core kernel for ranks (RK, RV); d = 128.  Offsets are
-// multiples of 1024 bytes from a 1024-byte aligned base (128-byte swizzle atoms).  With ROPE
-// the scores are formed from rebuilt, rotated keys of width d instead of latents of width RK.
-template <int RK, int RV, bool ROPE = false>
+// Shared-memory and TMEM plan of the tensor-core kernel for ranks (RK, RV), d = 128, NT query tiles
+// per CTA and QP bf16 parts of q~ and of the softmax weights.  Offsets are multiples of 1024 bytes
+// from a 1024-byte aligned base (128-byte swizzle atoms).  With ROPE the scores are formed from
+// rebuilt, rotated keys of width d instead of latents of width RK.
+template <int RK, int RV, int NT, bool ROPE, int QP>
 struct PF {
     static constexpr int D = 128;
-    static constexpr int RS = ROPE ? D : RK;         // contraction width of the scores
-    static constexpr int NKC = RK / 8;               // 16-byte chunks of a K row
-    static constexpr int NVC = RV / 8;               // 16-byte chunks of a V row
-    static constexpr int VATOMS = (RV + 63) / 64;    // 64-column atoms of a V page (TMA boxes)
-    static constexpr int N0 = RV > 256 ? 256 : RV;   // PV MMA split on atom boundaries
-    static constexpr int N1 = RV - N0;
+    static constexpr int RKX = (RK + 15) / 16 * 16;  // padded with zero columns of q~ and a zero granule
+    static constexpr int RS = ROPE ? D : RKX;        // contraction width of the scores
+    static constexpr int ORV = (RV + 15) / 16 * 16;  // O columns of a tile
+    static constexpr int VATOMS = (RV + 63) / 64;    // 64-column boxes of a V page, of W_up,t^V
+    static constexpr int KATOMS = (RK + 63) / 64;    // 64-column boxes of W_up,t^K
+    static constexpr int N0 = ORV > 256 ? 256 : ORV; // PV MMA split on atom boundaries
+    static constexpr int N1 = ORV - N0;
     static constexpr int KPAGE = kPT * RS * 2;
+    static constexpr int KCOPY = ROPE ? KPAGE : kPT * RK * 2;
     static constexpr int VPAGE = VATOMS * kPT * 128;
-    static constexpr int QT = kBM * RS * 2;          // q~ (or rotated q) operand
-    static constexpr int PB = kBM * kPT * 2;         // P operand (one of two)
-    static constexpr int QA = kBM * D * 2;           // q operand (prologue)
-    static constexpr int WK = D * RK * 2;            // W_up,t^K operand (prologue)
-    static constexpr int WV = D * RV * 2;            // W_up,t^V operand (epilogue)
-    static constexpr int OA = kBM * RV * 2;          // O / l operand (epilogue)
-    // K and V pipeline stages: as deep as shared memory allows (up to 4), V at least 2 deep
-    static constexpr int BUDGET = 220 * 1024 - QT - 2 * PB;
-    static constexpr int STV = (BUDGET - 2 * KPAGE) / VPAGE >= 4 ? 4 : (BUDGET - 2 * KPAGE) / VPAGE >= 3 ? 3 : 2;
-    static constexpr int STK0 = (BUDGET - STV * VPAGE) / KPAGE;
+    static constexpr int QT1 = kBM * RS * 2;         // q~ (or rotated q) operand: one part of one tile
+    static constexpr int QT = NT * QP * QT1;
+    static constexpr int QA1 = kBM * D * 2;          // q operand of one tile (prologue)
+    static constexpr int WK = KATOMS * D * 128;      // W_up,t^K operand (prologue)
+    static constexpr int WV = VATOMS * D * 128;      // W_up,t^V operand (epilogue)
+    static constexpr int BUDGET = 222 * 1024;
+    // W_up,t^V has room of its own, or takes q~'s and the K ring's once every score product is done
+    static constexpr bool WVOWN = QT + 2 * KPAGE + 3 * VPAGE + WV <= BUDGET;
+    static constexpr int LEFT = BUDGET - QT - (WVOWN ? WV : 0);
+    static constexpr int STV0 = (LEFT - 2 * KPAGE) / VPAGE;
+    static constexpr int STV = STV0 > 4 ? 4 : STV0;
+    static constexpr int STK0 = (LEFT - STV * VPAGE) / KPAGE;
     static constexpr int STK = STK0 > 4 ? 4 : STK0;
     static constexpr int oQT = 0;
     static constexpr int oK = oQT + QT;
     static constexpr int oV = oK + STK * KPAGE;
-    static constexpr int oP = oV + STV * VPAGE;
-    static constexpr int oEnd = oP + 2 * PB;
-    // the prologue operands alias the V ring and P; the epilogue operands alias K, V and P
-    static constexpr int oQA = oV, oWK = oV + QA;
-    static constexpr int oOA = oK, oWV = oK + OA;
-    static constexpr int oX = oEnd;                   // [2 pages][2 halves][128 rows] maxima
-    static constexpr int oL = oX + 2 * 2 * kBM * 4;   // [2 halves][128 rows] row sums
-    static constexpr int oBar = oL + 2 * kBM * 4;
-    static constexpr int NBAR = 40;
-    static constexpr int SMEM = 1024 + oBar + NBAR * 8 + 16;
-    // TMEM columns: S double buffer [0, 128), O [128, 128 + RV); q~ and out reuse [0, ...)
-    static constexpr uint32_t TM_S = 0, TM_O = 128, TM_COLS = 512;
-    static_assert(RK % 32 == 0 && RV % 32 == 0 && RK <= 256 && 128 + RV <= 512, "ranks");
-    static_assert(N0 % 16 == 0 && N1 % 16 == 0 && N1 <= 256, "PV split");
+    static constexpr int oW = oV + STV * VPAGE;
+    static constexpr int oEnd = oW + (WVOWN ? WV : 0);
+    static constexpr int oQA = oV;                        // the prologue's q operands alias the V ring
+    static constexpr int oWK = WVOWN ? oW : oV + NT * QA1;
+    static constexpr int oWV = WVOWN ? oW : oQT;
+    static constexpr int oM = oEnd;                       // NT = 1: [128] running maxima
+    static constexpr int oX = oM + kBM * 4;               // NT = 1: [2 groups][128] (maximum, sum)
+    static constexpr int oBar = oX + 2 * kBM * 8;
+    static constexpr int NBAR = 48;
+    static constexpr int SMEM = 1024 + oBar + NBAR * 8;
+    // TMEM columns: S of each group, P of each group (packed pairs), O of each tile; q~ starts in O
+    static constexpr uint32_t TM_S = 0, TM_P = 2 * kPT, TM_O = TM_P + 2 * QP * (kPT / 2), TM_COLS = 512;
+    static_assert(RK % 8 == 0 && RV % 8 == 0 && RKX <= 256 && RKX <= ORV, "ranks");
+    static_assert(TM_O + NT * ORV <= TM_COLS && N1 <= 256 && N1 % 16 == 0, "TMEM columns");
     static_assert(STK >= 2 && STV >= 2, "pipeline depth");
-    static_assert(oK % 1024 == 0 && oV % 1024 == 0 && oP % 1024 == 0 && VPAGE % 1024 == 0, "align");
-    static_assert(oWK + WK <= oEnd && oWV + WV <= oEnd, "aliased operands fit");
+    static_assert(KPAGE % 1024 == 0 && QT1 % 1024 == 0, "align");
+    static_assert(NT * QA1 <= STV * VPAGE && (WVOWN ? WK <= WV : NT * QA1 + WK <= STV * VPAGE), "prologue operands fit");
+    static_assert(WVOWN || WV <= QT + STK * KPAGE, "epilogue operand fits");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// barrier indices
+// barrier indices ([2]: by softmax group, which is the tile for NT = 2)
 enum {
-    kBSetup = 0, kBQt, kBQs, kBOa, kBWv, kBOut, kBUnused, kBOfin,
-    kBSfull = 8 /* [2] */, kBSfree = 10, kBPfull = 12, kBPfree = 14,
-    kBOa2 = 16, kBOut1 = 17,
-    kBKfull = 18 /* [4] */, kBKempty = 22, kBVfull = 26, kBVempty = 30,
-    kBAbort = 34  // slot used as the CTA's abort flag
+    kBWk = 0, kBWv, kBSfin, kBOfin /* [2] */, kBQa = 5 /* [2] */, kBQt = 7 /* [2] */, kBQs = 9 /* [2] */,
+    kBOa = 11 /* [2] */, kBOut = 13 /* [2] */, kBOfree = 15 /* [2] */,
+    kBSfull = 17 /* [2] */, kBSfree = 19, kBPfull = 21, kBPfree = 23,
+    kBKfull = 25 /* [4] */, kBKempty = 29, kBVfull = 33, kBVempty = 37,
+    kBAbort = 41,  // slot used as the CTA's abort flag
+    kBTmem = 42    // and as the TMEM address
 };
 
-template <int RK, int RV, bool ROPE>
+// Two consecutive TMEM loads of 32 columns each, waited for once.
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
+    uint32_t a[32], b[32];
+    tmem_ld32_nowait(taddr, a);
+    tmem_ld32_nowait(taddr + 32, b);
+    tmem_wait_ld(a);
+    tmem_wait_ld(b);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        v[i] = __uint_as_float(a[i]);
+        v[32 + i] = __uint_as_float(b[i]);
+    }
+}
+
+template <int RK, int RV, int NT, bool ROPE, int QP>
 __global__ void __launch_bounds__(kPThreads, 1)
-    prefill_tc_kernel(const __grid_constant__ CUtensorMap tv, const PParams p) {
-    using F = PF<RK, RV, ROPE>;
+    prefill_tc_kernel(const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap twk,
+                      const __grid_constant__ CUtensorMap twv, const __grid_constant__ PParams p) {
+    using F = PF<RK, RV, NT, ROPE, QP>;
     constexpr int D = F::D;
     extern __shared__ __align__(1024) char sm_raw[];
     char *sm = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + F::oBar);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar + kBAbort);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + F::NBAR);
-    float *xmax = reinterpret_cast<float *>(sm + F::oX);
-    float *xsum = reinterpret_cast<float *>(sm + F::oL);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + kBTmem);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
-    const int nqt = (p.max_len + kBM - 1) / kBM;
+    const int nqt = (p.max_len + NT * kBM - 1) / (NT * kBM);
     const int qt = nqt - 1 - static_cast<int>(blockIdx.x);  // longest causal ranges first
     const int b = blockIdx.y, h = blockIdx.z;
     pdl_wait();
@@ -156,23 +188,31 @@ __global__ void __launch_bounds__(kPThreads, 1)
         if (tid == 0 && qt == nqt - 1) atomicOr(p.err, LLA_DEVERR_CONTEXT);
         return;
     }
-    const int i0 = qt * kBM;
+    const int i0 = qt * NT * kBM;
     if (i0 >= L) return;  // uniform over the CTA, before any barrier or TMEM use
-    const int iend = min(L, i0 + kBM);
-    const int NP = (iend - 1) / kPT + 1;  // pages 0..NP-1 hold every key of the tile
-    const int64_t wofs = (static_cast<int64_t>(h) * p.T + p.loop) * D;
+    // pages 0 .. np(g) - 1 hold every key of tile g (none past the prompt); NP: of the CTA
+    auto np = [&](int g) { return i0 + g * kBM < L ? (min(L, i0 + (g + 1) * kBM) - 1) / kPT + 1 : 0; };
+    const int NP = max(np(0), NT == 2 ? np(1) : 0);
+    const int wrow = (h * p.T + p.loop) * D;  // first row of W_up,t of this head
     const int32_t *bt = p.block_table + static_cast<int64_t>(b) * p.max_blocks;
 
     if (tid == 0) {
-        mbar_init(&bar[kBSetup], 32 + kSThreads);
-        mbar_init(&bar[kBQt], 1);
-        mbar_init(&bar[kBQs], kSThreads);
-        mbar_init(&bar[kBOa], kSThreads);
-        mbar_init(&bar[kBOa2], kSThreads);
-        mbar_init(&bar[kBWv], 32);
-        mbar_init(&bar[kBOut1], 1);
-        mbar_init(&bar[kBOut], 1);
-        mbar_init(&bar[kBOfin], 1);
+        mbar_init(&bar[kBWk], 1);
+        mbar_init(&bar[kBWv], 1);
+        mbar_init(&bar[kBSfin], 1);
+        for (int g = 0; g < 2; ++g) {
+            mbar_init(&bar[kBOfin + g], 1);
+            mbar_init(&bar[kBQa + g], kGroup);
+            mbar_init(&bar[kBQt + g], 1);
+            mbar_init(&bar[kBQs + g], NT == 1 ? 2 * kGroup : kGroup);
+            mbar_init(&bar[kBOa + g], NT == 1 ? 2 * kGroup : kGroup);
+            mbar_init(&bar[kBOut + g], 1);
+            mbar_init(&bar[kBOfree + g], kGroup);
+            mbar_init(&bar[kBSfull + g], 1);
+            mbar_init(&bar[kBSfree + g], kGroup);
+            mbar_init(&bar[kBPfull + g], kGroup);
+            mbar_init(&bar[kBPfree + g], 1);
+        }
         for (int s = 0; s < F::STK; ++s) {
             mbar_init(&bar[kBKfull + s], 1);
             mbar_init(&bar[kBKempty + s], 1);
@@ -181,38 +221,44 @@ __global__ void __launch_bounds__(kPThreads, 1)
             mbar_init(&bar[kBVfull + s], 1);
             mbar_init(&bar[kBVempty + s], 1);
         }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&bar[kBSfull + s], 1);
-            mbar_init(&bar[kBSfree + s], kSThreads);
-            mbar_init(&bar[kBPfull + s], kSThreads);
-            mbar_init(&bar[kBPfree + s], 1);
-        }
         *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tslot, F::TM_COLS);
+    if constexpr (F::KPAGE > F::KCOPY) {  // the K granules past r_k, against zero columns of q~
+        for (int s = 0; s < F::STK; ++s)
+            for (int i = tid; i < (F::KPAGE - F::KCOPY) / 16; i += kPThreads)
+                reinterpret_cast<uint4 *>(sm + F::oK + s * F::KPAGE + F::KCOPY)[i] = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    // the whole of TMEM is allocated, so its address is 0: a constant, and the page counts broadcast
+    // from one lane, keep the issuing warps' code uniform
+    constexpr uint32_t tmem = 0;
+    const int np0 = __shfl_sync(0xffffffffu, np(0), 0), np1 = __shfl_sync(0xffffffffu, NT == 2 ? np(1) : 0, 0);
+    auto npu = [&](int g) { return g ? np1 : np0; };
+    const int NPU = max(np0, np1);
 
     if (warp == 0) {
-        // ------------------------------------------------------------------------- producer
-        if constexpr (!ROPE) {
-            const char *wk = static_cast<const char *>(p.w_up_k) + wofs * RK * 2;
-            // W_up,t^K [d][r_k] as an MN-major operand: (row e, column chunk g) at g*(d*16) + e*16
-            for (int i = lane; i < D * F::NKC; i += 32) {
-                const int e = i / F::NKC, g = i - e * F::NKC;
-                cp_async16(sm + F::oWK + g * (D * 16) + e * 16, wk + (static_cast<int64_t>(e) * RK + g * 8) * 2);
+        // ----------------------------------------------- producer: W_up,t^K, K-planes, W_up,t^V
+        if (lane == 0) {
+            if constexpr (!ROPE) {  // rows e of W_up,t^K as the MN-major operand of Q~
+                mbar_arrive_expect_tx(&bar[kBWk], F::WK);
+#pragma unroll
+                for (int a = 0; a < F::KATOMS; ++a)
+                    tma_load_2d(sm + F::oWK + a * (D * 128), &twk, a * 64, wrow, &bar[kBWk]);
             }
-            cp_async_commit();
-            cp_async_wait_all();
-            fence_proxy_async_smem();
-        }
-        mbar_arrive(&bar[kBSetup]);
-        if (lane == 0) {  // K-planes: one bulk copy per page
             const uint64_t pol = policy_evict_first();
             int nk = 0;  // copies issued
+            auto load_wv = [&] {
+                mbar_arrive_expect_tx(&bar[kBWv], F::WV);
+#pragma unroll
+                for (int a = 0; a < F::VATOMS; ++a)
+                    tma_load_2d(sm + F::oWV + a * (D * 128), &twv, a * 64, wrow, &bar[kBWv]);
+            };
+            bool wv = false;
             for (int j = 0; j < NP; ++j) {
                 const int s = j % F::STK;
                 const uint32_t ph = (j / F::STK) & 1;
@@ -226,36 +272,46 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 const char *src = ROPE ? p.krot + ((static_cast<int64_t>(b) * p.kpps + j) * p.H + h) * F::KPAGE
                                        : p.pool + hp * p.head_page_bytes;
                 if (!mbar_wait(&bar[kBKempty + s], ph ^ 1u, abort_flag, p.err) || *abort_flag) break;
-                mbar_arrive_expect_tx(&bar[kBKfull + s], F::KPAGE);
-                bulk_g2s(sm + F::oK + s * F::KPAGE, src, F::KPAGE, &bar[kBKfull + s], pol);
+                mbar_arrive_expect_tx(&bar[kBKfull + s], F::KCOPY);
+                bulk_g2s(sm + F::oK + s * F::KPAGE, src, F::KCOPY, &bar[kBKfull + s], pol);
                 ++nk;
+                // W_up,t^V's own room held W_up,t^K until every q~ was formed
+                if (F::WVOWN && !wv && j == min(F::STK, NP) - 1) {
+                    bool ok = true;
+                    if constexpr (!ROPE) {
+                        for (int g = 0; g < NT; ++g)
+                            if (np(g) > 0) ok = mbar_wait(&bar[kBQt + g], 0, abort_flag, p.err) && ok;
+                    }
+                    if (ok) {
+                        load_wv();
+                        wv = true;
+                    }
+                }
             }
             // every copy has landed before the ring is reused or the CTA exits, even after an
             // abort (no copy is issued once a wait has failed)
             volatile int never = 0;
             for (int j = max(0, nk - F::STK); j < nk; ++j)
                 mbar_wait(&bar[kBKfull + j % F::STK], (j / F::STK) & 1, &never, p.err);
+            if constexpr (!ROPE) mbar_wait(&bar[kBWk], 0, &never, p.err);
+            if (!F::WVOWN && mbar_wait(&bar[kBSfin], 0, abort_flag, p.err) && !*abort_flag) {
+                load_wv();  // over q~ and the K ring, which every score product has read
+                wv = true;
+            }
+            if (wv) mbar_wait(&bar[kBWv], 0, &never, p.err);
         }
         __syncwarp();
-        // epilogue operand W_up,t^V [d][r_v] (K-major): (row e, chunk c) at c*(d*16) + e*16,
-        // into the K ring once every MMA of the loop has completed
-        mbar_wait(&bar[kBOfin], 0, abort_flag, p.err);
-        const char *wv = static_cast<const char *>(p.w_up_v) + wofs * RV * 2;
-        for (int i = lane; i < D * F::NVC; i += 32) {
-            const int e = i / F::NVC, c = i - e * F::NVC;
-            cp_async16(sm + F::oWV + c * (D * 16) + e * 16, wv + (static_cast<int64_t>(e) * RV + c * 8) * 2);
-        }
-        cp_async_commit();
-        cp_async_wait_all();
-        fence_proxy_async_smem();
-        mbar_arrive(&bar[kBWv]);
     } else if (warp == 2) {
         // ---------------------------------------------------------------------- V producer
         if (lane == 0) {  // V-planes: one TMA tensor load with 128-byte swizzle per 64 columns
-            // the V ring aliases the prologue operands: wait until Q~ has been computed
-            mbar_wait(&bar[kBQt], 0, abort_flag, p.err);
+            // the V ring aliases the prologue operands: wait until q~ has been computed
+            bool ok = true;
+            if constexpr (!ROPE) {
+                for (int g = 0; g < NT; ++g)
+                    if (np(g) > 0) ok = mbar_wait(&bar[kBQt + g], 0, abort_flag, p.err) && ok;
+            }
             int nv = 0;  // copies issued
-            for (int j = 0; j < NP; ++j) {
+            for (int j = 0; j < NP && ok; ++j) {
                 const int s = j % F::STV;
                 const uint32_t ph = (j / F::STV) & 1;
                 int32_t blk = bt[j];
@@ -276,203 +332,278 @@ __global__ void __launch_bounds__(kPThreads, 1)
         __syncwarp();
     } else if (warp == 1) {
         // -------------------------------------------------------------- Q~ and S MMA issuer
-        if (lane == 0) {
+        {
             const uint32_t base = smem_addr(sm);
-            mbar_wait(&bar[kBSetup], 0, abort_flag, p.err);
-            tc_fence_after();
-            if constexpr (ROPE) {
-                mbar_arrive(&bar[kBQt]);  // the rotated queries come ready from global memory
-            } else {
-                constexpr uint32_t idq = umma_idesc_bf16(128, RK, 0, 1);
-                const uint64_t dqa = umma_desc(base + F::oQA, 2048, 128);
-                const uint64_t dwk = umma_desc(base + F::oWK, 128, 2048);
+            if constexpr (!ROPE) {
+                mbar_wait_warp(&bar[kBWk], 0, abort_flag, p.err);
+                constexpr uint32_t idq = umma_idesc_bf16(128, F::RKX, 0, 1);
+                const uint64_t dwk = umma_desc_sw128_mn(base + F::oWK, D * 128);
+                for (int g = 0; g < NT; ++g) {
+                    if (npu(g) == 0) continue;
+                    mbar_wait_warp(&bar[kBQa + g], 0, abort_flag, p.err);
+                    tc_fence_after();
+                    const uint64_t dqa = umma_desc(base + F::oQA + g * F::QA1, 2048, 128);
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks)
-                    umma_bf16(tmem + 0, dqa + ks * (4096 >> 4), dwk + ks * (256 >> 4), idq, ks > 0);
-                umma_commit(&bar[kBQt]);
+                    for (int ks = 0; ks < D / 16; ++ks)
+                        umma_bf16_warp(tmem + F::TM_O + g * F::ORV, dqa + ks * (4096 >> 4), dwk + ks * (2048 >> 4), idq, ks > 0);
+                    umma_commit_warp(&bar[kBQt + g]);
+                }
             }
-            mbar_wait(&bar[kBQs], 0, abort_flag, p.err);
-            tc_fence_after();
             constexpr uint32_t ids = umma_idesc_bf16(128, kPT, 0, 0);
             // descriptors are built once; a byte offset moves the start-address field by offset/16
-            const uint64_t dq = umma_desc(base + F::oQT, 2048, 128);
+            const uint64_t dq0 = umma_desc(base + F::oQT, 2048, 128);
             const uint64_t dk0 = umma_desc(base + F::oK, 1024, 128);
 #pragma unroll 1
-            for (int j = 0; j < NP; ++j) {
-                const int s = j & 1, sk = j % F::STK;
-                mbar_wait(&bar[kBKfull + sk], (j / F::STK) & 1, abort_flag, p.err);
-                if (j >= 2) mbar_wait(&bar[kBSfree + s], ((j - 2) >> 1) & 1, abort_flag, p.err);
-                tc_fence_after();
+            for (int j = 0; j < NPU; ++j) {
+                const int sk = j % F::STK;
+                mbar_wait_warp(&bar[kBKfull + sk], (j / F::STK) & 1, abort_flag, p.err);
                 const uint64_t dk = dk0 + static_cast<uint64_t>(sk * (F::KPAGE >> 4));
-                const uint32_t ds = tmem + F::TM_S + s * kPT;
 #pragma unroll
-                for (int ks = 0; ks < F::RS / 16; ++ks)
-                    umma_bf16(ds, dq + ks * (4096 >> 4), dk + ks * (2048 >> 4), ids, ks > 0);
-                umma_commit(&bar[kBSfull + s]);
-                umma_commit(&bar[kBKempty + sk]);
+                for (int i = 0; i < NT; ++i) {
+                    // NT = 2: tile i's softmax group takes page j; NT = 1: the groups take turns
+                    const int g = NT == 2 ? i : (j & 1), jj = NT == 2 ? j : (j >> 1);
+                    if (NT == 2 && j >= npu(i)) continue;
+                    if (j == 0) mbar_wait_warp(&bar[kBQs + (NT == 2 ? g : 0)], 0, abort_flag, p.err);
+                    if (jj > 0) mbar_wait_warp(&bar[kBSfree + g], (jj - 1) & 1, abort_flag, p.err);
+                    tc_fence_after();
+                    const uint32_t ds = tmem + F::TM_S + g * kPT;
+#pragma unroll
+                    for (int part = 0; part < QP; ++part) {
+                        const uint64_t dq = dq0 + static_cast<uint64_t>((i * QP + part) * (F::QT1 >> 4));
+#pragma unroll
+                        for (int ks = 0; ks < F::RS / 16; ++ks)
+                            umma_bf16_warp(ds, dq + ks * (4096 >> 4), dk + ks * (2048 >> 4), ids, part > 0 || ks > 0);
+                    }
+                    umma_commit_warp(&bar[kBSfull + g]);
+                }
+                umma_commit_warp(&bar[kBKempty + sk]);
             }
+            umma_commit_warp(&bar[kBSfin]);
             // every product of this thread has completed before TMEM is released, even after an
-            // abort (when the softmax warps stop waiting for them): a commit tracks all earlier
-            // products of its thread, so the last one suffices
+            // abort (when the softmax warps stop waiting for them)
             volatile int never = 0;
-            if (NP > 0)
-                mbar_wait(&bar[kBSfull + ((NP - 1) & 1)], ((NP - 1) >> 1) & 1, &never, p.err);
-            else if constexpr (!ROPE)
-                mbar_wait(&bar[kBQt], 0, &never, p.err);
+            mbar_wait_warp(&bar[kBSfin], 0, &never, p.err);
         }
         __syncwarp();
     } else if (warp == 3) {
         // ----------------------------------------------------------- PV and output MMA issuer
-        if (lane == 0) {
+        {
             const uint32_t base = smem_addr(sm);
             constexpr uint32_t idv0 = umma_idesc_bf16(128, F::N0, 0, 1);
             constexpr uint32_t idv1 = umma_idesc_bf16(128, F::N1 > 0 ? F::N1 : 16, 0, 1);
-            const uint64_t dp0 = umma_desc(base + F::oP, 2048, 128);
             const uint64_t dv0 = umma_desc_sw128_mn(base + F::oV, kPT * 128);
 #pragma unroll 1
-            for (int jj = 0; jj < NP; ++jj) {
-                const int s = jj & 1, sv = jj % F::STV;
-                mbar_wait(&bar[kBPfull + s], (jj >> 1) & 1, abort_flag, p.err);
-                mbar_wait(&bar[kBVfull + sv], (jj / F::STV) & 1, abort_flag, p.err);
-                tc_fence_after();
-                const uint64_t dp = dp0 + static_cast<uint64_t>(s * (F::PB >> 4));
+            for (int j = 0; j < NPU; ++j) {
+                const int sv = j % F::STV;
+                mbar_wait_warp(&bar[kBVfull + sv], (j / F::STV) & 1, abort_flag, p.err);
                 const uint64_t dv = dv0 + static_cast<uint64_t>(sv * (F::VPAGE >> 4));
-                const bool acc = jj > 0;
 #pragma unroll
-                for (int ks = 0; ks < kPT / 16; ++ks) {
-                    umma_bf16(tmem + F::TM_O, dp + ks * (4096 >> 4), dv + ks * (2048 >> 4), idv0, acc || ks > 0);
-                    if constexpr (F::N1 > 0)
-                        umma_bf16(tmem + F::TM_O + F::N0, dp + ks * (4096 >> 4),
-                                  dv + ((F::N0 / 64) * (kPT * 128) >> 4) + ks * (2048 >> 4), idv1,
-                                  acc || ks > 0);
+                for (int i = 0; i < NT; ++i) {
+                    const int g = NT == 2 ? i : (j & 1), jj = NT == 2 ? j : (j >> 1);
+                    if (NT == 2 && j >= npu(i)) continue;
+                    mbar_wait_warp(&bar[kBPfull + g], jj & 1, abort_flag, p.err);
+                    tc_fence_after();
+                    const uint32_t to = tmem + F::TM_O + i * F::ORV;
+                    const bool acc = j > 0;
+#pragma unroll
+                    for (int part = 0; part < QP; ++part)
+#pragma unroll
+                        for (int ks = 0; ks < kPT / 16; ++ks) {
+                            const uint32_t tp = tmem + F::TM_P + (g * QP + part) * (kPT / 2) + ks * 8;
+                            umma_bf16_ts_warp(to, tp, dv + ks * (2048 >> 4), idv0, acc || part > 0 || ks > 0);
+                            if constexpr (F::N1 > 0)
+                                umma_bf16_ts_warp(to + F::N0, tp, dv + ((F::N0 / 64) * (kPT * 128) >> 4) + ks * (2048 >> 4), idv1,
+                                             acc || part > 0 || ks > 0);
+                        }
+                    umma_commit_warp(&bar[kBPfree + g]);
+                    if (NT == 2 && j == npu(i) - 1) umma_commit_warp(&bar[kBOfin + i]);
                 }
-                umma_commit(&bar[kBVempty + sv]);
-                umma_commit(&bar[kBPfree + s]);
+                umma_commit_warp(&bar[kBVempty + sv]);
             }
-            umma_commit(&bar[kBOfin]);  // every PV MMA (and, before them, every S MMA) has completed
-            // out = (O / l) W_up,t^V^T, with O / l = hi + lo as two bf16 operands in turn, so
-            // that the projection sees O / l to about 16 significant bits
-            mbar_wait(&bar[kBWv], 0, abort_flag, p.err);
-            constexpr uint32_t ido = umma_idesc_bf16(128, D, 0, 0);
-            const uint64_t doa = umma_desc(base + F::oOA, 2048, 128);
-            const uint64_t dwv = umma_desc(base + F::oWV, 2048, 128);
-#pragma unroll 1
-            for (int part = 0; part < 2; ++part) {
-                mbar_wait(&bar[part ? kBOa2 : kBOa], 0, abort_flag, p.err);
+            if constexpr (NT == 1) umma_commit_warp(&bar[kBOfin]);
+            // out = (O / l) W_up,t^V^T in two halves of 64 output columns, with O / l = hi + lo as two
+            // bf16 operands in TMEM, so that the projection sees O / l to about 16 significant bits.
+            // Chunk c of 64 latent columns: hi in the first half of its columns, lo in the second.
+            mbar_wait_warp(&bar[kBWv], 0, abort_flag, p.err);
+            constexpr uint32_t ido = umma_idesc_bf16(128, D / 2, 0, 0);
+            const uint64_t dwv = umma_desc_sw128_k(base + F::oWV);
+            auto project = [&](int tile, int half, uint32_t ds, uint64_t *done) {
+                bool acc = false;
+#pragma unroll
+                for (int c = 0; c < F::VATOMS; ++c) {
+                    constexpr int last = F::ORV - (F::VATOMS - 1) * 64;  // columns of the last chunk
+                    const int cols = c == F::VATOMS - 1 ? last : 64;
+#pragma unroll
+                    for (int part = 0; part < 2; ++part)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) {
+                            if (ks * 16 >= cols) continue;
+                            umma_bf16_ts_warp(ds, tmem + F::TM_O + tile * F::ORV + c * 64 + part * (cols / 2) + ks * 8,
+                                         dwv + ((c * (D * 128) + half * (64 * 128) + ks * 32) >> 4), ido, acc);
+                            acc = true;
+                        }
+                }
+                umma_commit_warp(done);
+            };
+            if constexpr (NT == 1) {
+                mbar_wait_warp(&bar[kBOa], 0, abort_flag, p.err);
                 tc_fence_after();
-#pragma unroll 1
-                for (int ks = 0; ks < RV / 16; ++ks)
-                    umma_bf16(tmem + 0, doa + ks * (4096 >> 4), dwv + ks * (4096 >> 4), ido, part > 0 || ks > 0);
-                umma_commit(&bar[part ? kBOut : kBOut1]);
+                for (int g = 0; g < 2; ++g) project(0, g, tmem + F::TM_S + g * kPT, &bar[kBOut + g]);
+            } else {
+                for (int half = 0; half < 2; ++half)
+                    for (int g = 0; g < 2; ++g) {
+                        if (npu(g) == 0) continue;
+                        // the first half has been read (so its product's phase has passed; after a failed
+                        // wait that product is awaited itself, so that the phases stay in step)
+                        if (!mbar_wait_warp(half ? &bar[kBOfree + g] : &bar[kBOa + g], 0, abort_flag, p.err) && half) {
+                            volatile int never = 0;
+                            mbar_wait_warp(&bar[kBOut + g], 0, &never, p.err);
+                        }
+                        tc_fence_after();
+                        project(g, half, tmem + F::TM_S + g * kPT, &bar[kBOut + g]);
+                    }
             }
-            volatile int never = 0;  // as for the S^T issuer: the last commit of this thread
-            mbar_wait(&bar[kBOut], 0, &never, p.err);
+            // as for the S issuer: this thread's last commits
+            volatile int never = 0;
+            for (int g = 0; g < 2; ++g) {
+                if (NT == 2 && npu(g) == 0) continue;
+                mbar_wait_warp(&bar[kBOut + g], NT == 1 ? 0 : 1, &never, p.err);
+            }
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ softmax and epilogue
-        // warps 4..11: quarter (TMEM lanes) = warp % 4, half = which 32 keys of a page (and which
-        // half of every other row-wise job) this thread owns; warps w and w + 4 share rows
+        // warps 4..7 are group 0, 8..11 group 1; thread = query row (TMEM lane) of the group's tile.
+        // NT = 2: group g owns tile g.  NT = 1: the groups take the tile's pages in turn.
         const int quarter = warp & 3;
-        const int half = (warp - kSWarp0) >> 2;
+        const int g = (warp - kSWarp0) >> 2;
+        const int tile = NT == 2 ? g : 0;
         const int row = quarter * 32 + lane;
-        const int pair_bar = 2 + quarter;  // named barrier of the two warps of this quarter
         const uint32_t tl = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-        const int qi = i0 + row;
+        const uint32_t ts = tl + F::TM_S + g * kPT, to = tl + F::TM_O + tile * F::ORV;
+        const uint32_t tp = tl + F::TM_P + g * QP * (kPT / 2);
+        const int qi = i0 + tile * kBM + row;
         const bool valid_row = qi < L;
         const int64_t qrow = (static_cast<int64_t>(q0) + qi) * p.H + h;
+        const int NPg = np(tile);
+        if (NT == 1 || NPg > 0) {
         if constexpr (ROPE) {
-            // the rotated, scaled q row (this half's 64 elements) -> the score operand directly
-            char *qt_ = sm + F::oQT + row * 16;
+            // the rotated, scaled q row -> the score operand directly (NT = 1: half a row per group)
+            char *qt_ = sm + F::oQT + tile * F::QT1 + row * 16;
             const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const char *>(p.qrot) + qrow * D * 2);
-            const int c0 = half * (D / 16);
+            constexpr int NC = NT == 1 ? D / 16 : D / 8;
+            const int c0 = NT == 1 ? g * NC : 0;
+            uint4 v[NC];
 #pragma unroll
-            for (int c = c0; c < c0 + D / 16; ++c)
-                *reinterpret_cast<uint4 *>(qt_ + c * 2048) = valid_row ? src[c] : make_uint4(0, 0, 0, 0);
+            for (int c = 0; c < NC; ++c) v[c] = valid_row ? src[c0 + c] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) *reinterpret_cast<uint4 *>(qt_ + (c0 + c) * 2048) = v[c];
             fence_proxy_async_smem();
-            mbar_arrive(&bar[kBSetup]);
-            mbar_wait(&bar[kBQt], 0, abort_flag, p.err);
-            mbar_arrive(&bar[kBQs]);
+            mbar_arrive(&bar[kBQs + (NT == 2 ? g : 0)]);
         } else {
-        // q row (this half's 64 elements) -> bf16 K-major operand: chunk c at c*2048 + row*16
-        {
-            char *qa = sm + F::oQA + row * 16;
-            const int c0 = half * (D / 16);
-            if (p.io_bf16) {
-                const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const char *>(p.q) + qrow * D * 2);
+            // q row -> bf16 K-major operand: chunk c at c*2048 + row*16 (NT = 1: group 0)
+            if (NT == 2 || g == 0) {
+                char *qa = sm + F::oQA + tile * F::QA1 + row * 16;
+                if (p.io_bf16) {
+                    const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const char *>(p.q) + qrow * D * 2);
+                    uint4 v[D / 8];
 #pragma unroll
-                for (int c = c0; c < c0 + D / 16; ++c)
-                    *reinterpret_cast<uint4 *>(qa + c * 2048) = valid_row ? src[c] : make_uint4(0, 0, 0, 0);
-            } else {
-                const float4 *src = reinterpret_cast<const float4 *>(static_cast<const char *>(p.q) + qrow * D * 4);
+                    for (int c = 0; c < D / 8; ++c) v[c] = valid_row ? src[c] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-                for (int c = c0; c < c0 + D / 16; ++c) {
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a;
-                    if (valid_row) {
-                        a = src[2 * c];
-                        b2 = src[2 * c + 1];
+                    for (int c = 0; c < D / 8; ++c) *reinterpret_cast<uint4 *>(qa + c * 2048) = v[c];
+                } else {
+                    const float4 *src = reinterpret_cast<const float4 *>(static_cast<const char *>(p.q) + qrow * D * 4);
+#pragma unroll
+                    for (int c = 0; c < D / 8; ++c) {
+                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a;
+                        if (valid_row) {
+                            a = src[2 * c];
+                            b2 = src[2 * c + 1];
+                        }
+                        *reinterpret_cast<uint4 *>(qa + c * 2048) =
+                            make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b2.x, b2.y),
+                                       pack_bf16x2(b2.z, b2.w));
                     }
-                    *reinterpret_cast<uint4 *>(qa + c * 2048) =
-                        make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b2.x, b2.y),
-                                   pack_bf16x2(b2.z, b2.w));
+                }
+                fence_proxy_async_smem();
+                mbar_arrive(&bar[kBQa + g]);
+            }
+            // q~ (scaled into the exp2 domain) -> bf16 K-major operand, in QP parts (each the rounding
+            // of what the part before leaves); NT = 1: the groups take its 16-column chunks in turn
+            mbar_wait(&bar[kBQt + tile], 0, abort_flag, p.err);
+            tc_fence_after();
+            char *qt_ = sm + F::oQT + tile * QP * F::QT1 + row * 16;
+            const float sc = p.scale_log2;
+#pragma unroll 1
+            for (int c0 = (NT == 1 ? g * 16 : 0); c0 < F::RKX; c0 += (NT == 1 ? 32 : 16)) {
+                float v[16];
+                tmem_ld16(to + c0, v);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) v[k] *= sc;
+#pragma unroll
+                for (int part = 0; part < QP; ++part) {
+#pragma unroll
+                    for (int k = 0; k < 16; k += 8) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            w[e] = pack_bf16x2(v[k + 2 * e], v[k + 2 * e + 1]);
+                            if (part + 1 < QP) {
+                                const float2 f = bf2_to_f2(w[e]);
+                                v[k + 2 * e] -= f.x;
+                                v[k + 2 * e + 1] -= f.y;
+                            }
+                        }
+                        *reinterpret_cast<uint4 *>(qt_ + part * F::QT1 + ((c0 + k) / 8) * 2048) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
                 }
             }
-        }
-        fence_proxy_async_smem();
-        mbar_arrive(&bar[kBSetup]);
-        // q~ (scaled into the exp2 domain) -> bf16 K-major operand; this half's RK/2 columns
-        mbar_wait(&bar[kBQt], 0, abort_flag, p.err);
-        tc_fence_after();
-#pragma unroll 1
-        for (int c0 = half * (RK / 2); c0 < (half + 1) * (RK / 2); c0 += 16) {
-            float v[16];
-            tmem_ld16(tl + c0, v);
-            char *qt_ = sm + F::oQT + row * 16;
-            const float sc = p.scale_log2;
-#pragma unroll
-            for (int k = 0; k < 16; k += 8)
-                *reinterpret_cast<uint4 *>(qt_ + ((c0 + k) / 8) * 2048) =
-                    make_uint4(pack_bf16x2(v[k] * sc, v[k + 1] * sc), pack_bf16x2(v[k + 2] * sc, v[k + 3] * sc),
-                               pack_bf16x2(v[k + 4] * sc, v[k + 5] * sc), pack_bf16x2(v[k + 6] * sc, v[k + 7] * sc));
-        }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        mbar_arrive(&bar[kBQs]);
+            fence_proxy_async_smem();
+            tc_fence_before();
+            mbar_arrive(&bar[kBQs + (NT == 2 ? g : 0)]);
         }
 
         const int lim = min(qi, L - 1);  // keys 0..lim are visible to this row
-        const int kofs = half * 32;      // this thread's keys within a page
+        float *mrun = reinterpret_cast<float *>(sm + F::oM);
         float m = -INFINITY, l = 0.f;
+        // jj counts this group's pages
 #pragma unroll 1
-        for (int j = 0; j < NP; ++j) {
-            const int s = j & 1;
+        for (int j = NT == 1 ? g : 0, jj = 0; j < NPg; j += NT == 1 ? 2 : 1, ++jj) {
             const int kb = j * kPT;
-            mbar_wait(&bar[kBSfull + s], (j >> 1) & 1, abort_flag, p.err);
+            mbar_wait(&bar[kBSfull + g], jj & 1, abort_flag, p.err);
             tc_fence_after();
-            float x[32];
-            tmem_ld32(tl + F::TM_S + s * kPT + kofs, x);
+            float x[kPT];
+            tmem_ld64(ts, x);
             tc_fence_before();
-            mbar_arrive(&bar[kBSfree + s]);
-            if (kb + kPT - 1 > i0) {  // a page on the diagonal (or past the prompt): mask
-                const int nv = lim - (kb + kofs);  // keys c <= nv are visible
+            mbar_arrive(&bar[kBSfree + g]);
+            if (kb + kPT - 1 > i0 + tile * kBM) {  // a page on the diagonal (or past the prompt): mask
+                const int nv = lim - kb;           // keys c <= nv are visible
 #pragma unroll
-                for (int c = 0; c < 32; ++c) x[c] = c <= nv ? x[c] : -INFINITY;
+                for (int c = 0; c < kPT; ++c) x[c] = c <= nv ? x[c] : -INFINITY;
             }
             float mx;
-            {  // tree maximum: 5 dependent steps instead of 32
-                float t[16];
+            {
+                float t[4];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) t[c] = fmaxf(x[c], x[c + 16]);
+                for (int c = 0; c < 4; ++c) t[c] = x[c];
 #pragma unroll
-                for (int w = 8; w >= 1; w >>= 1)
+                for (int c = 4; c < kPT; c += 8)
 #pragma unroll
-                    for (int c = 0; c < w; ++c) t[c] = fmaxf(t[c], t[c + w]);
-                mx = t[0];
+                    for (int e = 0; e < 4; ++e) t[e] = c + 4 + e < kPT ? fmaxf(fmaxf(t[e], x[c + e]), x[c + 4 + e]) : fmaxf(t[e], x[c + e]);
+                mx = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3]));
             }
-            // the row maximum over both halves
-            xmax[(s * 2 + half) * kBM + row] = mx;
-            named_bar_sync(pair_bar, 64);
-            mx = fmaxf(mx, xmax[(s * 2 + (half ^ 1)) * kBM + row]);
+            if constexpr (NT == 1) {
+                // the running maximum after page j - 1, from the other group's thread of this row; every
+                // page's weights are relative to the running maximum its own step leaves
+                if (j > 0) {
+                    named_bar_sync(1 + quarter * 2 + ((j - 1) & 1), 64);
+                    const float mp = mrun[row];
+                    if (mp != m) {
+                        l *= ex2_approx(m - mp);  // (m = -inf: no page yet, l = 0)
+                        m = mp;
+                    }
+                }
+            }
             const float m_new = fmaxf(m, mx);
             const bool need = m_new > m + kRescaleLog2;  // also the first finite maximum
             const float factor = need ? ex2_approx(m - m_new) : 1.f;
@@ -480,42 +611,65 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 l *= factor;
                 m = m_new;
             }
-            if (__any_sync(0xffffffffu, need && j > 0)) {
-                // O holds pages 0..j-1: wait for the last of them, then rescale this half.  The
-                // product of page j - 1 releases P buffer (j - 1) & 1; the one of page j - 3 had
-                // released it before this row wrote page j - 1, so the parity test cannot pass a
-                // phase early (a barrier committed once per page could be two phases behind)
-                mbar_wait(&bar[kBPfree + ((j - 1) & 1)], ((j - 1) >> 1) & 1, abort_flag, p.err);
-                tc_fence_after();
-#pragma unroll 1
-                for (int c0 = half * (RV / 2); c0 < (half + 1) * (RV / 2); c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tl + F::TM_O + c0, v);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] *= factor;
-                    tmem_st16(tl + F::TM_O + c0, v);
+            if constexpr (NT == 1) {
+                if (j + 1 < NPg) {
+                    mrun[row] = m;
+                    named_bar_arrive(1 + quarter * 2 + (j & 1), 64);
                 }
             }
-            if (j >= 2) mbar_wait(&bar[kBPfree + s], ((j - 2) >> 1) & 1, abort_flag, p.err);
-            char *pr = sm + F::oP + s * F::PB + row * 16 + (kofs / 8) * 2048;
+            const bool any = __any_sync(0xffffffffu, need && j > 0);
+            // this group's previous page has been read by its product (and O holds it)
+            auto wait_own = [&] {
+                if (jj > 0) mbar_wait(&bar[kBPfree + g], (jj - 1) & 1, abort_flag, p.err);
+            };
+            if (any) {
+                // O holds pages 0..j-1: wait for the last of them, then rescale.  For NT = 1 that page
+                // is the other group's; this group's own, one page earlier, is waited for first: products
+                // complete in order, so the other group's barrier is then at most one phase behind
+                // and its parity test cannot pass a phase early.
+                wait_own();
+                if constexpr (NT == 1) mbar_wait(&bar[kBPfree + (g ^ 1)], ((j - 1) >> 1) & 1, abort_flag, p.err);
+                tc_fence_after();
+#pragma unroll 1
+                for (int c0 = 0; c0 < F::ORV; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(to + c0, v);
 #pragma unroll
-            for (int c = 0; c < 32; ++c) x[c] = ex2_approx(x[c] - m);
-#pragma unroll
-            for (int c = 0; c < 32; c += 8)
-                *reinterpret_cast<uint4 *>(pr + (c / 8) * 2048) =
-                    make_uint4(pack_bf16x2(x[c], x[c + 1]), pack_bf16x2(x[c + 2], x[c + 3]),
-                               pack_bf16x2(x[c + 4], x[c + 5]), pack_bf16x2(x[c + 6], x[c + 7]));
-            {  // tree sum of this half's probabilities
-                float t[16];
-#pragma unroll
-                for (int c = 0; c < 16; ++c) t[c] = x[c] + x[c + 16];
-#pragma unroll
-                for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-                    for (int c = 0; c < w; ++c) t[c] += t[c + w];
-                l += t[0];
+                    for (int c = 0; c < 16; ++c) v[c] *= factor;
+                    tmem_st16(to + c0, v);
+                }
             }
-            if (j == NP - 1 && kb + kPT > L) {
+            {
+                const float2 mm = make_float2(-m, -m);
+                float2 s4[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s4[e] = make_float2(0.f, 0.f);
+                uint32_t w[kPT / 2];
+#pragma unroll
+                for (int c = 0; c < kPT; c += 2) {
+                    float2 y = __fadd2_rn(make_float2(x[c], x[c + 1]), mm);
+                    y.x = ex2_approx(y.x);
+                    y.y = ex2_approx(y.y);
+                    s4[(c >> 1) & 3] = __fadd2_rn(s4[(c >> 1) & 3], y);
+                    w[c / 2] = pack_bf16x2(y.x, y.y);
+                    if constexpr (QP > 1) {
+                        const float2 f = bf2_to_f2(w[c / 2]);
+                        x[c] = y.x - f.x;
+                        x[c + 1] = y.y - f.y;
+                    }
+                }
+                const float2 sa = __fadd2_rn(s4[0], s4[1]), sb = __fadd2_rn(s4[2], s4[3]);
+                l += (sa.x + sa.y) + (sb.x + sb.y);
+                if (!any) wait_own();
+                tc_fence_after();
+                tmem_st32u_nowait(tp, w);
+                if constexpr (QP > 1) {
+#pragma unroll
+                    for (int c = 0; c < kPT; c += 2) w[c / 2] = pack_bf16x2(x[c], x[c + 1]);
+                    tmem_st32u_nowait(tp + kPT / 2, w);
+                }
+            }
+            if (j == NPg - 1 && kb + kPT > L) {
                 // last page of the prompt: V rows past it hold no latents; zero them before the
                 // PV product reads them (0 * NaN would poison the sum)
                 const int sv = j % F::STV;
@@ -523,77 +677,94 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 char *vs = sm + F::oV + sv * F::VPAGE;
                 const int valid = L - kb;
                 const int nz = (kPT - valid) * F::VATOMS * 8;  // 16-byte words to clear
-                for (int w = tid - kSWarp0 * 32; w < nz; w += kSThreads) {
+                for (int w = row; w < nz; w += kGroup) {
                     const int c = w & 7, r2 = w >> 3;
                     const int a = r2 % F::VATOMS, i = valid + r2 / F::VATOMS;
                     *reinterpret_cast<uint4 *>(vs + a * (kPT * 128) + i * 128 + c * 16) = make_uint4(0, 0, 0, 0);
                 }
+                fence_proxy_async_smem();
             }
-            fence_proxy_async_smem();
+            tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(&bar[kBPfull + s]);
+            mbar_arrive(&bar[kBPfull + g]);
         }
-        // the row sum over both halves
-        xsum[half * kBM + row] = l;
-        named_bar_sync(pair_bar, 64);
-        l += xsum[(half ^ 1) * kBM + row];
-        // epilogue: O / l -> two bf16 K-major operands in turn (hi, then lo = O/l - hi) in one
-        // buffer that aliases the K ring; O stays in TMEM between the two
-        mbar_wait(&bar[kBOfin], 0, abort_flag, p.err);
+        if constexpr (NT == 1) {
+            // the row's sum over both groups, relative to the later maximum
+            float2 *xs = reinterpret_cast<float2 *>(sm + F::oX);
+            xs[g * kBM + row] = make_float2(m, l);
+            named_bar_sync(9 + quarter, 64);
+            const float2 o = xs[(g ^ 1) * kBM + row];
+            const float mf = fmaxf(m, o.x);
+            l = (m == mf ? l : l * ex2_approx(m - mf)) + (o.x == mf ? o.y : o.y * ex2_approx(o.x - mf));
+        }
+        // epilogue: O / l -> hi and lo = O/l - hi as packed bf16 pairs in the chunk's own columns
+        mbar_wait(&bar[kBOfin + tile], 0, abort_flag, p.err);
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
+        // (a loop of its own code, not unrolled over the chunks: straight-line code run once is
+        // fetched at every instruction)
+        constexpr int last = F::ORV - (F::VATOMS - 1) * 64;
+        static_assert(last == 64 || last == 32, "columns of the last chunk");
 #pragma unroll 1
-        for (int part = 0; part < 2; ++part) {
-            if (part) {
-                mbar_wait(&bar[kBOut1], 0, abort_flag, p.err);  // the hi product has read the buffer
-                tc_fence_after();
-            }
-#pragma unroll 1
-            for (int c0 = half * (RV / 2); c0 < (half + 1) * (RV / 2); c0 += 16) {
-                float v[16];
-                tmem_ld16(tl + F::TM_O + c0, v);
+        for (int c = NT == 1 ? g : 0; c < F::VATOMS; c += NT == 1 ? 2 : 1) {
+            const uint32_t half = c == F::VATOMS - 1 ? last / 2 : 32;  // packed columns of hi, of lo
+            // 32 columns at a time: a chunk's first 32 hold its hi, so its second half is read first
+            float v[32], u[32];
+            tmem_ld32(to + c * 64, v);
+            if (half == 32) tmem_ld32(to + c * 64 + 32, u);
+            uint32_t hi[16], lo[16];
+            auto convert = [&](const float (&v)[32]) {
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
-                    const float xv = v[k] * inv;
-                    const float hi = __bfloat162float(__float2bfloat16_rn(xv));
-                    v[k] = part ? xv - hi : hi;
+                    const float a = v[2 * k] * inv, bb = v[2 * k + 1] * inv;
+                    hi[k] = pack_bf16x2(a, bb);
+                    const float2 f = bf2_to_f2(hi[k]);
+                    lo[k] = pack_bf16x2(a - f.x, bb - f.y);
                 }
-                char *oa = sm + F::oOA + row * 16;
-#pragma unroll
-                for (int k = 0; k < 16; k += 8)
-                    *reinterpret_cast<uint4 *>(oa + ((c0 + k) / 8) * 2048) =
-                        make_uint4(pack_bf16x2(v[k], v[k + 1]), pack_bf16x2(v[k + 2], v[k + 3]),
-                                   pack_bf16x2(v[k + 4], v[k + 5]), pack_bf16x2(v[k + 6], v[k + 7]));
+            };
+            convert(v);
+            tmem_st16u(to + c * 64, hi);
+            tmem_st16u(to + c * 64 + half, lo);
+            if (half == 32) {
+                convert(u);
+                tmem_st16u(to + c * 64 + 16, hi);
+                tmem_st16u(to + c * 64 + 48, lo);
             }
-            fence_proxy_async_smem();
-            tc_fence_before();
-            mbar_arrive(&bar[part ? kBOa2 : kBOa]);
         }
-        mbar_wait(&bar[kBOut], 0, abort_flag, p.err);
-        tc_fence_after();
-        const float *muv = p.mu_v ? p.mu_v + wofs : nullptr;
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(&bar[kBOa + tile]);
+        const float *muv = p.mu_v ? p.mu_v + wrow : nullptr;
+        // NT = 1: group g stores half g of the output columns; NT = 2: both halves, one after the other
 #pragma unroll 1
-        for (int c0 = half * (D / 2); c0 < (half + 1) * (D / 2); c0 += 32) {
-            float v[32];
-            tmem_ld32(tl + c0, v);
+        for (int half = NT == 1 ? g : 0; half < (NT == 1 ? g + 1 : 2); ++half) {
+            mbar_wait(&bar[kBOut + g], NT == 1 ? 0 : half, abort_flag, p.err);
+            tc_fence_after();
+            float v[64];
+            tmem_ld64(ts, v);
+            if (NT == 2 && half == 0) {
+                tc_fence_before();
+                mbar_arrive(&bar[kBOfree + g]);
+            }
             if (muv) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) v[c] += muv[c0 + c];
+                for (int c = 0; c < 64; ++c) v[c] += muv[half * 64 + c];
             }
             if (valid_row) {
-                char *dst = static_cast<char *>(p.out) + (qrow * D + c0) * (p.io_bf16 ? 2 : 4);
+                char *dst = static_cast<char *>(p.out) + (qrow * D + half * 64) * (p.io_bf16 ? 2 : 4);
                 if (p.io_bf16) {
 #pragma unroll
-                    for (int k = 0; k < 32; k += 8)
+                    for (int k = 0; k < 64; k += 8)
                         *reinterpret_cast<uint4 *>(dst + k * 2) =
                             make_uint4(pack_bf16x2(v[k], v[k + 1]), pack_bf16x2(v[k + 2], v[k + 3]),
                                        pack_bf16x2(v[k + 4], v[k + 5]), pack_bf16x2(v[k + 6], v[k + 7]));
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 32; k += 4)
+                    for (int k = 0; k < 64; k += 4)
                         *reinterpret_cast<float4 *>(dst + k * 4) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
                 }
             }
+        }
         }
     }
     pdl_trigger();
@@ -1002,31 +1173,68 @@ lla_status launch_pf(K kern, dim3 grid, int threads, int smem, cudaStream_t stre
     return LLA_OK;
 }
 
-template <int RK, int RV, bool ROPE = false>
-lla_status launch_tc(const PParams &prm, int nqt, int B, int H, cudaStream_t stream) {
+template <int RK, int RV, int NT, bool ROPE, int QP>
+lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {
+    using F = PF<RK, RV, NT, ROPE, QP>;
     static DeviceOnce configured;
-    if (raise_smem_limit(prefill_tc_kernel<RK, RV, ROPE>, PF<RK, RV, ROPE>::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
+    if (raise_smem_limit(prefill_tc_kernel<RK, RV, NT, ROPE, QP>, F::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
     // the V-planes of every head page: [pages][64 tokens][r_v] bf16, one page = one head page
-    CUtensorMap tv;
+    CUtensorMap tv, twk, twv;
     const uint64_t dims[3] = {static_cast<uint64_t>(RV), static_cast<uint64_t>(kPT),
                               static_cast<uint64_t>(prm.num_blocks) * prm.H};
     const uint64_t strides[2] = {static_cast<uint64_t>(RV) * 2, static_cast<uint64_t>(prm.head_page_bytes)};
     const uint32_t box[3] = {64, kPT, 1};
     if (!encode_tmap_bf16(&tv, prm.pool + kPT * RK * 2, 3, dims, strides, box, true)) return LLA_ERR_CUDA;
+    // W_up of both axes: [H T d][r] bf16, the d rows of one (head, loop) at a time
+    const uint64_t wk[2] = {static_cast<uint64_t>(RK), static_cast<uint64_t>(prm.H) * prm.T * F::D};
+    const uint64_t wv[2] = {static_cast<uint64_t>(RV), wk[1]};
+    const uint64_t sk[1] = {static_cast<uint64_t>(RK) * 2}, sv[1] = {static_cast<uint64_t>(RV) * 2};
+    const uint32_t wbox[2] = {64, F::D};
+    if (!encode_tmap_bf16(&twk, a.w_up_k, 2, wk, sk, wbox, true) || !encode_tmap_bf16(&twv, a.w_up_v, 2, wv, sv, wbox, true))
+        return LLA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     // x fastest: the tiles of one (sequence, head), longest first, run together and share its
     // pages in L2 (ordering the longest tiles of every head first was slower: 1.90 -> 2.17 ms)
-    cfg.gridDim = dim3(nqt, B, H);
+    cfg.gridDim = dim3((a.max_len + NT * kBM - 1) / (NT * kBM), a.B, a.H);
     cfg.blockDim = dim3(kPThreads);
-    cfg.dynamicSmemBytes = PF<RK, RV, ROPE>::SMEM;
+    cfg.dynamicSmemBytes = F::SMEM;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, prefill_tc_kernel<RK, RV, ROPE>, tv, prm) != cudaSuccess) return LLA_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, prefill_tc_kernel<RK, RV, NT, ROPE, QP>, tv, twk, twv, prm) != cudaSuccess) return LLA_ERR_CUDA;
     return LLA_OK;
+}
+
+// One query tile per CTA, or two that share every page.  Two halve the pages' way through L2 and need no
+// hand-over of maxima, but a CTA's work is twice as long, so that few CTAs end unevenly: one prompt of
+// 8192 tokens at (96, 160) (512 pairs of tiles) takes 255 us with one tile and 274 with two, two such
+// prompts (1024) 496 and 493, four 994 and 944.  With rotated keys (128 wide instead of 96) the pages
+// weigh more: 396 and 375 us at 512 pairs, 135 and 146 at 256.  With two bf16 parts the products bound
+// it either way (1317 and 1333 us), so (72, 120) takes one.
+template <int RK, int RV, bool ROPE, int QP = 1>
+lla_status launch_tc(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {
+    if constexpr (RV <= 160 && QP == 1) {
+        const int64_t pairs = static_cast<int64_t>((a.max_len + 2 * kBM - 1) / (2 * kBM)) * a.B * a.H;
+        if (pairs >= (ROPE ? 512 : 1024)) return launch_tiles<RK, RV, 2, ROPE, QP>(prm, a, stream);
+    }
+    return launch_tiles<RK, RV, 1, ROPE, QP>(prm, a, stream);
+}
+
+PParams tc_params(const PrefillArgs &a, int hpb, unsigned *err) {
+    PParams p = {};
+    p.T = a.T; p.H = a.H; p.loop = a.loop; p.io_bf16 = a.io_bf16;
+    p.scale_log2 = a.scale * kLog2e;
+    p.mu_v = a.mu_v;
+    p.pool = static_cast<const char *>(a.pool);
+    p.num_blocks = a.num_blocks;
+    p.head_page_bytes = hpb;
+    p.block_table = a.block_table; p.max_blocks = a.max_blocks;
+    p.cu_seqlens = a.cu_seqlens; p.max_len = a.max_len;
+    p.q = a.q; p.out = a.out; p.err = err;
+    return p;
 }
 
 }  // namespace
@@ -1040,24 +1248,11 @@ lla_status launch_prefill(const PrefillArgs &a, cudaStream_t stream) {
     if (a.B > 65535 || a.H > 65535) return LLA_ERR_UNSUPPORTED;
     // the tensor-core kernel addresses head pages with a 32-bit TMA coordinate
     if (a.storage_bf16 && a.d == 128 && a.num_blocks * a.H < (int64_t(1) << 31)) {
-        PParams p = {};
-        p.T = a.T; p.H = a.H; p.loop = a.loop; p.io_bf16 = a.io_bf16;
-        p.scale_log2 = a.scale * kLog2e;
-        p.w_up_k = a.w_up_k; p.w_up_v = a.w_up_v; p.mu_v = a.mu_v;
-        p.pool = static_cast<const char *>(a.pool);
-        p.num_blocks = a.num_blocks;
-        p.head_page_bytes = hpb;
-        p.block_bytes = static_cast<int64_t>(hpb) * a.H;
-        p.block_table = a.block_table; p.max_blocks = a.max_blocks;
-        p.cu_seqlens = a.cu_seqlens; p.B = a.B; p.max_len = a.max_len;
-        p.q = a.q; p.out = a.out; p.err = err;
-        const int nqt = (a.max_len + kBM - 1) / kBM;
-#define LLA_PF(K, V) \
-        if (a.r_k == K && a.r_v == V) return launch_tc<K, V>(p, nqt, a.B, a.H, stream);
-        LLA_PF(96, 160)
-        LLA_PF(192, 320)
-        LLA_PF(128, 128)
-#undef LLA_PF
+        const PParams p = tc_params(a, hpb, err);
+        if (a.r_k == 96 && a.r_v == 160) return launch_tc<96, 160, false>(p, a, stream);
+        if (a.r_k == 192 && a.r_v == 320) return launch_tc<192, 320, false>(p, a, stream);
+        if (a.r_k == 128 && a.r_v == 128) return launch_tc<128, 128, false>(p, a, stream);
+        if (a.r_k == 72 && a.r_v == 120 && a.io_bf16) return launch_tc<72, 120, false, 2>(p, a, stream);
     }
     GParams g = {};
     g.T = a.T; g.H = a.H; g.d = a.d; g.r_k = a.r_k; g.r_v = a.r_v; g.loop = a.loop;
@@ -1133,23 +1328,12 @@ lla_status launch_prefill_rope(const PrefillArgs &a, double base, int pairing, v
     else if (a.r_k == 128) rs = launch_rebuild<128>(r, kpps, a.B, stream);
     if (rs != LLA_OK) return rs;
 
-    PParams p = {};
-    p.T = a.T; p.H = a.H; p.loop = a.loop; p.io_bf16 = a.io_bf16;
-    p.scale_log2 = a.scale * kLog2e;
-    p.w_up_k = a.w_up_k; p.w_up_v = a.w_up_v; p.mu_v = a.mu_v;
-    p.pool = static_cast<const char *>(a.pool);
-    p.num_blocks = a.num_blocks;
-    p.head_page_bytes = hpb;
-    p.block_bytes = static_cast<int64_t>(hpb) * a.H;
-    p.block_table = a.block_table; p.max_blocks = a.max_blocks;
-    p.cu_seqlens = a.cu_seqlens; p.B = a.B; p.max_len = a.max_len;
-    p.q = a.q; p.out = a.out; p.err = err;
+    PParams p = tc_params(a, hpb, err);
     p.krot = krot; p.qrot = qrot; p.kpps = kpps;
     p.qrows = static_cast<int64_t>(a.B) * a.max_len;
-    const int nqt = (a.max_len + kBM - 1) / kBM;
-    if (a.r_k == 96) return launch_tc<96, 160, true>(p, nqt, a.B, a.H, stream);
-    if (a.r_k == 192) return launch_tc<192, 320, true>(p, nqt, a.B, a.H, stream);
-    return launch_tc<128, 128, true>(p, nqt, a.B, a.H, stream);
+    if (a.r_k == 96) return launch_tc<96, 160, true>(p, a, stream);
+    if (a.r_k == 192) return launch_tc<192, 320, true>(p, a, stream);
+    return launch_tc<128, 128, true>(p, a, stream);
 }
 
 }  // namespace lla

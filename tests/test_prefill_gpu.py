@@ -107,3 +107,55 @@ def test_prefill_rejects_bad_context(lla):
     torch.cuda.synchronize()
     assert lla.lla_get_device_error() & 0x2  # LLA_DEVERR_CONTEXT
     lla.lla_clear_device_error()
+
+
+def _rising_scores_case(lla, r_k, r_v, H, lens, seed, tol):
+    """Row maxima that rise from page to page: token i's keys are scaled by 1 + i / 64, so the running
+    maximum passes the rescale threshold (2^8) every page or two, in some rows of a warp and not in
+    others."""
+    from paper_2607_15456_gb300 import workloads as W
+    sc = Scene(lla, T=4, H=H, d=128, r_k=r_k, r_v=r_v, storage="bf16", io="bf16", lens=lens, seed=seed,
+               with_mu=True, extra_tokens=0)
+    N = sum(lens)
+    grow = torch.cat([1 + torch.arange(L, device=DEV) / 64 for L in lens]).view(1, N, 1, 1)
+    x = [(W.normal((4, N, H, 128), seed, 70 + i, dtype=torch.float32, device=DEV) * (grow if i == 0 else 1)).to(torch.bfloat16)
+         for i in range(2)]
+    slots = torch.cat([sc.pt.slots(b, range(L)) for b, L in enumerate(lens)]).to(DEV)
+    lla.lla_encode(sc.geom, sc.codec, sc.cache, x[0].contiguous(), x[1].contiguous(), slots)
+    q = W.normal((N, H, 128), seed, 72, device=DEV)
+    out = torch.full_like(q, float("nan"))
+    cu = torch.tensor(np.cumsum([0] + list(lens)), dtype=torch.int32, device=DEV)
+    lla.lla_prefill_attn(sc.geom, sc.codec, sc.cache, cu, max(lens), 1, q, out)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    got, q64, w, off = f64(out), f64(q), sc.w64, 0
+    for b, L in enumerate(lens):
+        for h in range(H):
+            gk, gv = sc.gpu_latents(b, h)
+            ref = oracle.prefill(1, gk, gv, w["w_up_k"][h], w["w_up_v"][h], w["mu_k"][h], w["mu_v"][h],
+                                 q64[off:off + L, h], sc.scale)
+            err = rel_l2(got[off:off + L, h], ref)
+            assert err <= tol, (b, h, err)
+        off += L
+
+
+def test_prefill_rising_scores_one_tile_per_cta(lla):
+    # the two softmax groups take a tile's pages in turn and hand the running maximum on.  At (72, 120)
+    # q~ and the softmax weights are sums of two bf16 parts: bf16 outputs are then as exact as their
+    # own rounding (2^-9 relative) however large the scores
+    _rising_scores_case(lla, 72, 120, 2, [700, 321], 31, 2 ** -9 + 1e-4)
+
+
+def test_prefill_rising_scores_two_tiles_per_cta(lla):
+    # 5 pairs of tiles x 13 prompts x 16 heads = 1040: each group owns a tile.  q~ is rounded to bf16
+    # (2^-9 / sqrt 3 of each term, so 1.1e-3 sigma of a score whose sigma reaches 1 + 1030 / 64 = 17, of
+    # which the few keys that share a row's weight see sqrt 2) and so is every weight (2^-9)
+    _rising_scores_case(lla, 96, 160, 16, [1030, 500, 385, 384, 257, 256, 255, 129, 128, 127, 64, 63, 1], 32,
+                        1.1e-3 * 17 * 2 ** 0.5 + 2 ** -8)
+
+
+@pytest.mark.parametrize("r_k,r_v,io", [(96, 160, "bf16"), (96, 160, "fp32"), (128, 128, "bf16")])
+def test_prefill_two_tiles_per_cta(lla, r_k, r_v, io):
+    # 5 pairs x 13 prompts x 16 heads = 1040: second tiles that are empty, one row, part of a page, full
+    _prefill_case(lla, r_k, r_v, "bf16", io, [1025, 520, 513, 512, 448, 385, 384, 383, 130, 129, 128, 64, 1], 2, True,
+                  H=16, seed=6)

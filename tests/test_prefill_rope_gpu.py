@@ -99,3 +99,29 @@ def test_rope_prefill_rejects_rows_past_the_workspace(lla):
     torch.cuda.synchronize()
     assert lla.lla_get_device_error() & lla.LLA_DEVERR_CONTEXT
     lla.lla_clear_device_error()
+
+
+@pytest.mark.parametrize("rk,rv", [(96, 160), (128, 128)])
+def test_rope_prefill_two_tiles_per_cta(lla, rk, rv):
+    """3 pairs of tiles x 15 prompts x 16 heads = 720 CTAs of two query tiles each, against the oracle on
+    the latents the GPU stored: relative L2 per (prompt, head), as in _case.  (No bound on the single
+    largest of 6 million values: rows of a few keys reach |o| = 6, where the bf16 roundings of weights,
+    rotated keys and output, 2^-9 each, add up to more than 2e-2 at some of them.)"""
+    lens, H, loop, base = [520, 385, 384, 300, 257, 256, 200, 129, 128, 127, 65, 64, 63, 2, 1], 16, 1, 10000.0
+    sc = Scene(lla, T=4, H=H, d=128, r_k=rk, r_v=rv, storage="bf16", io="bf16", lens=lens, seed=84, with_mu=True,
+               extra_tokens=0)
+    q = sc.W.normal((sum(lens), H, 128), 84, 70, loop, device=DEV)
+    out = torch.full_like(q, float("nan"))
+    cu = torch.tensor(np.cumsum([0] + lens), dtype=torch.int32, device=DEV)
+    ws = torch.empty(lla.lla_prefill_rope_workspace_size(sc.geom, len(lens), max(lens)), dtype=torch.uint8, device=DEV)
+    lla.lla_prefill_attn_rope(sc.geom, sc.codec, sc.cache, base, 1, cu, max(lens), loop, q, out, ws)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    got, q64, w, off = f64(out), f64(q), sc.w64, 0
+    for b, L in enumerate(lens):
+        for h in range(H):
+            gk, gv = sc.gpu_latents(b, h)
+            ref = oracle.prefill_rope(loop, gk, gv, w["w_up_k"][h], w["w_up_v"][h], w["mu_k"][h], w["mu_v"][h],
+                                      q64[off:off + L, h], sc.scale, base, 1)
+            assert rel_l2(got[off:off + L, h], ref) <= 5e-3, (b, h)
+        off += L

@@ -1,8 +1,10 @@
-"""Builds liblla.so (the CUDA library behind include/lla.h) in-tree for sm_103a.
+"""Builds liblla.so (the CUDA library behind include/lla.h) in-tree for sm_103a, and _lla_native.so
+(csrc/lla_binding.cpp: the native marshalling of the Python binding, linked to liblla.so beside it).
 
 Each translation unit is compiled by nvcc in parallel, then linked into
 paper_2607_15456_gb300/liblla.so with the CUDA runtime linked statically, so the library
-needs nothing but the driver at run time.
+needs nothing but the driver at run time.  The binding is one host translation unit against torch's
+headers, compiled beside them.
 """
 from __future__ import annotations
 
@@ -10,6 +12,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +20,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "liblla.so")
+NATIVE = os.path.join(PKG, "_lla_native.so")
+BINDING = os.path.join(CSRC, "lla_binding.cpp")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
@@ -36,14 +41,42 @@ def _sources():
 
 def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
-        os.path.join(CSRC, "*.h")) + [os.path.join(ROOT, "include", "lla.h"), __file__]
+        os.path.join(CSRC, "*.h")) + [BINDING, os.path.join(ROOT, "include", "lla.h"), __file__]
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(NATIVE)):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     return all(os.path.getmtime(p) <= t for p in _deps())
+
+
+def _run(cmd, what: str):
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"{what} failed:\n{res.stdout}\n{res.stderr}")
+
+
+def compile_binding() -> str:
+    """lla_binding.cpp as an object file, against this interpreter's Python and torch headers."""
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")
+    obj = os.path.join(BUILD, "lla_binding.o")
+    _run(["g++", "-O2", "-std=c++17", "-fPIC", "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+          "-I" + os.path.join(ROOT, "include"), "-I" + sysconfig.get_paths()["include"], "-isystem", inc,
+          "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", cuda, "-c", BINDING, "-o", obj],
+         "g++ on lla_binding.cpp")
+    return obj
+
+
+def link_binding(obj: str) -> None:
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = NATIVE + ".tmp%d" % os.getpid()
+    _run(["g++", "-shared", obj, "-o", tmp, "-L" + PKG, "-l:liblla.so", "-Wl,-rpath,$ORIGIN", "-L" + lib, "-ltorch_python",
+          "-ltorch_cpu", "-lc10", "-lc10_cuda"], "linking _lla_native.so")
+    os.replace(tmp, NATIVE)
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
@@ -66,13 +99,16 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         return obj
 
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 2)) as ex:
+        binding = ex.submit(compile_binding)
         objs = list(ex.map(compile_one, _sources()))
+        binding = binding.result()
     tmp = LIB + ".tmp%d" % os.getpid()
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", *objs, "-o", tmp]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
     os.replace(tmp, LIB)
+    link_binding(binding)
     return LIB
 
 

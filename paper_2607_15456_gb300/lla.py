@@ -2,7 +2,9 @@
 
 Every function here has the name of the C entry point it calls and does nothing but turn
 torch tensors into device pointers, fill the ABI structs and raise ``LLAError`` on a non-zero
-status.  All computation happens in the CUDA kernels of liblla.so; there is no fallback: if
+status.  The calls of a decode step and of a prompt are marshalled by ``_lla_native``
+(csrc/lla_binding.cpp) when their arguments are the ordinary ones, contiguous CUDA tensors and ints;
+it answers None to anything else, which the Python marshalling below takes or refuses.  All computation happens in the CUDA kernels of liblla.so; there is no fallback: if
 the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -15,7 +17,7 @@ from typing import Optional
 
 import torch
 
-from .build import LIB
+from .build import LIB, NATIVE
 
 LLA_BLOCK_TOKENS = 64
 LLA_MAX_BATCH = 1024
@@ -65,6 +67,20 @@ QUERY_FN = ctypes.CFUNCTYPE(ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
                             ctypes.c_void_p, ctypes.c_void_p)
 
 _lib = None
+_native_module = None
+
+
+def _native():
+    """The native marshalling module, loaded with the library it calls."""
+    global _native_module
+    if _native_module is None:
+        library()
+        if not os.path.exists(NATIVE):
+            raise RuntimeError(f"_lla_native.so not found at {NATIVE}: build it first "
+                               "(python -c 'import __graft_entry__ as g; g.build()')")
+        from . import _lla_native
+        _native_module = _lla_native
+    return _native_module
 
 
 def library() -> ctypes.CDLL:
@@ -152,6 +168,20 @@ def _stream(stream) -> Optional[int]:
     return stream.cuda_stream
 
 
+def _handle(stream):
+    """A stream for _lla_native: None (the current stream, looked up there) or its handle."""
+    return None if stream is None else _stream(stream)
+
+
+def _done(fn: str, status) -> bool:
+    """Whether _lla_native took the call (a status; non-zero raises) or left it (None)."""
+    if status is None:
+        return False
+    if status != 0:
+        raise LLAError(fn, status)
+    return True
+
+
 @dataclass
 class Geometry:
     T: int
@@ -220,6 +250,9 @@ def lla_cache_block_bytes(geom: Geometry) -> int:
 def lla_encode(geom: Geometry, codec: Codec, cache: Cache, x_k: torch.Tensor, x_v: torch.Tensor,
                slot_mapping: torch.Tensor, stream=None) -> None:
     """x_k, x_v [T][N][H][d] (bf16 or fp32); slot_mapping [N] int64."""
+    if _done("lla_encode", _native().encode(
+            geom, codec, cache, x_k, x_v, slot_mapping, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     N = x_k.shape[1] if x_k.dim() == 4 else 0
     _check("lla_encode", library().lla_encode(
@@ -231,6 +264,9 @@ def lla_encode_layers(geom: Geometry, codecs, caches, x_k, x_v, slot_mapping: to
                       stream=None) -> None:
     """The same encode in several layers at once: codecs, caches, x_k, x_v are per-layer lists
     (x_k[l], x_v[l] [T][N][H][d]); slot_mapping [N] int64 is shared."""
+    if _done("lla_encode_layers", _native().encode_layers(
+            geom, codecs, caches, x_k, x_v, slot_mapping, _handle(stream))):
+        return
     L = len(codecs)
     if not (len(caches) == len(x_k) == len(x_v) == L):
         raise ValueError("one codec, cache and input pair per layer")
@@ -264,6 +300,9 @@ def lla_decode_attn(geom: Geometry, codec: Codec, cache: Cache, context_lens: to
                     cur_v: Optional[torch.Tensor], out: torch.Tensor, workspace: torch.Tensor,
                     stream=None) -> None:
     """q, cur_k, cur_v, out [B][H][d]; cur_k = cur_v = None selects pass 2."""
+    if _done("lla_decode_attn", _native().decode_attn(
+            geom, codec, cache, context_lens, max_ctx, loop, q, cur_k, cur_v, out, workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     B = q.shape[0]
     _check("lla_decode_attn", library().lla_decode_attn(
@@ -279,6 +318,10 @@ def lla_decode_attn_rope(geom: Geometry, codec: Codec, cache: Cache, rope_base: 
                          workspace: torch.Tensor, stream=None) -> None:
     """lla_decode_attn with RoPE after reconstruction; q and cur_k pre-RoPE.  rope_pairing:
     LLA_ROPE_HALF (pairs (j, j + d/2)) or LLA_ROPE_ADJACENT (pairs (2j, 2j + 1))."""
+    if _done("lla_decode_attn_rope", _native().decode_attn_rope(
+            geom, codec, cache, rope_base, rope_pairing, context_lens, max_ctx, loop, q, cur_k, cur_v, out,
+            workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     rp = lla_rope(float(rope_base), int(rope_pairing))
     _check("lla_decode_attn_rope", library().lla_decode_attn_rope(
@@ -301,6 +344,9 @@ def lla_decode_attn_loops(geom: Geometry, codec: Codec, cache: Cache, context_le
                           cur_v: Optional[torch.Tensor], out: torch.Tensor,
                           workspace: torch.Tensor, stream=None) -> None:
     """All T loops' decode calls in one pass over the latents: q, cur_k, cur_v, out [T][B][H][d]."""
+    if _done("lla_decode_attn_loops", _native().decode_attn_loops(
+            geom, codec, cache, context_lens, max_ctx, q, cur_k, cur_v, out, workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     _check("lla_decode_attn_loops", library().lla_decode_attn_loops(
         ctypes.byref(g), ctypes.byref(cd), ctypes.byref(ch), _ptr(context_lens), q.shape[1],
@@ -326,6 +372,9 @@ def lla_prefill_attn(geom: Geometry, codec: Codec, cache: Cache, cu_seqlens: tor
                      max_len: int, loop: int, q: torch.Tensor, out: torch.Tensor,
                      stream=None) -> None:
     """q, out [Ntok][H][d]; cu_seqlens [B+1] int32."""
+    if _done("lla_prefill_attn", _native().prefill_attn(
+            geom, codec, cache, cu_seqlens, max_len, loop, q, out, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     B = cu_seqlens.shape[0] - 1
     _check("lla_prefill_attn", library().lla_prefill_attn(
@@ -346,6 +395,9 @@ def lla_prefill_attn_rope(geom: Geometry, codec: Codec, cache: Cache, rope_base:
                           q: torch.Tensor, out: torch.Tensor, workspace: torch.Tensor,
                           stream=None) -> None:
     """lla_prefill_attn with RoPE after reconstruction; q pre-RoPE [Ntok][H][d]."""
+    if _done("lla_prefill_attn_rope", _native().prefill_attn_rope(
+            geom, codec, cache, rope_base, rope_pairing, cu_seqlens, max_len, loop, q, out, workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     rp = lla_rope(float(rope_base), int(rope_pairing))
     B = cu_seqlens.shape[0] - 1
@@ -421,6 +473,9 @@ def lla_encode_2d(geom: Geometry, codec: Codec, cache: Cache, x_k: torch.Tensor,
                   x_v: torch.Tensor, slot_mapping: torch.Tensor, stream=None) -> None:
     """LLA-2D encode.  x_k, x_v [T][N][H][d]; codec w_down_* [T*H*d][r], mu_* [T*H*d];
     cache with one page per block."""
+    if _done("lla_encode_2d", _native().encode_2d(
+            geom, codec, cache, x_k, x_v, slot_mapping, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     N = x_k.shape[1] if x_k.dim() == 4 else 0
     _check("lla_encode_2d", library().lla_encode_2d(
@@ -441,6 +496,9 @@ def lla_decode_attn_2d(geom: Geometry, codec: Codec, cache: Cache, context_lens:
                        cur_v: Optional[torch.Tensor], out: torch.Tensor, workspace: torch.Tensor,
                        stream=None) -> None:
     """LLA-2D decode call; codec w_up_* [T][H][d][r]; q, cur_k, cur_v, out [B][H][d]."""
+    if _done("lla_decode_attn_2d", _native().decode_attn_2d(
+            geom, codec, cache, context_lens, max_ctx, loop, q, cur_k, cur_v, out, workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     _check("lla_decode_attn_2d", library().lla_decode_attn_2d(
         ctypes.byref(g), ctypes.byref(cd), ctypes.byref(ch), _ptr(context_lens), q.shape[0],
@@ -481,6 +539,10 @@ def lla_decode_attn_decoupled(geom: Geometry, codec: Codec, cache: Cache, rope_p
                               out: torch.Tensor, workspace: torch.Tensor, stream=None) -> None:
     """Per-head LLA decode with the decoupled rotary branch; q, cur_k, cur_v, out [B][H][d],
     q_rope [B][H][d_rope], cur_k_rope [B][d_rope] (pass 1) or None."""
+    if _done("lla_decode_attn_decoupled", _native().decode_attn_decoupled(
+            geom, codec, cache, rope_pool, d_rope, rope_base, rope_pairing, context_lens, max_ctx, loop, q, q_rope,
+            cur_k, cur_v, cur_k_rope, out, workspace, _handle(stream))):
+        return
     g, cd, ch = geom.c(), codec.c(), cache.c()
     rp = lla_rope(float(rope_base), int(rope_pairing))
     _check("lla_decode_attn_decoupled", library().lla_decode_attn_decoupled(

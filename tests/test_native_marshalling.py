@@ -1,0 +1,55 @@
+"""The native marshalling of the binding (csrc/lla_binding.cpp) takes only ordinary calls: to anything
+else it answers None, and the Python marshalling accepts or refuses the call as without it (no GPU)."""
+import inspect
+
+import pytest
+import torch
+
+from helpers import ensure_library
+
+FAKE = 0x10000
+
+
+@pytest.fixture(scope="module")
+def lla():
+    ensure_library()
+    from paper_2607_15456_gb300 import lla as m
+    return m
+
+
+def _args(lla, name, x):
+    """The native function's arguments for a call of lla.<name> with x in every tensor's place."""
+    geom, cache = lla.Geometry(4, 2, 128, 96, 160), lla.Cache(x, 4, x, 2)
+    cd = lla.Codec(x, x, x, x)
+    scalar = {"geom": geom, "codec": cd, "cache": cache, "codecs": [cd], "caches": [cache], "max_ctx": 64, "max_len": 64,
+              "loop": 0, "rope_base": 10000.0, "rope_pairing": 0, "d_rope": 64, "stream": 0}
+    names = list(inspect.signature(getattr(lla, "lla_" + name)).parameters)
+    return [scalar[n] if n in scalar else ([x] if name == "encode_layers" and n in ("x_k", "x_v") else x) for n in names]
+
+
+NAMES = ["encode", "encode_2d", "encode_layers", "decode_attn", "decode_attn_2d", "decode_attn_loops", "decode_attn_rope",
+         "decode_attn_decoupled", "prefill_attn", "prefill_attn_rope"]
+
+
+@pytest.mark.parametrize("name", NAMES)
+@pytest.mark.parametrize("what", ["host tensor", "address", "other object", "subclass"])
+def test_unusual_arguments_are_left_to_python(lla, name, what):
+    x = {"host tensor": torch.zeros(4, 4, 2, 128), "address": FAKE, "other object": "x",
+         "subclass": torch.nn.Parameter(torch.zeros(4, 4, 2, 128))}[what]
+    assert getattr(lla._native(), name)(*_args(lla, name, x)) is None
+    if what in ("host tensor", "subclass"):
+        with pytest.raises(ValueError, match="CUDA tensors"):
+            getattr(lla, "lla_" + name)(*_args(lla, name, x))
+
+
+@pytest.mark.parametrize("name", NAMES)
+def test_wrong_number_of_arguments(lla, name):
+    with pytest.raises(TypeError):
+        getattr(lla._native(), name)(None)
+
+
+@pytest.mark.parametrize("field,value", [("T", 2 ** 40), ("d", "128"), ("scale", 1), ("storage", 3)])
+def test_unusual_geometry_is_left_to_python(lla, field, value):
+    args = _args(lla, "decode_attn", None)
+    setattr(args[0], field, value)
+    assert lla._native().decode_attn(*args) is None

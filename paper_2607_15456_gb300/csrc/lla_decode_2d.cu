@@ -86,6 +86,10 @@ struct Z2 {
     static constexpr int QS = NQ == 4 ? 3 : 2;
     static constexpr int PSPL = NQ == 4 ? 3 : 1;
     static constexpr int NS = (QS * NQ + 7) / 8 * 8;    // score MMA N: the q~ parts, padded
+    // products issued by a converged warp (descriptors in uniform registers) for the loops; by one thread
+    // for LLA-2D pages, whose stream is bound by HBM and ran 2 % slower beside the faster issue (632 and
+    // 645 us on the 128-sequence batch at (288, 480))
+    static constexpr bool WARP = NQ == 4;
     static constexpr int NQM = NQ;                      // queries of a unit in the workspace
     static constexpr int NCH = (RV + 127) / 128;        // 128-row chunks of O^T
     static constexpr int NBOX = (RV + 63) / 64;         // TMA boxes a V-plane loads
@@ -107,9 +111,10 @@ struct Z2 {
     static constexpr int oP = oQ + QB;
     static constexpr int oRed = oP + 2 * PBUF;
     static constexpr int oBar = oRed + RED;
-    static constexpr int SMEM = 1024 + oBar + NBAR * 8;
+    // (at least half of an SM's: one CTA per SM, which holds all of TMEM)
+    static constexpr int SMEM0 = 1024 + oBar + NBAR * 8, SMEM = SMEM0 > 116 * 1024 ? SMEM0 : 116 * 1024;
     // TMEM columns: S^T double buffer [0, 2 NS), O^T chunks [2 NS, 2 NS + 16 NCH)
-    static constexpr uint32_t TM_S = 0, TM_O = 2 * NS, TM_COLS = 128;
+    static constexpr uint32_t TM_S = 0, TM_O = 2 * NS, TM_COLS = 512;
     static constexpr uint32_t IDESC_S = umma_idesc_bf16(64, NS, 0, 0);
     static constexpr uint32_t IDESC_O = umma_idesc_bf16(128, kNQ, 1, 0);
     // a run partial: O^T of each query ([NQM][RV]), then 16 maxima and 16 sums
@@ -158,11 +163,10 @@ struct T2Params {
     const char *pool;
     int64_t num_blocks, page_bytes;
     const int32_t *block_table;
-    int max_blocks;
+    int max_blocks, max_ctx;
     const int32_t *context_lens;
     const float *qt;
     const float *beta;
-    const int *pstart;
     float *part;  // [U + grid][PSTRIDE]: run (unit u, CTA c) at slot u + c
     unsigned *err;
 };
@@ -246,6 +250,7 @@ __global__ void __launch_bounds__(256) absorb2d_kernel(const A2Params p) {
 #pragma unroll
     for (int u = 0; u < 16; ++u) wv[u] = col < RK ? bf_to_f(W[(warp * 16 + u) * RK]) : 0.f;
     pdl_wait();  // the queries may come from the previous kernel; the workspace is free after it
+    pdl_trigger();
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) page_prefix(p);
     for (int i = tid; i < 16 * kD; i += 256) {
         const int bi = i >> 7, e = i & (kD - 1);
@@ -287,16 +292,83 @@ __global__ void __launch_bounds__(256) absorb2d_kernel(const A2Params p) {
 
 // ------------------------------------------------------------------------- attention kernel
 
-// First unit with pages at or after global page g0: the last u with pstart[u] <= g0.
-__device__ __forceinline__ int first_unit(const int *pstart, int U, int g0) {
-    int lo = 0, hi = U - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pstart[mid] <= g0) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+// Pages of unit u: none where the length is out of range (the absorb kernel's prefix counts alike).
+__device__ __forceinline__ int unit_pages(const T2Params &p, int u) {
+    const int L = p.context_lens[u / p.hu];
+    return L < 0 || L > min(p.max_ctx, p.max_blocks * kPT) ? 0 : (L + kPT - 1) / kPT;
 }
+
+// A CTA's share of the global pages, and its first unit with that unit's first page: worked out from
+// the context lengths, which are inputs of the call, by all threads of the CTA, so that the producer
+// can start on the pages while the absorb kernel still runs.  (A search of the prefix sums that the
+// absorb kernel leaves took log2(units) dependent loads after the wait for it.)
+struct Share {
+    int g0, g1, u, s;
+};
+template <int THREADS>
+__device__ Share find_share(const T2Params &p, int G, int c) {
+    __shared__ int wsum[THREADS / 32], first[2];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int B = p.U / p.hu, per = (B + THREADS - 1) / THREADS;
+    int tot = 0;
+    for (int b = tid * per; b < min(B, (tid + 1) * per); ++b) tot += unit_pages(p, b * p.hu) * p.hu;
+    int x = tot;  // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    int pre = 0, np = 0;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) {
+        if (w < warp) pre += wsum[w];
+        np += wsum[w];
+    }
+    // with fewer pages than CTAs the first np CTAs take one each
+    const int Ge = min(G, np);
+    Share r;
+    r.g0 = c < Ge ? page_lo(c, np, Ge) : 0;
+    r.g1 = c < Ge ? page_lo(c + 1, np, Ge) : 0;
+    if (r.g0 < r.g1) {
+        int ex = pre + x - tot;  // first page of this thread's sequences
+        for (int b = tid * per; b < min(B, (tid + 1) * per); ++b) {
+            const int n = unit_pages(p, b * p.hu);
+            if (ex <= r.g0 && r.g0 < ex + n * p.hu) {
+                const int k = (r.g0 - ex) / n;
+                first[0] = b * p.hu + k;
+                first[1] = ex + k * n;
+            }
+            ex += n * p.hu;
+        }
+    }
+    __syncthreads();
+    r.u = r.g0 < r.g1 ? first[0] : p.U;
+    r.s = r.g0 < r.g1 ? first[1] : 0;
+    return r;
+}
+
+// Products issued by a converged warp (WARP) or by one thread.
+template <bool WARP>
+struct Issue {
+    static __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool acc) {
+        if constexpr (WARP) umma_bf16_warp(d, a, b, idesc, acc);
+        else umma_bf16(d, a, b, idesc, acc);
+    }
+    static __device__ __forceinline__ void commit(uint64_t *bar) {
+        if constexpr (WARP) umma_commit_warp(bar);
+        else umma_commit(bar);
+    }
+    static __device__ __forceinline__ bool wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag, unsigned *err) {
+        if constexpr (WARP) return mbar_wait_warp(bar, parity, abort_flag, err);
+        else return mbar_wait(bar, parity, abort_flag, err);
+    }
+    static __device__ __forceinline__ int uniform(int v) {
+        if constexpr (WARP) return __shfl_sync(0xffffffffu, v, 0);
+        else return v;
+    }
+};
 
 template <int N>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[N]) {
@@ -328,7 +400,7 @@ __global__ void __launch_bounds__(kT2, 1)
     float *red = reinterpret_cast<float *>(sm + Z::oRed);  // [2 pages][4 warps][16] maxima
     float *lsum = red + 128;                                // [4 warps][16] run sums
     float *betas = lsum + 64;                               // [16]
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int G = gridDim.x, c = blockIdx.x;
 
     if (tid == 0) {
@@ -376,12 +448,13 @@ __global__ void __launch_bounds__(kT2, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
-    pdl_wait();  // q~, beta and the page prefix sums come from the absorb kernel
-
-    const int NP = p.pstart[p.U];
-    const int g0 = page_lo(c, NP, G), g1 = page_lo(c + 1, NP, G);
-    const int ufirst = g0 < g1 ? first_unit(p.pstart, p.U, g0) : p.U;
+    constexpr uint32_t tmem = 0;  // the whole of TMEM is allocated (one CTA per SM)
+    const Share sh = find_share<kT2>(p, G, c);
+    const int g0 = sh.g0, g1 = sh.g1;
+    // q~ and beta come from the absorb kernel, and the workspace is free once it has waited for the
+    // kernel before it; the producer reads only inputs of the call, which that kernel's wait ordered
+    // before this launch, and waits at its end
+    if (warp != 0) pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------------------- producer
@@ -392,8 +465,8 @@ __global__ void __launch_bounds__(kT2, 1)
             const uint64_t pol = policy_evict_first();
             int itk = 0, itv = 0;
             bool stop = false;
-            for (int u = ufirst; u < p.U && !stop; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U && !stop; ++u, s0 = s1) {
+                s1 = s0 + unit_pages(p, u);
                 if (s0 >= g1) break;
                 const int pa = max(g0, s0) - s0, pe = min(g1, s1) - s0;
                 const int b = u / p.hu, hh = u - b * p.hu;
@@ -436,35 +509,35 @@ __global__ void __launch_bounds__(kT2, 1)
                 mbar_wait(&bar[bVfull + j % Z::ST], (j / Z::ST) & 1, &never, p.err);
         }
         __syncwarp();
+        pdl_wait();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- S^T issuer
-        // (an MMA takes its issuing thread tens of cycles: the score and value products of a
-        // page are issued by two threads, each committing only its own products)
-        if (lane == 0) {
+        // (the score and value products of a page are issued by two warps, each committing only its own)
+        if (Z::WARP || lane == 0) {
             const uint32_t base = smem_addr(sm);
             const uint64_t dq = umma_desc(base + Z::oQ, Z::NS * 16, 128);
             const uint64_t dk0 = umma_desc(base + Z::oK, kPT * 16, 128);
             int it = 0, r = 0;
-            for (int u = ufirst; u < p.U; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+                s1 = s0 + Issue<Z::WARP>::uniform(unit_pages(p, u));
                 if (s0 >= g1) break;
                 const int n = min(g1, s1) - max(g0, s0);
                 if (n <= 0) continue;
-                mbar_wait(&bar[bQready], r & 1, abort_flag, p.err);
+                Issue<Z::WARP>::wait(&bar[bQready], r & 1, abort_flag, p.err);
                 tc_fence_after();
                 for (int k = 0; k < n; ++k, ++it) {
                     const int s = it & 1, st = it % Z::ST;
-                    mbar_wait(&bar[bKfull + st], (it / Z::ST) & 1, abort_flag, p.err);
-                    if (it >= 2) mbar_wait(&bar[bSfree + s], ((it - 2) >> 1) & 1, abort_flag, p.err);
+                    Issue<Z::WARP>::wait(&bar[bKfull + st], (it / Z::ST) & 1, abort_flag, p.err);
+                    if (it >= 2) Issue<Z::WARP>::wait(&bar[bSfree + s], ((it - 2) >> 1) & 1, abort_flag, p.err);
                     tc_fence_after();
                     const uint64_t dk = dk0 + static_cast<uint64_t>((st * Z::KPAGE) >> 4);
 #pragma unroll
                     for (int ks = 0; ks < Z::RKX / 16; ++ks)
-                        umma_bf16(tmem + Z::TM_S + s * Z::NS, dk + ks * ((2 * kPT * 16) >> 4),
+                        Issue<Z::WARP>::mma(tmem + Z::TM_S + s * Z::NS, dk + ks * ((2 * kPT * 16) >> 4),
                                   dq + ks * ((2 * Z::NS * 16) >> 4), Z::IDESC_S, ks > 0);
-                    umma_commit(&bar[bSfull + s]);
-                    umma_commit(&bar[bKempty + st]);
-                    if (k == n - 1) umma_commit(&bar[bQfree]);
+                    Issue<Z::WARP>::commit(&bar[bSfull + s]);
+                    Issue<Z::WARP>::commit(&bar[bKempty + st]);
+                    if (k == n - 1) Issue<Z::WARP>::commit(&bar[bQfree]);
                 }
                 ++r;
             }
@@ -472,18 +545,18 @@ __global__ void __launch_bounds__(kT2, 1)
             // softmax warps stop waiting for them): the last commit on each S^T buffer
             volatile int never = 0;
             for (int j = max(0, it - 2); j < it; ++j)
-                mbar_wait(&bar[bSfull + (j & 1)], (j >> 1) & 1, &never, p.err);
+                Issue<Z::WARP>::wait(&bar[bSfull + (j & 1)], (j >> 1) & 1, &never, p.err);
         }
         __syncwarp();
     } else if (warp == kPvWarp) {
         // ---------------------------------------------------------------- O^T issuer
-        if (lane == 0) {
+        if (Z::WARP || lane == 0) {
             const uint32_t base = smem_addr(sm);
             const uint64_t dp0 = umma_desc(base + Z::oP, kNQ * 16, 128);
             const uint64_t dv0 = umma_desc_sw128_mn(base + Z::oV, Z::BOX);
             int it = 0, r = 0;
-            for (int u = ufirst; u < p.U; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+                s1 = s0 + Issue<Z::WARP>::uniform(unit_pages(p, u));
                 if (s0 >= g1) break;
                 const int n = min(g1, s1) - max(g0, s0);
                 if (n <= 0) continue;
@@ -491,9 +564,9 @@ __global__ void __launch_bounds__(kT2, 1)
                     // O^T += C_v^T P^T for page it (the first page of run r zeroes O^T, once the
                     // softmax warps have read run r - 1's)
                     const int s = it & 1, st = it % Z::ST;
-                    mbar_wait(&bar[bPfull + s], (it >> 1) & 1, abort_flag, p.err);
-                    mbar_wait(&bar[bVfull + st], (it / Z::ST) & 1, abort_flag, p.err);
-                    if (k == 0 && r > 0) mbar_wait(&bar[bOfree], (r - 1) & 1, abort_flag, p.err);
+                    Issue<Z::WARP>::wait(&bar[bPfull + s], (it >> 1) & 1, abort_flag, p.err);
+                    Issue<Z::WARP>::wait(&bar[bVfull + st], (it / Z::ST) & 1, abort_flag, p.err);
+                    if (k == 0 && r > 0) Issue<Z::WARP>::wait(&bar[bOfree], (r - 1) & 1, abort_flag, p.err);
                     tc_fence_after();
                     const uint64_t dv = dv0 + static_cast<uint64_t>((st * Z::VPAGE) >> 4);
                     const uint64_t dp = dp0 + static_cast<uint64_t>((s * Z::PBUF) >> 4);
@@ -501,10 +574,10 @@ __global__ void __launch_bounds__(kT2, 1)
                     for (int ch = 0; ch < Z::NCH; ++ch)
 #pragma unroll
                         for (int ks = 0; ks < kPT / 16; ++ks)
-                            umma_bf16(tmem + Z::TM_O + ch * kNQ, dv + ((ch * 2 * Z::BOX + ks * 2048) >> 4),
+                            Issue<Z::WARP>::mma(tmem + Z::TM_O + ch * kNQ, dv + ((ch * 2 * Z::BOX + ks * 2048) >> 4),
                                       dp + ks * ((2 * kNQ * 16) >> 4), Z::IDESC_O, k > 0 || ks > 0);
-                    umma_commit(&bar[bVempty + st]);
-                    umma_commit(&bar[bPfree + s]);  // also: O^T holds pages up to it
+                    Issue<Z::WARP>::commit(&bar[bVempty + st]);
+                    Issue<Z::WARP>::commit(&bar[bPfree + s]);  // also: O^T holds pages up to it
                 }
                 ++r;
             }
@@ -513,7 +586,7 @@ __global__ void __launch_bounds__(kT2, 1)
             // completed before the softmax released the last page)
             if (it > 0) {
                 volatile int never = 0;
-                mbar_wait(&bar[bPfree + ((it - 1) & 1)], ((it - 1) >> 1) & 1, &never, p.err);
+                Issue<Z::WARP>::wait(&bar[bPfree + ((it - 1) & 1)], ((it - 1) >> 1) & 1, &never, p.err);
             }
         }
         __syncwarp();
@@ -524,8 +597,8 @@ __global__ void __launch_bounds__(kT2, 1)
         const int st_tid = tid - kSm0;
         const int tok = 16 * q4 + lane;  // the token of this lane in the M = 64 layout (lane < 16)
         int it = 0, r = 0;
-        for (int u = ufirst; u < p.U; ++u) {
-            const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+        for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+            s1 = s0 + unit_pages(p, u);
             if (s0 >= g1) break;
             const int pa = max(g0, s0) - s0, pe = min(g1, s1) - s0;
             if (pe <= pa) continue;
@@ -797,7 +870,7 @@ __global__ void __launch_bounds__(256, 1)
     float *red = reinterpret_cast<float *>(sm + Z::oRed);  // [2 pages][4 warps][16] maxima
     float *lsum = red + 128;                                // [4 warps][16] run sums
     float *betas = lsum + 64;                               // [16]
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int G = gridDim.x, c = blockIdx.x;
 
     if (tid == 0) {
@@ -826,12 +899,10 @@ __global__ void __launch_bounds__(256, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
-    pdl_wait();  // q~, beta and the page prefix sums come from the absorb kernel
-
-    const int NP = p.pstart[p.U];
-    const int g0 = page_lo(c, NP, G), g1 = page_lo(c + 1, NP, G);
-    const int ufirst = g0 < g1 ? first_unit(p.pstart, p.U, g0) : p.U;
+    constexpr uint32_t tmem = 0;  // the whole of TMEM is allocated (one CTA per SM)
+    const Share sh = find_share<256>(p, G, c);
+    const int g0 = sh.g0, g1 = sh.g1;
+    if (warp != 0 && warp != 7) pdl_wait();  // as in attn2d_kernel; the producers wait at their ends
 
     if (warp == 0) {
         // ----------------------------------------------------------------------- K producer
@@ -839,8 +910,8 @@ __global__ void __launch_bounds__(256, 1)
             const uint64_t pol = policy_evict_first();
             int itk = 0;
             bool stop = false;
-            for (int u = ufirst; u < p.U && !stop; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U && !stop; ++u, s0 = s1) {
+                s1 = s0 + unit_pages(p, u);
                 if (s0 >= g1) break;
                 const int pa = max(g0, s0) - s0, pe = min(g1, s1) - s0;
                 const int32_t *bt = p.block_table + static_cast<int64_t>(u) * p.max_blocks;
@@ -868,6 +939,7 @@ __global__ void __launch_bounds__(256, 1)
                 mbar_wait(&bar[cKfull + j % Z::KST], (j / Z::KST) & 1, &never, p.err);
         }
         __syncwarp();
+        pdl_wait();
     } else if (warp == 7) {
         // ---------------------------------------------------------- V producer and hand-over
         int itv = 0, handed = 0;
@@ -896,8 +968,8 @@ __global__ void __launch_bounds__(256, 1)
             if (lane == 0) mbar_arrive(&bar[cVok + st]);
         };
         bool stop = false;
-        for (int u = ufirst; u < p.U && !stop; ++u) {
-            const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+        for (int u = sh.u, s0 = sh.s, s1; u < p.U && !stop; ++u, s0 = s1) {
+            s1 = s0 + unit_pages(p, u);
             if (s0 >= g1) break;
             const int pa = max(g0, s0) - s0, pe = min(g1, s1) - s0;
             const int L = p.context_lens[u];
@@ -931,36 +1003,37 @@ __global__ void __launch_bounds__(256, 1)
             }
         }
         while (handed < itv) hand_over(handed++);  // also drains every copy after an abort
+        pdl_wait();
     } else if (warp == 1) {
         // ----------------------------------------------------------------------- S^T issuer
-        if (lane == 0) {
+        {
             const uint32_t base = smem_addr(sm);
             const uint64_t dq = umma_desc(base + Z::oQ, Z::NS * 16, 128);
             int it = 0, itk = 0, r = 0;
-            for (int u = ufirst; u < p.U; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+                s1 = s0 + __shfl_sync(0xffffffffu, unit_pages(p, u), 0);
                 if (s0 >= g1) break;
                 const int n = min(g1, s1) - max(g0, s0);
                 if (n <= 0) continue;
-                mbar_wait(&bar[cQready], r & 1, abort_flag, p.err);
+                mbar_wait_warp(&bar[cQready], r & 1, abort_flag, p.err);
                 tc_fence_after();
                 for (int k = 0; k < n; ++k, ++it) {
                     const int s = it & 1;
-                    if (it >= 2) mbar_wait(&bar[cSfree + s], ((it - 2) >> 1) & 1, abort_flag, p.err);
+                    if (it >= 2) mbar_wait_warp(&bar[cSfree + s], ((it - 2) >> 1) & 1, abort_flag, p.err);
                     for (int kc = 0; kc < Z::KC; ++kc, ++itk) {
                         const int st = itk % Z::KST;
-                        mbar_wait(&bar[cKfull + st], (itk / Z::KST) & 1, abort_flag, p.err);
+                        mbar_wait_warp(&bar[cKfull + st], (itk / Z::KST) & 1, abort_flag, p.err);
                         tc_fence_after();
                         const uint64_t dk = umma_desc(base + Z::oK + st * Z::KCB, kPT * 16, 128);
 #pragma unroll 6
                         for (int ks = 0; ks < Z::RKC / 16; ++ks)
-                            umma_bf16(tmem + Z::TM_S + s * Z::NS, dk + ks * ((2 * kPT * 16) >> 4),
+                            umma_bf16_warp(tmem + Z::TM_S + s * Z::NS, dk + ks * ((2 * kPT * 16) >> 4),
                                       dq + (kc * (Z::RKC / 8) + 2 * ks) * ((Z::NS * 16) >> 4), Z::IDESC_S,
                                       kc > 0 || ks > 0);
-                        umma_commit(&bar[cKempty + st]);
+                        umma_commit_warp(&bar[cKempty + st]);
                     }
-                    umma_commit(&bar[cSfull + s]);
-                    if (k == n - 1) umma_commit(&bar[cQfree]);
+                    umma_commit_warp(&bar[cSfull + s]);
+                    if (k == n - 1) umma_commit_warp(&bar[cQfree]);
                 }
                 ++r;
             }
@@ -968,43 +1041,43 @@ __global__ void __launch_bounds__(256, 1)
             // commit on each S^T buffer
             volatile int never = 0;
             for (int j = max(0, it - 2); j < it; ++j)
-                mbar_wait(&bar[cSfull + (j & 1)], (j >> 1) & 1, &never, p.err);
+                mbar_wait_warp(&bar[cSfull + (j & 1)], (j >> 1) & 1, &never, p.err);
         }
         __syncwarp();
     } else if (warp == 6) {
         // ----------------------------------------------------------------------- O^T issuer
-        if (lane == 0) {
+        {
             const uint32_t base = smem_addr(sm);
             const uint64_t dp0 = umma_desc(base + Z::oP, kNQ * 16, 128);
             int it = 0, itv = 0, r = 0;
-            for (int u = ufirst; u < p.U; ++u) {
-                const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+            for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+                s1 = s0 + __shfl_sync(0xffffffffu, unit_pages(p, u), 0);
                 if (s0 >= g1) break;
                 const int n = min(g1, s1) - max(g0, s0);
                 if (n <= 0) continue;
                 for (int k = 0; k < n; ++k, ++it) {
                     const int s = it & 1;
-                    mbar_wait(&bar[cPfull + s], (it >> 1) & 1, abort_flag, p.err);
-                    if (k == 0 && r > 0) mbar_wait(&bar[cOfree], (r - 1) & 1, abort_flag, p.err);
+                    mbar_wait_warp(&bar[cPfull + s], (it >> 1) & 1, abort_flag, p.err);
+                    if (k == 0 && r > 0) mbar_wait_warp(&bar[cOfree], (r - 1) & 1, abort_flag, p.err);
                     const uint64_t dp = dp0 + static_cast<uint64_t>((s * Z::PBUF) >> 4);
                     for (int vc = 0; vc < Z::VC; ++vc, ++itv) {
                         const int st = itv % Z::VST;
-                        mbar_wait(&bar[cVok + st], (itv / Z::VST) & 1, abort_flag, p.err);
+                        mbar_wait_warp(&bar[cVok + st], (itv / Z::VST) & 1, abort_flag, p.err);
                         tc_fence_after();
                         const uint64_t dv = umma_desc_sw128_mn(base + Z::oV + st * Z::VCB, Z::BOX);
 #pragma unroll
                         for (int ks = 0; ks < kPT / 16; ++ks)
-                            umma_bf16(tmem + Z::TM_O + vc * kNQ, dv + ((ks * 2048) >> 4),
+                            umma_bf16_warp(tmem + Z::TM_O + vc * kNQ, dv + ((ks * 2048) >> 4),
                                       dp + ks * ((2 * kNQ * 16) >> 4), Z::IDESC_O, k > 0 || ks > 0);
-                        umma_commit(&bar[cVempty + st]);
+                        umma_commit_warp(&bar[cVempty + st]);
                     }
-                    umma_commit(&bar[cPfree + s]);  // also: O^T holds pages up to it
+                    umma_commit_warp(&bar[cPfree + s]);  // also: O^T holds pages up to it
                 }
                 ++r;
             }
             if (it > 0) {
                 volatile int never = 0;
-                mbar_wait(&bar[cPfree + ((it - 1) & 1)], ((it - 1) >> 1) & 1, &never, p.err);
+                mbar_wait_warp(&bar[cPfree + ((it - 1) & 1)], ((it - 1) >> 1) & 1, &never, p.err);
             }
         }
         __syncwarp();
@@ -1015,8 +1088,8 @@ __global__ void __launch_bounds__(256, 1)
         const int st_tid = tid - kSm0;
         const int tok = 16 * q4 + lane;
         int it = 0, r = 0;
-        for (int u = ufirst; u < p.U; ++u) {
-            const int s0 = p.pstart[u], s1 = p.pstart[u + 1];
+        for (int u = sh.u, s0 = sh.s, s1; u < p.U; ++u, s0 = s1) {
+            s1 = s0 + unit_pages(p, u);
             if (s0 >= g1) break;
             const int pa = max(g0, s0) - s0, pe = min(g1, s1) - s0;
             if (pe <= pa) continue;
@@ -1236,7 +1309,7 @@ __global__ void __launch_bounds__(128, 1) finish2d_kernel(const F2Params p) {
     }
     __syncthreads();
     pdl_wait();
-    const int NP = p.pstart[p.U];
+    const int NP = p.pstart[p.U], Ge = min(p.grid, NP);  // the split of find_share
     // G warps per unit (all four for one unit, two each for two): warp `sub` of a group takes
     // the columns j = lane + 32 (sub + G q)
     const int G = nb == 1 ? 4 : nb == 2 ? 2 : 1;
@@ -1258,17 +1331,17 @@ __global__ void __launch_bounds__(128, 1) finish2d_kernel(const F2Params p) {
 #pragma unroll
         for (int q = 0; q < NJ; ++q) acc[q] = 0.f;
         if (s1 > s0) {
-            // the runs of unit u: the CTAs c0 .. c1 that hold pages (a CTA between them may hold
-            // none and writes nothing), partials at slots u + c
-            const int c0 = cta_of(s0, NP, p.grid), c1 = cta_of(s1 - 1, NP, p.grid);
+            // the runs of unit u: the CTAs c0 .. c1, each of which holds pages of it, partials at slots
+            // u + c.  (Split over all CTAs whatever the pages, one sequence of 13 pages spread over 140
+            // CTAs' slots, 128 of them empty, and its merge took 37 us instead of 8.)
+            const int c0 = cta_of(s0, NP, Ge), c1 = cta_of(s1 - 1, NP, Ge);
             const int nr = c1 - c0 + 1;
             const float *pu = p.part + static_cast<int64_t>(u + c0) * PS;
             // the run maxima and sums in one round of loads
             float mm = -INFINITY;
             for (int i = lane; i < nr; i += 32) {
-                const bool has = page_lo(c0 + i + 1, NP, p.grid) > page_lo(c0 + i, NP, p.grid);
-                wt[i] = has ? pu[static_cast<int64_t>(i) * PS + PO_M + qn] : -INFINITY;
-                wl[i] = has ? pu[static_cast<int64_t>(i) * PS + PO_L + qn] : 0.f;
+                wt[i] = pu[static_cast<int64_t>(i) * PS + PO_M + qn];
+                wl[i] = pu[static_cast<int64_t>(i) * PS + PO_L + qn];
                 mm = fmaxf(mm, wt[i]);
             }
             M = warp_max(mm);
@@ -1280,9 +1353,7 @@ __global__ void __launch_bounds__(128, 1) finish2d_kernel(const F2Params p) {
             }
             l = warp_sum(ls);
             __syncwarp();
-            // the column loads of KR runs in flight at once, then their sums: a slot between the
-            // unit's first and last CTA that holds no run (weight 0) is read, inside the
-            // workspace, but its values are never used
+            // the column loads of KR runs in flight at once, then their sums
             for (int i0 = 0; i0 < nr; i0 += KR) {
                 float v[KR][NJ];
 #pragma unroll
@@ -1442,7 +1513,7 @@ lla_status launch_units(const DecodeArgs &a, bool loops, cudaStream_t stream) {
     tp.num_blocks = a.num_blocks; tp.page_bytes = page_bytes;
     tp.block_table = a.block_table; tp.max_blocks = a.max_blocks;
     tp.context_lens = a.context_lens;
-    tp.qt = ap.qt; tp.beta = ap.beta; tp.pstart = ap.pstart;
+    tp.qt = ap.qt; tp.beta = ap.beta; tp.max_ctx = a.max_ctx;
     tp.part = reinterpret_cast<float *>(ws + w.part);
     tp.err = err;
     if ((st = launch_ex(attn2d_kernel<RK, RV, NQ>, dim3(grid), kT2, Z::SMEM, stream, tv, tp)) != LLA_OK)
@@ -1600,7 +1671,7 @@ lla_status launch_big(const DecodeArgs &a, cudaStream_t stream) {
     tp.num_blocks = a.num_blocks; tp.page_bytes = page_bytes;
     tp.block_table = a.block_table; tp.max_blocks = a.max_blocks;
     tp.context_lens = a.context_lens;
-    tp.qt = ap.qt; tp.beta = ap.beta; tp.pstart = ap.pstart;
+    tp.qt = ap.qt; tp.beta = ap.beta; tp.max_ctx = a.max_ctx;
     tp.part = reinterpret_cast<float *>(ws + w.part);
     tp.err = err;
     if ((st = launch_ex(attn2d_big_kernel<RK, RV>, dim3(grid), 256, Z::SMEM, stream, tv, tp)) != LLA_OK)

@@ -285,8 +285,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = *tslot;
     pdl_wait();  // inputs may come from the previous kernel; the workspace is free after it
     seq_prefix(p.context_lens, p.B, p.max_ctx, p.max_blocks, p.pass1, c == 0, p.err, PB);
-    const int NP = p.H * PB[p.B];
-    const int g0 = page_lo(c, NP, G), g1 = page_lo(c + 1, NP, G);
+    // with fewer pages than CTAs the first NP CTAs take one each
+    const int NP = p.H * PB[p.B], Ge = min(G, NP);
+    const int g0 = c < Ge ? page_lo(c, NP, Ge) : 0, g1 = c < Ge ? page_lo(c + 1, NP, Ge) : 0;
     Runs runs(PB, p.H, p.B, g0, g1);
     int rb, rh, pa, pe;
 
@@ -711,7 +712,7 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
     }
     __syncthreads();
     pdl_wait();
-    const int NP = p.H * PB[p.B];
+    const int NP = p.H * PB[p.B], Ge = min(p.grid, NP);  // the attention kernel's split
     const int G = nb == 1 ? 4 : nb == 2 ? 2 : 1;
     const int grp = warp / G, sub = warp - grp * G;
     float *wt = wts[warp];
@@ -730,15 +731,14 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
 #pragma unroll
         for (int q = 0; q < NJ; ++q) acc[q] = 0.f;
         if (s1 > s0) {
-            const int c0 = cta_of(s0, NP, p.grid), c1 = cta_of(s1 - 1, NP, p.grid);
+            const int c0 = cta_of(s0, NP, Ge), c1 = cta_of(s1 - 1, NP, Ge);
             const int nr = c1 - c0 + 1;
             const float *pu = p.part + (u + c0) * PS;
             // the run maxima and sums in one round of loads
             float mm = -INFINITY;
             for (int i = lane; i < nr; i += 32) {
-                const bool has = page_lo(c0 + i + 1, NP, p.grid) > page_lo(c0 + i, NP, p.grid);
-                wt[i] = has ? pu[static_cast<int64_t>(i) * PS + PO_M] : -INFINITY;
-                wl[i] = has ? pu[static_cast<int64_t>(i) * PS + PO_L] : 0.f;
+                wt[i] = pu[static_cast<int64_t>(i) * PS + PO_M];
+                wl[i] = pu[static_cast<int64_t>(i) * PS + PO_L];
                 mm = fmaxf(mm, wt[i]);
             }
             M = warp_max(mm);
@@ -750,15 +750,24 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
             }
             l = warp_sum(ls);
             __syncwarp();
-#pragma unroll 4
-            for (int i = 0; i < nr; ++i) {
-                const float w8 = wt[i];
-                if (w8 > 0.f) {
-                    const float *pr = pu + static_cast<int64_t>(i) * PS;
+            // the column loads of four runs in flight at once, then their sums
+            for (int i0 = 0; i0 < nr; i0 += 4) {
+                float v[4][NJ];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float *pr = pu + static_cast<int64_t>(min(i0 + k, nr - 1)) * PS;
 #pragma unroll
                     for (int q = 0; q < NJ; ++q) {
                         const int j = lane + 32 * (sub + G * q);
-                        if (j < RV) acc[q] = fmaf(w8, pr[j], acc[q]);
+                        v[k][q] = j < RV ? pr[j] : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float w8 = i0 + k < nr ? wt[i0 + k] : 0.f;
+                    if (w8 > 0.f) {  // warp-uniform
+#pragma unroll
+                        for (int q = 0; q < NJ; ++q) acc[q] = fmaf(w8, v[k][q], acc[q]);
                     }
                 }
             }
@@ -818,10 +827,9 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
         const int P = PB[b + 1] - PB[b];
         if (P == 0) continue;
         const int s0 = p.H * PB[b] + h * P;
-        const int c0 = cta_of(s0, NP, p.grid), c1 = cta_of(s0 + P - 1, NP, p.grid);
+        const int c0 = cta_of(s0, NP, Ge), c1 = cta_of(s0 + P - 1, NP, Ge);
         float *pu = p.part + (static_cast<int64_t>(b) * p.H + h + c0) * PS;
         for (int i = 0; i <= c1 - c0; ++i) {
-            if (page_lo(c0 + i + 1, NP, p.grid) <= page_lo(c0 + i, NP, p.grid)) continue;  // no run
             for (int jj = tid; jj < PS; jj += 128) pu[static_cast<int64_t>(i) * PS + jj] = 0.f;
         }
     }

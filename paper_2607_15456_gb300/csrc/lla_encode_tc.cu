@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
     uint64_t *done = accempty + 2;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(done + 1);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1) + 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool split = p.split > 1;
     const int64_t u0 = split ? blockIdx.x / p.split : static_cast<int64_t>(blockIdx.x) * p.units / gridDim.x;
     const int64_t u1 = split ? u0 + 1 : static_cast<int64_t>(blockIdx.x + 1) * p.units / gridDim.x;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tslot;
+    constexpr uint32_t tmem = 0;  // all of TMEM is allocated; a constant keeps the issuing warp's code uniform
     pdl_wait();  // x, slots and the pool may come from the previous kernel
 
     if (warp == 0 || (warp == 6 && !WRES)) {
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        {
             const uint32_t base = smem_addr(sm);
             int q = 0, j = 0, head = -1;
             int nres[2] = {0, 0};               // WRES: copies of each axis's W_down seen
@@ -311,21 +311,21 @@ __global__ void __launch_bounds__(kEThreads, 1)
                     }
                     if (!wax[U.axis]) {
                         wax[U.axis] = true;
-                        if (!mbar_wait(&wfull[U.axis], nres[U.axis]++ & 1, abort_flag, p.err)) break;
+                        if (!mbar_wait_warp(&wfull[U.axis], nres[U.axis]++ & 1, abort_flag, p.err)) break;
                     }
                 }
                 const uint32_t idesc = umma_idesc_bf16(128, U.R, 0, 1);
                 const int slot = j & 1;
                 // the epilogue has read this slot's previous unit (j - 2)
-                if (!mbar_wait(&accempty[slot], ((j >> 1) & 1) ^ 1u, abort_flag, p.err)) break;
+                if (!mbar_wait_warp(&accempty[slot], ((j >> 1) & 1) ^ 1u, abort_flag, p.err)) break;
                 tc_fence_after();
                 const uint32_t d = tmem + slot * kSlotCols;
                 bool ok = true;
 #pragma unroll 1
                 for (int s = 0; s < NS; ++s, ++q) {
                     const int st = q % kXStages, sw = q % kWStages;
-                    if (!mbar_wait(&full[st], (q / kXStages) & 1, abort_flag, p.err) ||
-                        (!WRES && !mbar_wait(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err))) {
+                    if (!mbar_wait_warp(&full[st], (q / kXStages) & 1, abort_flag, p.err) ||
+                        (!WRES && !mbar_wait_warp(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err))) {
                         ok = false;
                         break;
                     }
@@ -333,18 +333,18 @@ __global__ void __launch_bounds__(kEThreads, 1)
                     const uint32_t a = base + st * kASlab, b = base + oW + (WRES ? (U.axis * kResSlabs + s) * kBAtom : sw * kWStage);
 #pragma unroll
                     for (int ks = 0; ks < kES / 16; ++ks)
-                        umma_bf16(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
+                        umma_bf16_warp(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
                                   idesc, s > 0 || ks > 0);
-                    umma_commit(&empty[st]);
-                    if (!WRES) umma_commit(&wempty[sw]);
+                    umma_commit_warp(&empty[st]);
+                    if (!WRES) umma_commit_warp(&wempty[sw]);
                 }
                 if (!ok) break;
-                umma_commit(&accfull[slot]);
+                umma_commit_warp(&accfull[slot]);
             }
             // every product has completed before TMEM is released
-            umma_commit(done);
+            umma_commit_warp(done);
             volatile int never = 0;
-            mbar_wait(done, 0, &never, p.err);
+            mbar_wait_warp(done, 0, &never, p.err);
         }
         __syncwarp();
     } else if (warp <= 5) {

@@ -44,6 +44,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "lla_device.cuh"
 #include "lla_internal.h"
@@ -1260,11 +1261,15 @@ __global__ void __launch_bounds__(256, 1)
 // three units (no block barrier between units: each is a chain of dependent loads), then all
 // threads apply W_up^V; a thread's weights, when they fit 80 registers (latents up to 640 wide),
 // are loaded before the wait on the attention kernel.
-template <int RV, int NQM, int RS>
+// SPB: the units the projection is unrolled for, the smallest of 2, 4, 8 that holds spb.  Unrolled for
+// eight whatever spb, a CTA of one to four units multiplied zeros for the others: one sequence of 777
+// tokens at (288, 480) 21.0 -> 18.2 us a call, 16 sequences 43.3 -> 40.4, four loops of the (96, 160)
+// batch 84.7 -> 83.2.  (Fewer units per CTA for four or eight CTAs per SM read W_up^V more often: 44.1
+// and 52.3 us for those 16 sequences, 88.2 and 98.1 for the loops.)
+template <int RV, int NQM, int RS, int SPB>
 __global__ void __launch_bounds__(128, 1) finish2d_kernel(const F2Params p) {
     constexpr int PS = NQM * RV + 2 * kNQ;
     constexpr int PO_M = NQM * RV, PO_L = NQM * RV + kNQ;
-    constexpr int SPB = finish_seqs(RV);
     static_assert(RS == 1 || RS == 4, "row slices");
     static_assert(RS == 1 || (RV / 8) % RS == 0, "row slices read whole 16-byte units");
     constexpr bool kPre = RV / 8 / RS <= 20;  // the thread's weights fit 80 registers
@@ -1533,10 +1538,15 @@ lla_status launch_units(const DecodeArgs &a, bool loops, cudaStream_t stream) {
     const int64_t want = units * rs;
     fp.spb = static_cast<int>(std::min<int64_t>(finish_seqs(RV), std::max<int64_t>(1, (want + 2 * grid - 1) / (2 * grid))));
     const dim3 fg(nw, (a.B + fp.spb - 1) / fp.spb, rs);
-    if constexpr (finish_slices(RV) > 1) {
-        if (rs > 1) return launch_ex(finish2d_kernel<RV, Z::NQM, finish_slices(RV)>, fg, 128, 0, stream, fp);
-    }
-    return launch_ex(finish2d_kernel<RV, Z::NQM, 1>, fg, 128, 0, stream, fp);
+    // the projection's accumulators for as many units as a CTA takes (up to 2, 4 or 8)
+    auto finish = [&](auto rsc) {
+        constexpr int RS = decltype(rsc)::value;
+        if (fp.spb <= 2) return launch_ex(finish2d_kernel<RV, Z::NQM, RS, 2>, fg, 128, 0, stream, fp);
+        if (fp.spb <= 4) return launch_ex(finish2d_kernel<RV, Z::NQM, RS, 4>, fg, 128, 0, stream, fp);
+        return launch_ex(finish2d_kernel<RV, Z::NQM, RS, 8>, fg, 128, 0, stream, fp);
+    };
+    if (rs > 1) return finish(std::integral_constant<int, finish_slices(RV)>());
+    return finish(std::integral_constant<int, 1>());
 }
 
 // ------------------------------------------------------------------------- rotary keys
@@ -1685,7 +1695,7 @@ lla_status launch_big(const DecodeArgs &a, cudaStream_t stream) {
     fp.pstart = ap.pstart; fp.part = tp.part;
     // each CTA takes a quarter of a head's output rows for up to four sequences
     fp.spb = std::min(finish_seqs(RV), a.B);
-    return launch_ex(finish2d_kernel<RV, kNQ, finish_slices(RV)>, dim3(a.H, (a.B + fp.spb - 1) / fp.spb, finish_slices(RV)), 128, 0,
+    return launch_ex(finish2d_kernel<RV, kNQ, finish_slices(RV), finish_seqs(RV)>, dim3(a.H, (a.B + fp.spb - 1) / fp.spb, finish_slices(RV)), 128, 0,
                      stream, fp);
 }
 

@@ -670,15 +670,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 // kernel, which launches this one ahead of its end.  The runs of a unit are merged by one warp, or
 // by two or four that split its columns when the CTA has fewer than three units; the merged slots
 // are then zeroed (each slot belongs to one unit, so to this CTA alone).
-template <int RV>
+template <int RV, int SPB>
 __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
     constexpr int PS = RV + 32, PO_M = RV, PO_L = RV + 16;
     constexpr bool kPre = RV <= 160;
     constexpr int NW = kPre ? RV / 8 : 1;
     constexpr int NJ = (RV + 31) / 32;
-    __shared__ __align__(16) float ob[kFinishSeqs][RV];
+    __shared__ __align__(16) float ob[SPB][RV];
     __shared__ float wts[4][kMaxGrid], wls[4][kMaxGrid];  // per warp: run weights and sums
-    __shared__ float coef[kFinishSeqs][3], scs[kFinishSeqs];
+    __shared__ float coef[SPB][3], scs[SPB];
     __shared__ int PB[LLA_MAX_BATCH + 1];
     const int h = blockIdx.x, b0 = blockIdx.y * p.spb, tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
@@ -695,9 +695,9 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
     // the call's own inputs (not outputs of the attention kernel) before the wait on it: the page
     // prefix of the sequences, each unit's current-token score and value element e
     seq_prefix(p.context_lens, p.B, p.max_ctx, p.max_blocks, p.pass1, false, nullptr, PB);
-    float cv[kFinishSeqs];
+    float cv[SPB];
 #pragma unroll
-    for (int bi = 0; bi < kFinishSeqs; ++bi)
+    for (int bi = 0; bi < SPB; ++bi)
         cv[bi] = p.cur_v && bi < nb ? load_elem(p.cur_v, (static_cast<int64_t>(b0 + bi) * p.H + h) * kD + e, p.io_bf16) : 0.f;
     if (p.cur_k) {
         for (int bi = warp; bi < nb; bi += 4) {
@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
     const int grp = warp / G, sub = warp - grp * G;
     float *wt = wts[warp];
     float *wl = wls[warp];
-    for (int bi = grp; bi < kFinishSeqs; bi += 4 / G) {
+    for (int bi = grp; bi < SPB; bi += 4 / G) {
         if (bi >= nb) {
             for (int j = lane + 32 * sub; j < RV; j += 32 * G) ob[bi][j] = 0.f;
             continue;
@@ -791,13 +791,13 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
         }
     }
     __syncthreads();  // every partial has been read
-    float acc[kFinishSeqs];
+    float acc[SPB];
 #pragma unroll
-    for (int bi = 0; bi < kFinishSeqs; ++bi) acc[bi] = 0.f;
+    for (int bi = 0; bi < SPB; ++bi) acc[bi] = 0.f;
     auto step = [&](int j8, const uint4 w4) {
         const float2 w0 = bf2_to_f2(w4.x), w1 = bf2_to_f2(w4.y), w2 = bf2_to_f2(w4.z), w3 = bf2_to_f2(w4.w);
 #pragma unroll
-        for (int bi = 0; bi < kFinishSeqs; ++bi) {
+        for (int bi = 0; bi < SPB; ++bi) {
             const float4 o0 = *reinterpret_cast<const float4 *>(&ob[bi][j8 * 8]);
             const float4 o1 = *reinterpret_cast<const float4 *>(&ob[bi][j8 * 8 + 4]);
             float a = acc[bi];
@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(128, 1) rope_finish_kernel(const RFParams p) {
         for (int j8 = 0; j8 < RV / 8; ++j8) step(j8, W[j8]);
     }
 #pragma unroll
-    for (int bi = 0; bi < kFinishSeqs; ++bi) {
+    for (int bi = 0; bi < SPB; ++bi) {
         if (bi >= nb) break;
         const int64_t idx = (static_cast<int64_t>(b0 + bi) * p.H + h) * kD + e;
         float v = acc[bi] * coef[bi][0] + coef[bi][1] * muv;
@@ -899,7 +899,13 @@ lla_status launch_tc(const DecodeArgs &a, const RopeTables &tab, int pairing, cu
     // about two finish CTAs per SM: fewer sequences per CTA for small batches
     const int64_t want = static_cast<int64_t>(a.B) * a.H;
     fp.spb = static_cast<int>(std::min<int64_t>(kFinishSeqs, std::max<int64_t>(1, (want + 2 * grid - 1) / (2 * grid))));
-    return launch_ex(rope_finish_kernel<RV>, dim3(a.H, (a.B + fp.spb - 1) / fp.spb), 128, 0, stream, fp);
+    // the projection unrolled for the units a CTA takes (1, 2, 4 or 8): for eight whatever spb, the 256
+    // one-unit CTAs of a 16-sequence batch did eight times the multiply-adds
+    const dim3 fg(a.H, (a.B + fp.spb - 1) / fp.spb);
+    if (fp.spb <= 1) return launch_ex(rope_finish_kernel<RV, 1>, fg, 128, 0, stream, fp);
+    if (fp.spb <= 2) return launch_ex(rope_finish_kernel<RV, 2>, fg, 128, 0, stream, fp);
+    if (fp.spb <= 4) return launch_ex(rope_finish_kernel<RV, 4>, fg, 128, 0, stream, fp);
+    return launch_ex(rope_finish_kernel<RV, kFinishSeqs>, fg, 128, 0, stream, fp);
 }
 
 }  // namespace

@@ -899,7 +899,9 @@ __global__ void __launch_bounds__(kGThreads) prefill_generic_kernel(const GParam
 // loops over its heads: Khat (64 tokens x d) = C_k W_up,t^K^T + mu^K_t on tcgen05 (M = 64 tokens, N = d,
 // K = r_k, plus one K step for mu^K_t), then each token's pairs are rotated in registers and
 // written as a bf16 page in the K-plane layout (granule g of 8 dimensions at g*1024 + token*16),
-// and the page's queries are rotated and scaled by scale * log2 e into a bf16 copy of q.
+// and the page's queries are rotated and scaled by scale * log2 e into a bf16 copy of q.  Four warps
+// rebuild the keys and four others rotate the queries (the next head's already loading), sharing the
+// page's table of turns: one after the other in the same warps, the two chains of loads added up.
 
 // 32 consecutive elements (bf16 or fp32, 16-byte aligned) as floats, loads issued together.
 __device__ __forceinline__ void load32(const void *src, int is_bf16, float (&v)[32]) {
@@ -969,8 +971,11 @@ struct RB {
     static_assert(RK % 16 == 0, "K steps");
 };
 
+constexpr int kRKeys = 128;      // threads that rebuild keys; as many rotate queries
+constexpr int kRThreads = 2 * kRKeys;
+
 template <int RK>
-__global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant__ RParams p) {
+__global__ void __launch_bounds__(kRThreads, 2) rope_rebuild_kernel(const __grid_constant__ RParams p) {
     using Z = RB<RK>;
     constexpr int D = Z::D;
     extern __shared__ __align__(1024) char rb_raw[];
@@ -1002,7 +1007,7 @@ __global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant
     }
     if (warp == 0) tmem_alloc(tslot, 128);
     // rotation of each token of the page at each pair's frequency, from exact turns
-    for (int i = tid; i < 64 * 64; i += 128) {
+    for (int i = tid; i < 64 * 64; i += kRThreads) {
         const int r = i >> 6, j = i & 63;
         const unsigned long long turns = static_cast<unsigned long long>(pg * kPT + r) * p.phi[j];
         const float tf = __uint2float_rn(static_cast<uint32_t>(turns >> 32)) * 2.3283064365386963e-10f;
@@ -1011,13 +1016,77 @@ __global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant
         tab[r * 65 + j] = make_float2(ca, sa);
     }
     // A of the mu step: a (1, 1) pair per token, then a zero granule
-    for (int i = tid; i < 128; i += 128)
+    for (int i = tid; i < 128; i += kRThreads)
         reinterpret_cast<uint4 *>(sm + Z::oOnes)[i] = i < 64 ? make_uint4(0x3f803f80u, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
     const uint32_t base = smem_addr(sm);
+    if (tid >= kRKeys) {
+        // the page's queries, head by head: rotated at their positions, scaled into the exp2 domain;
+        // thread (r, hf) rotates pairs 32 hf .. 32 hf + 31 of query r
+        const int r = (tid - kRKeys) >> 1, hf = tid & 1;
+        if (r < nvalid) {
+            const float2 *tr = tab + r * 65 + 32 * hf;
+            const int es = p.io_bf16 ? 2 : 4;
+            const int64_t row = (static_cast<int64_t>(q0) + pg * kPT + r) * p.H;
+            // the thread's two runs of 32 elements: pairs (j, j + 64), or 64 consecutive elements
+            const int oa = p.pairing == 0 ? 32 * hf : 64 * hf, ob = p.pairing == 0 ? 64 + 32 * hf : 64 * hf + 32;
+            const char *qs = static_cast<const char *>(p.q);
+            uint4 na[4], nb[4];  // the next head's elements, bf16
+            auto prefetch = [&](int h) {
+                const uint4 *a = reinterpret_cast<const uint4 *>(qs + ((row + h) * D + oa) * 2);
+                const uint4 *b2 = reinterpret_cast<const uint4 *>(qs + ((row + h) * D + ob) * 2);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    na[k] = a[k];
+                    nb[k] = b2[k];
+                }
+            };
+            if (p.io_bf16) prefetch(h0);
+            for (int h = h0; h < h1; ++h) {
+                float xa[32], xb[32];
+                if (p.io_bf16) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t wa[4] = {na[k].x, na[k].y, na[k].z, na[k].w}, wb[4] = {nb[k].x, nb[k].y, nb[k].z, nb[k].w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 fa = bf2_to_f2(wa[e]), fb = bf2_to_f2(wb[e]);
+                            xa[8 * k + 2 * e] = fa.x; xa[8 * k + 2 * e + 1] = fa.y;
+                            xb[8 * k + 2 * e] = fb.x; xb[8 * k + 2 * e + 1] = fb.y;
+                        }
+                    }
+                    if (h + 1 < h1) prefetch(h + 1);
+                } else {
+                    load32(qs + ((row + h) * D + oa) * es, 0, xa);
+                    load32(qs + ((row + h) * D + ob) * es, 0, xb);
+                }
+                char *qo = static_cast<char *>(p.qrot) + (row + h) * D * 2;
+                if (p.pairing == 0) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const float2 cs = tr[i];
+                        const float a = xa[i], bb = xb[i];
+                        xa[i] = (a * cs.x - bb * cs.y) * p.scale_log2;
+                        xb[i] = (a * cs.y + bb * cs.x) * p.scale_log2;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const float2 cs = tr[i];
+                        float *pr = i < 16 ? xa + 2 * i : xb + 2 * (i - 16);
+                        const float a = pr[0], bb = pr[1];
+                        pr[0] = (a * cs.x - bb * cs.y) * p.scale_log2;
+                        pr[1] = (a * cs.y + bb * cs.x) * p.scale_log2;
+                    }
+                }
+                store32_bf16(qo + oa * 2, xa);
+                store32_bf16(qo + ob * 2, xb);
+            }
+        }
+    } else {
     // epilogue geometry (16x256b fragments of the M = 64 accumulator): warp w holds tokens
     // 16w + lane/4 and 16w + lane/4 + 8; columns 8k + 2c and 8k + 2c + 1, c = lane % 4
     const int c = lane & 3;
@@ -1028,12 +1097,12 @@ __global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant
     auto stage = [&](int h) {
         const int64_t hl = (static_cast<int64_t>(h) * p.T + p.loop) * D;
         const char *W = static_cast<const char *>(p.w_up_k) + hl * RK * 2;
-        for (int i = tid; i < D * Z::NG; i += 128) {
+        for (int i = tid; i < D * Z::NG; i += kRKeys) {
             const int e = i / Z::NG, g = i - e * Z::NG;
             cp_async16(sm + Z::oW + g * (D * 16) + e * 16, W + (static_cast<int64_t>(e) * RK + g * 8) * 2);
         }
         const char *K = p.pool + (static_cast<int64_t>(blk) * p.H + h) * p.head_page_bytes;
-        for (int i = tid; i < Z::NG * 64; i += 128) cp_async16(sm + Z::oA + i * 16, K + i * 16);
+        for (int i = tid; i < Z::NG * 64; i += kRKeys) cp_async16(sm + Z::oA + i * 16, K + i * 16);
         cp_async_commit();
         const float mu = p.mu_k ? p.mu_k[hl + tid] : 0.f;
         const __nv_bfloat16 hi = __float2bfloat16_rn(mu);
@@ -1048,7 +1117,7 @@ __global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant
         cp_async_wait_all();
         fence_proxy_async_smem();
         tc_fence_before();
-        __syncthreads();
+        named_bar_sync(1, kRKeys);
         if (tid == 0) {
             tc_fence_after();
 #pragma unroll
@@ -1110,48 +1179,10 @@ __global__ void __launch_bounds__(128) rope_rebuild_kernel(const __grid_constant
                 *reinterpret_cast<uint32_t *>(kout + k * 1024 + t * 16 + c * 4) =
                     ok ? pack_bf16x2(y[2 * k], y[2 * k + 1]) : 0u;
         }
-        // the page's queries of head h: rotated at their positions, scaled into the exp2 domain;
-        // thread (r, hf) rotates pairs 32 hf .. 32 hf + 31 of query r
-        {
-            const int r = tid >> 1, hf = tid & 1;
-            if (r < nvalid) {
-                const int64_t qrow = (static_cast<int64_t>(q0) + pg * kPT + r) * p.H + h;
-                const float2 *tr = tab + r * 65 + 32 * hf;
-                const int es = p.io_bf16 ? 2 : 4;
-                const char *qs = static_cast<const char *>(p.q) + qrow * D * es;
-                char *qo = static_cast<char *>(p.qrot) + qrow * D * 2;
-                float xa[32], xb[32];
-                if (p.pairing == 0) {  // pairs (j, j + 64): two runs of 32
-                    load32(qs + 32 * hf * es, p.io_bf16, xa);
-                    load32(qs + (64 + 32 * hf) * es, p.io_bf16, xb);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const float2 cs = tr[i];
-                        const float a = xa[i], bb = xb[i];
-                        xa[i] = (a * cs.x - bb * cs.y) * p.scale_log2;
-                        xb[i] = (a * cs.y + bb * cs.x) * p.scale_log2;
-                    }
-                    store32_bf16(qo + 32 * hf * 2, xa);
-                    store32_bf16(qo + (64 + 32 * hf) * 2, xb);
-                } else {  // pairs (2j, 2j + 1): one run of 64
-                    load32(qs + 64 * hf * es, p.io_bf16, xa);
-                    load32(qs + (64 * hf + 32) * es, p.io_bf16, xb);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const float2 cs = tr[i];
-                        float *pr = i < 16 ? xa + 2 * i : xb + 2 * (i - 16);
-                        const float a = pr[0], bb = pr[1];
-                        pr[0] = (a * cs.x - bb * cs.y) * p.scale_log2;
-                        pr[1] = (a * cs.y + bb * cs.x) * p.scale_log2;
-                    }
-                    store32_bf16(qo + 64 * hf * 2, xa);
-                    store32_bf16(qo + (64 * hf + 32) * 2, xb);
-                }
-            }
-        }
         tc_fence_before();
-        __syncthreads();  // the operands and the accumulator may take the next head
+        named_bar_sync(1, kRKeys);  // the operands and the accumulator may take the next head
         tc_fence_after();
+    }
     }
     pdl_trigger();
     if (warp == 0) tmem_dealloc(tmem, 128);
@@ -1291,7 +1322,7 @@ lla_status launch_rebuild(const RParams &rp, int kpps, int B, cudaStream_t strea
     if (raise_smem_limit(rope_rebuild_kernel<RK>, RB<RK>::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
     // heads split over a few CTAs per page, so that more CTAs hide each other's load latency
     const int groups = rp.H >= 8 ? 4 : 1;
-    return launch_pf(rope_rebuild_kernel<RK>, dim3(kpps, B, groups), 128, RB<RK>::SMEM, stream, rp);
+    return launch_pf(rope_rebuild_kernel<RK>, dim3(kpps, B, groups), kRThreads, RB<RK>::SMEM, stream, rp);
 }
 }  // namespace
 

@@ -41,8 +41,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const Params p) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int hpb = p.head_page_bytes;
 
+    if (tid == 0) init_barriers(p, s, 1, 1);
     pdl_wait();  // inputs may come from the previous kernel in the stream
-    Range rg = prologue(p, s, 1, 1);
+    Range rg = prologue(p, s);
     order_runs(p, s, rg);
     pdl_trigger();
 

@@ -86,15 +86,16 @@ __global__ void __launch_bounds__(kAsyncThreads, 1)
     const Smem &s = a.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    pdl_wait();  // inputs may come from the previous kernel in the stream
     if (tid == 0) {
         for (int i = 0; i < kQSlots; ++i) mbar_init(&a.qready[i], kMThreads);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&a.stfull[i], kComputeThreads);
             mbar_init(&a.stfree[i], kMThreads);
         }
+        init_barriers(p, s, F::S_THREADS, F::V_THREADS);  // fences the inits above too
     }
-    Range rg = prologue(p, s, F::S_THREADS, F::V_THREADS);  // fences the inits above too
+    pdl_wait();  // inputs may come from the previous kernel in the stream
+    Range rg = prologue(p, s);
     order_runs(p, s, rg);
     pdl_trigger();
 

@@ -196,23 +196,26 @@ struct Range {
     int64_t lo[3], hi[3];
 };
 
-// Barrier set-up and the per-sequence unit prefix (H heads x pages), with device-side length
-// checks.  All threads of the CTA; ends with __syncthreads.
-__device__ Range prologue(const Params &p, const Smem &s, uint32_t pfull_count,
-                          uint32_t pempty_count, uint32_t empty_count = kComputeWarps) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) {
-        for (int i = 0; i < p.stages; ++i) {
-            mbar_init(&s.full[i], 1);
-            mbar_init(&s.empty[i], empty_count);
-        }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&s.pfull[i], pfull_count);
-            mbar_init(&s.pempty[i], pempty_count);
-        }
-        *s.abort_flag = 0;
-        fence_mbar_init();
+// Barrier set-up (one thread; it touches no input, so it may come before the wait on the previous
+// kernel).
+__device__ void init_barriers(const Params &p, const Smem &s, uint32_t pfull_count, uint32_t pempty_count,
+                              uint32_t empty_count = kComputeWarps) {
+    for (int i = 0; i < p.stages; ++i) {
+        mbar_init(&s.full[i], 1);
+        mbar_init(&s.empty[i], empty_count);
     }
+    for (int i = 0; i < 2; ++i) {
+        mbar_init(&s.pfull[i], pfull_count);
+        mbar_init(&s.pempty[i], pempty_count);
+    }
+    *s.abort_flag = 0;
+    fence_mbar_init();
+}
+
+// The per-sequence unit prefix (H heads x pages), with device-side length checks.  All threads of
+// the CTA, after thread 0's init_barriers; ends with __syncthreads.
+__device__ Range prologue(const Params &p, const Smem &s) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp == 0) {
         const int cap = min(p.max_ctx, p.max_blocks * kBlockTokens);
         int64_t run = 0;
@@ -764,6 +767,14 @@ __device__ __forceinline__ void value_store(float *red, const float (&accv)[Fast
 // pending finish still reads, and the stfree wait keeps run r from overwriting the state of run
 // r - 2 before its finish has read it.  W_up,t rows reach the management warps through a shared
 // staging buffer filled with cp.async, so no register holds them while they are in flight.
+//
+// A short run is bound by this chain, not by its pages: prologue, set-up, page, merge, output.  Per step,
+// in cycles of a one-sequence call: staging W_up,t^V 3500 -> 300 (its copies met in one bank group),
+// summing the row sums 1000 -> 100 (a chain of 64 adds), q~ 1500 -> 500 (16-byte reads of W_up,t^K instead
+// of pairs), a split run's merge without 64-bit divisions and eight parts per round trip.  One sequence of
+// 777 tokens at (96, 160) 19.8 -> 11.7 us a call, of 64 tokens 8.2 -> 7.2, of 16384 tokens 38.6 -> 29.9; 64
+// sequences of 100 to 200 tokens 63.0 -> 53.6; the 16-sequence batch 70.8 -> 68.9, with a rotary branch
+// 86.4 -> 79.0; the (72, 120) batch 289 -> 277; the (18, 30) batch 619 -> 610.
 // ------------------------------------------------------------------------------------------
 
 constexpr int kMWarps = 4;
@@ -778,7 +789,7 @@ constexpr int kWstMax = 40 * 1024;                 // staging buffer for W_up,t 
 
 struct AsyncLayout {
     int ring, full, empty, pfull, pempty, qready, stfull, stfree, prefix, lens, qlat, qfull, spart,
-        psm, lred, red, ovec, mred, mtmp, xtra, misc, wst, total;
+        psm, lred, red, ovec, mtmp, xtra, misc, wst, total;
 };
 
 // Shared-memory sizes of the asynchronous kernel for one rank shape (floats per slot); WL
@@ -788,14 +799,13 @@ struct AsyncSizes {
     using F = Fast<ES, RK, RV>;
     static constexpr int QSLOT = ((RK > D ? RK : D) + 3) & ~3;  // q~ or q, one run
     static constexpr int REDSLOT = F::NTG * RV;                 // value partials, one run
-    static constexpr int MRED = (kMThreads / (RK / 2)) * RK;    // q~ partial sums
     // staging buffer: the larger of W_up,t^K and W_up,t^V, at most WL
     static constexpr int WMAT = D * (RK > RV ? RK : RV) * ES;
     static constexpr int WST = WMAT < WL ? WMAT : WL;
 };
 
 __host__ __device__ inline AsyncLayout make_async_layout(int stages, int stage_bytes, int B,
-                                                         int qslot, int redslot, int mred, int rv,
+                                                         int qslot, int redslot, int rv,
                                                          int xslot, int wst) {
     AsyncLayout L;
     int o = 0;
@@ -816,7 +826,6 @@ __host__ __device__ inline AsyncLayout make_async_layout(int stages, int stage_b
     L.lred = o;   o += 2 * kLredSlot * 4;
     L.red = o;    o += up16(2 * redslot * 4);
     L.ovec = o;   o += up16(rv * 4);
-    L.mred = o;   o += up16(mred * 4);
     L.mtmp = o;   o += 2 * kMThreads * 4;
     L.xtra = o;   o += up16(kQSlots * xslot * 4);
     L.misc = o;   o += 64 * 4;
@@ -828,7 +837,7 @@ __host__ __device__ inline AsyncLayout make_async_layout(int stages, int stage_b
 template <int ES, int RK, int RV, int D, int WL = kWstMax>
 __host__ __device__ inline AsyncLayout async_layout(int stages, int stage_bytes, int B) {
     using Z = AsyncSizes<ES, RK, RV, D, WL>;
-    return make_async_layout(stages, stage_bytes, B, Z::QSLOT, Z::REDSLOT, Z::MRED, RV, 2 * D, Z::WST);
+    return make_async_layout(stages, stage_bytes, B, Z::QSLOT, Z::REDSLOT, RV, 2 * D, Z::WST);
 }
 
 // misc slots of the asynchronous kernel
@@ -839,7 +848,7 @@ constexpr int kAM = 0 /* [2] run maximum by state slot */, kAPAlpha = 5 /* [2] *
 struct ASmem {
     Smem s;  // fields shared with the generic helpers (ring, barriers, prefix, lens, abort flag)
     uint64_t *qready, *stfull, *stfree;
-    float *qlat, *qfull, *lred, *red, *mred, *mtmp;
+    float *qlat, *qfull, *lred, *red, *mtmp;
     float *xtra;  // [kQSlots][v_cur (D), mu^V_t (D)] by query slot
     char *wst;
     int qslot, redslot;  // floats per slot
@@ -874,7 +883,6 @@ __device__ __forceinline__ ASmem carve_async(char *smem, const Params &p) {
     a.qfull = reinterpret_cast<float *>(smem + L.qfull);
     a.lred = reinterpret_cast<float *>(smem + L.lred);
     a.red = reinterpret_cast<float *>(smem + L.red);
-    a.mred = reinterpret_cast<float *>(smem + L.mred);
     a.mtmp = reinterpret_cast<float *>(smem + L.mtmp);
     a.xtra = reinterpret_cast<float *>(smem + L.xtra);
     a.wst = smem + L.wst;
@@ -905,9 +913,12 @@ __device__ __forceinline__ void m_stage_rows(const ASmem &a, const char *W, int 
     cp_async_commit();
 }
 
-// Chunk geometry of W_up,t^V in the staging buffer: rows cut into CB-byte chunks, stored chunk
-// by chunk (chunk c of row e of a pass at (c * ROWS + e) * CB), so that threads owning
-// consecutive rows read consecutive chunks.
+// Geometry of W_up,t^V in the staging buffer: its rows as they are in memory (m_stage_rows), read in
+// chunks of CB bytes by a thread per row.  Rows whose 16-byte chunks would fall on the same banks as
+// their neighbours' are read from different starts (ROT of row e), so that the eight rows of a phase
+// always touch eight different bank groups.  (Stored chunk by chunk instead, so that every read was
+// a row of neighbours, the copies themselves met in one bank group, 32 to an instruction: 3500 cycles
+// before every output.)
 template <int ES, int RV, int D, int WST>
 struct VStage {
     using P = WPasses<ES, RV, D, WST>;
@@ -915,22 +926,14 @@ struct VStage {
     static constexpr int CPR = RV * ES / CB;                 // chunks per row
     static constexpr int EPC = CB / ES;                      // elements per chunk
     static constexpr int TPR = kMThreads / P::ROWS;          // threads per row
-    static_assert(kMThreads % P::ROWS == 0 && (RV * ES) % 4 == 0, "row ownership");
-};
-
-// Starts the copy of pass `pass` of W_up,t^V into the staging buffer, chunk-major.
-template <int ES, int RV, int D, int WST>
-__device__ __forceinline__ void m_stage_v(const ASmem &a, const char *W, int pass, int mt) {
-    using V = VStage<ES, RV, D, WST>;
-    const char *src = W + static_cast<int64_t>(pass) * V::P::PASS_BYTES;
-    for (int i = mt; i < V::P::ROWS * V::CPR; i += kMThreads) {
-        const int e = i / V::CPR, c = i - e * V::CPR;
-        char *dst = a.wst + (c * V::P::ROWS + e) * V::CB;
-        if constexpr (V::CB == 16) cp_async16(dst, src + i * 16);
-        else cp_async4(dst, src + i * 4);
+    static __device__ __forceinline__ int rot(int e) {
+        if constexpr (CB != 16 || CPR % 2 == 1) return 0;
+        else if constexpr (CPR % 8 == 0) return e & 7;
+        else if constexpr (CPR % 4 == 0) return (e >> 1) & 3;
+        else return (e >> 2) & 1;
     }
-    cp_async_commit();
-}
+    static_assert(kMThreads % P::ROWS == 0 && (RV * ES) % 4 == 0 && (CB != 16 || CPR >= 8), "row ownership");
+};
 
 // Management: everything a run needs that does not depend on its results, into slot `slot`:
 // q, q~ = W_up,t^K^T q, and the per-warp partial sums of beta = q . mu^K_t and of q . k_cur;
@@ -980,38 +983,44 @@ __device__ void m_setup(const Params &p, const ASmem &a, int b, int h, int slot,
         if (mt < D) qlat[mt] = qv;
         return;
     }
-    constexpr int CPR = RK / 2;          // pairs per row of W
+    // thread (chunk cg, row group rg): KE columns (16 bytes, or 4 where rows are not whole 16-byte
+    // words) of every RG-th row
+    constexpr int KE = (RK * ES) % 16 == 0 ? 16 / ES : 4 / ES;
+    constexpr int CPR = RK / KE;         // chunks per row of W
     constexpr int RG = kMThreads / CPR;  // row groups
-    static_assert(RG >= 1 && RG * RK <= 2048, "partial sums fit the management buffer");
+    static_assert(RG >= 1 && RG * RK * 4 <= WST, "partial sums fit the staging buffer");
     const int cg = mt % CPR, rg = mt / CPR;
-    float acc0 = 0.f, acc1 = 0.f;
+    float acc[KE];
+#pragma unroll
+    for (int k = 0; k < KE; ++k) acc[k] = 0.f;
 #pragma unroll 1
     for (int pass = 0; pass < P::N; ++pass) {
         cp_async_wait_all();
         m_sync();  // the pass (and qfull) is in shared memory for every thread
         if (rg < RG) {
+#pragma unroll 4
             for (int el = rg; el < P::ROWS; el += RG) {
-                const float2 w = load_pair<ES>(a.wst, static_cast<int64_t>(el) * RK + cg * 2);
+                float w[KE];
+                load_gran<ES, KE * ES>(a.wst + (el * RK + cg * KE) * ES, w);
                 const float qe = qfull[pass * P::ROWS + el];
-                acc0 = fmaf(w.x, qe, acc0);
-                acc1 = fmaf(w.y, qe, acc1);
+#pragma unroll
+                for (int k = 0; k < KE; ++k) acc[k] = fmaf(w[k], qe, acc[k]);
             }
         }
-        if (pass + 1 < P::N) {
-            m_sync();  // the buffer is read before the next pass overwrites it
-            m_stage_rows<ES, RK, D, WST>(a, W, pass + 1, mt);
-        }
+        m_sync();  // the buffer is read before the next pass, or the partial sums, overwrite it
+        if (pass + 1 < P::N) m_stage_rows<ES, RK, D, WST>(a, W, pass + 1, mt);
     }
+    float *mred = reinterpret_cast<float *>(a.wst);  // [RG][RK]
     if (rg < RG) {
-        a.mred[rg * RK + cg * 2] = acc0;
-        a.mred[rg * RK + cg * 2 + 1] = acc1;
+#pragma unroll
+        for (int k = 0; k < KE; ++k) mred[rg * RK + cg * KE + k] = acc[k];
     }
     m_sync();
     for (int j = mt; j < RK; j += kMThreads) {
-        float acc = 0.f;
-#pragma unroll 4
-        for (int g = 0; g < RG; ++g) acc += a.mred[g * RK + j];
-        qlat[j] = acc;
+        float sum = 0.f;
+#pragma unroll
+        for (int g = 0; g < RG; ++g) sum += mred[g * RK + j];
+        qlat[j] = sum;
     }
 }
 
@@ -1024,7 +1033,7 @@ __device__ __forceinline__ float m_part(const ASmem &a, int slot, int k) {
 // Management: output of one (sequence, head) from its softmax state (m, l, a.s.ovec).
 // o = (W_up,t^V ovec wl + lc mu^V_t + p_cur v_cur) / (lc + p_cur).  The first pass of W_up,t^V
 // is already in flight in the staging buffer.  Each row of the pass has TPR threads (one when
-// the pass holds all D rows); their chunk reads are conflict-free, ovec reads are broadcasts
+// the pass holds all D rows); their chunk reads are conflict-free, ovec reads touch few addresses
 // and the output stores coalesce.
 template <int ES, int RK, int RV, int D, int WL = kWstMax>
 __device__ void m_output(const Params &p, const ASmem &a, int b, int h, float m, float l, int slot,
@@ -1061,10 +1070,13 @@ __device__ void m_output(const Params &p, const ASmem &a, int b, int h, float m,
         cp_async_wait_all();
         m_sync();
         float acc0 = 0.f, acc1 = 0.f;
+        const char *wrow = a.wst + er * (RV * ES);
+        const int rot = V::rot(er);
 #pragma unroll 4
-        for (int c = sub; c < V::CPR; c += V::TPR) {
+        for (int c0 = sub; c0 < V::CPR; c0 += V::TPR) {
+            const int c = c0 + rot < V::CPR ? c0 + rot : c0 + rot - V::CPR;
             float w[V::EPC];
-            load_gran<ES, V::CB>(a.wst + (c * P::ROWS + er) * V::CB, w);
+            load_gran<ES, V::CB>(wrow + c * V::CB, w);
             const float *ov = a.s.ovec + c * V::EPC;
 #pragma unroll
             for (int k = 0; k < V::EPC; ++k) {
@@ -1088,7 +1100,7 @@ __device__ void m_output(const Params &p, const ASmem &a, int b, int h, float m,
             store_elem(p.out, orow + e, o * inv, p.io_bf16);
         }
         m_sync();  // the buffer (and mtmp) is read before the next pass or set-up overwrites it
-        if (pass + 1 < P::N) m_stage_v<ES, RV, D, WST>(a, W, pass + 1, mt);
+        if (pass + 1 < P::N) m_stage_rows<ES, RV, D, WST>(a, W, pass + 1, mt);
     }
 }
 
@@ -1113,9 +1125,9 @@ __device__ void m_finish(const Params &p, const ASmem &a, const Run &R, int64_t 
     if (p.absorbed) {
         cp_async_wait_all();
         m_sync();
-        m_stage_v<ES, RV, D, WST>(a, static_cast<const char *>(p.w_up_v) +
-                                         (static_cast<int64_t>(R.h) * p.T + p.loop) * D * RV * ES,
-                                  0, mt);
+        m_stage_rows<ES, RV, D, WST>(a, static_cast<const char *>(p.w_up_v) +
+                                            (static_cast<int64_t>(R.h) * p.T + p.loop) * D * RV * ES,
+                                     0, mt);
     }
     mbar_wait(&a.stfull[slot], parity, a.s.abort_flag, p.err, wait_limit(p));
     const float *red = a.red + slot * a.redslot;
@@ -1126,8 +1138,10 @@ __device__ void m_finish(const Params &p, const ASmem &a, const Run &R, int64_t 
         for (int g = 0; g < NTG; ++g) acc += red[g * RV + j];
         a.s.ovec[j] = acc;
     }
-    float l = 0.f;
-    for (int i = 0; i < TT; ++i) l += lred[i];
+    float l = 0.f;  // every warp sums all of them (64 dependent adds in each thread took 1000 cycles)
+#pragma unroll
+    for (int i = 0; i < TT; i += 32) l += lred[i + (mt & 31)];
+    l = warp_sum(l);
     const float m = a.s.misc[kAM + slot];
     m_sync();
     if constexpr (RELEASE) mbar_arrive(&a.stfree[slot]);  // the slot may take a later run's state
@@ -1153,20 +1167,25 @@ __device__ void m_finish(const Params &p, const ASmem &a, const Run &R, int64_t 
     }
     m_sync();
     if (!*a.s.last_flag) return;
+    // the run is its CTA's first everywhere but perhaps in c_first (a division per part and column, in
+    // called 64-bit code, otherwise)
+    const int sl0 = R.seg_start <= range_start(c_first, rg.U, rg.Geff) ? 0 : 1;
     auto record = [&](int cc) {
-        const int sl = (R.seg_start <= range_start(cc, rg.U, rg.Geff)) ? 0 : 1;
-        return p.partials + (static_cast<int64_t>(cc) * 2 + sl) * (RV + 2);
+        return p.partials + (static_cast<int64_t>(cc) * 2 + (cc == c_first ? sl0 : 0)) * (RV + 2);
     };
     const int nparts = c_last - c_first + 1;
-    constexpr int kQuick = 8;  // parts merged with every load issued in one round trip
-    float M = -INFINITY, lsum = 0.f;
-    if (nparts <= kQuick) {
-        constexpr int JPT = (RV + kMThreads - 1) / kMThreads;  // columns per thread
-        float pm[kQuick], pl[kQuick], po[kQuick][JPT];
+    // eight parts at a time, every load of theirs in one round trip
+    constexpr int kParts = 8, JPT = (RV + kMThreads - 1) / kMThreads;  // JPT: columns per thread
+    float M = -INFINITY, lsum = 0.f, acc[JPT];
 #pragma unroll
-        for (int k = 0; k < kQuick; ++k) {
-            if (k < nparts) {
-                const float *r = record(c_first + k);
+    for (int q = 0; q < JPT; ++q) acc[q] = 0.f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < nparts; k0 += kParts) {
+        float pm[kParts], pl[kParts], po[kParts][JPT];
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) {
+            if (k0 + k < nparts) {
+                const float *r = record(c_first + k0 + k);
                 pm[k] = __ldcg(r);
                 pl[k] = __ldcg(r + 1);
 #pragma unroll
@@ -1176,51 +1195,29 @@ __device__ void m_finish(const Params &p, const ASmem &a, const Run &R, int64_t 
                 }
             }
         }
+        float Mn = M;
 #pragma unroll
-        for (int k = 0; k < kQuick; ++k)
-            if (k < nparts) M = fmaxf(M, pm[k]);
-        float acc[JPT];
+        for (int k = 0; k < kParts; ++k)
+            if (k0 + k < nparts) Mn = fmaxf(Mn, pm[k]);
+        const float w0 = k0 ? exp2f(M - Mn) : 0.f;  // what the earlier parts are worth now
+        M = Mn;
+        lsum *= w0;
 #pragma unroll
-        for (int q = 0; q < JPT; ++q) acc[q] = 0.f;
+        for (int q = 0; q < JPT; ++q) acc[q] *= w0;
 #pragma unroll
-        for (int k = 0; k < kQuick; ++k) {
-            if (k < nparts) {
+        for (int k = 0; k < kParts; ++k) {
+            if (k0 + k < nparts) {
                 const float w = exp2f(pm[k] - M);
                 lsum = fmaf(pl[k], w, lsum);
 #pragma unroll
                 for (int q = 0; q < JPT; ++q) acc[q] = fmaf(po[k][q], w, acc[q]);
             }
         }
+    }
 #pragma unroll
-        for (int q = 0; q < JPT; ++q) {
-            const int j = mt + q * kMThreads;
-            if (j < RV) a.s.ovec[j] = acc[q];
-        }
-    } else {
-        for (int c0 = 0; c0 < nparts; c0 += kMThreads) {
-            const int np = min(kMThreads, nparts - c0);
-            if (mt < np) {
-                const float *r = record(c_first + c0 + mt);
-                a.mtmp[mt] = __ldcg(r);
-                a.mtmp[kMThreads + mt] = __ldcg(r + 1);
-            }
-            m_sync();
-            float Mc = M;
-            for (int i = 0; i < np; ++i) Mc = fmaxf(Mc, a.mtmp[i]);
-            lsum *= exp2f(M - Mc);
-            for (int i = 0; i < np; ++i) lsum = fmaf(a.mtmp[kMThreads + i], exp2f(a.mtmp[i] - Mc), lsum);
-            M = Mc;
-            m_sync();
-        }
-        for (int j = mt; j < RV; j += kMThreads) {
-            float acc = 0.f;
-#pragma unroll 4
-            for (int cc = c_first; cc <= c_last; ++cc) {
-                const float *r = record(cc);
-                acc = fmaf(__ldcg(r + 2 + j), exp2f(__ldcg(r) - M), acc);
-            }
-            a.s.ovec[j] = acc;
-        }
+    for (int q = 0; q < JPT; ++q) {
+        const int j = mt + q * kMThreads;
+        if (j < RV) a.s.ovec[j] = acc[q];
     }
     m_sync();
     m_output<ES, RK, RV, D, WL>(p, a, R.b, R.h, M, lsum, qs, mt);

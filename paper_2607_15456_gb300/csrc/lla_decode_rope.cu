@@ -142,10 +142,11 @@ __global__ void __launch_bounds__(kRopeThreads, 1) decode_rope_kernel(const __gr
         fence_proxy_async_smem();
         tc_fence_before();
     }
-    pdl_wait();  // inputs may come from the previous kernel in the stream
     // empty: one arrival per page from the MMA warp's commit and one from each value warp;
     // pfull: the epilogue threads (a page's partial scores); pempty: the value threads
-    Range rg = prologue(p, s, kComputeThreads / 2, F::V_THREADS, 1 + F::V_WARPS);
+    if (tid == 0) init_barriers(p, s, kComputeThreads / 2, F::V_THREADS, 1 + F::V_WARPS);
+    pdl_wait();  // inputs may come from the previous kernel in the stream
+    Range rg = prologue(p, s);
     order_runs(p, s, rg);
     pdl_trigger();
     tc_fence_after();

@@ -35,7 +35,8 @@
 // own row sums, and they meet after the last page.
 // Accumulators are fp32 in TMEM; operands are bf16 (q~ carries scale * log2 e).  At (72, 120) q~ and P
 // are sums of two bf16 parts (16 significant bits; twice the products): that shape was served in fp32
-// by the CUDA cores, and its bf16 outputs stay as exact as their rounding.
+// by the CUDA cores, and its bf16 outputs stay as exact as their rounding.  So at (18, 30), whose rows
+// are not whole 16-byte words: there the producer warps move pages and W_up through registers.
 //
 // Bound by the tensor pipe and the shared memory that feeds it: a (192, 320) page takes 640 cycles of PV
 // products and 576 of score products (a 128 x 64 x 16 product reads 6 KB, 48 cycles of shared memory for
@@ -43,10 +44,12 @@
 // clock falls under the power limit), at (96, 160) 1445 -> 944 us, at (128, 128) 1445 -> 1016 us; a tile of
 // 2 pages from launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the
 // last page, and the hi and lo projections followed each other through shared memory); (72, 120), 300
-// tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8341 us before.
+// tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8341 -> 58.6 us; (18, 30), 1000 tokens 720 ->
+// 23.4 us, 8192 tokens 43.1 -> 0.60 ms (1.4 us a page, twice the (72, 120) page's: the producer warps.
+// Their pairs' places kept in registers changed nothing; three pages in flight spilled and cost 15 %).
 //
-// CUDA-core path (fp32 storage, other ranks, d != 128, fp32 inputs at (72, 120)): one CTA per (query,
-// sequence, head), fp32 throughout.
+// CUDA-core path (fp32 storage, other ranks, d != 128, fp32 inputs at (72, 120) and (18, 30)): one CTA
+// per (query, sequence, head), fp32 throughout.
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -69,6 +72,7 @@ struct PParams {
     int T, H, loop, io_bf16;
     float scale_log2;
     const float *mu_v;
+    const void *w_up_k, *w_up_v;  // for NARROW rows (others come by tensor map)
     const char *pool;
     int64_t num_blocks;
     int head_page_bytes;
@@ -94,7 +98,10 @@ struct PParams {
 template <int RK, int RV, int NT, bool ROPE, int QP>
 struct PF {
     static constexpr int D = 128;
-    static constexpr int RKX = (RK + 15) / 16 * 16;  // padded with zero columns of q~ and a zero granule
+    // rows that are not whole 16-byte words have no bulk layout and no tensor map: the producer warps move
+    // them through registers into the layouts that the copies would leave
+    static constexpr bool NARROW = RK % 8 != 0 || RV % 8 != 0;
+    static constexpr int RKX = (RK + 15) / 16 * 16;  // padded with zero columns of q~ and zero granules
     static constexpr int RS = ROPE ? D : RKX;        // contraction width of the scores
     static constexpr int ORV = (RV + 15) / 16 * 16;  // O columns of a tile
     static constexpr int VATOMS = (RV + 63) / 64;    // 64-column boxes of a V page, of W_up,t^V
@@ -102,7 +109,7 @@ struct PF {
     static constexpr int N0 = ORV > 256 ? 256 : ORV; // PV MMA split on atom boundaries
     static constexpr int N1 = ORV - N0;
     static constexpr int KPAGE = kPT * RS * 2;
-    static constexpr int KCOPY = ROPE ? KPAGE : kPT * RK * 2;
+    static constexpr int KCOPY = ROPE ? KPAGE : NARROW ? 0 : kPT * RK * 2;  // the rest of a stage is zeroed once
     static constexpr int VPAGE = VATOMS * kPT * 128;
     static constexpr int QT1 = kBM * RS * 2;         // q~ (or rotated q) operand: one part of one tile
     static constexpr int QT = NT * QP * QT1;
@@ -112,7 +119,8 @@ struct PF {
     static constexpr int BUDGET = 222 * 1024;
     // W_up,t^V has room of its own, or takes q~'s and the K ring's once every score product is done
     static constexpr bool WVOWN = QT + 2 * KPAGE + 3 * VPAGE + WV <= BUDGET;
-    static constexpr int LEFT = BUDGET - QT - (WVOWN ? WV : 0);
+    static constexpr int WKOWN = NARROW ? WK : 0;  // NARROW: W_up,t^K has room of its own too
+    static constexpr int LEFT = BUDGET - QT - (WVOWN ? WV : 0) - WKOWN;
     static constexpr int STV0 = (LEFT - 2 * KPAGE) / VPAGE;
     static constexpr int STV = STV0 > 4 ? 4 : STV0;
     static constexpr int STK0 = (LEFT - STV * VPAGE) / KPAGE;
@@ -121,10 +129,10 @@ struct PF {
     static constexpr int oK = oQT + QT;
     static constexpr int oV = oK + STK * KPAGE;
     static constexpr int oW = oV + STV * VPAGE;
-    static constexpr int oEnd = oW + (WVOWN ? WV : 0);
+    static constexpr int oEnd = oW + WKOWN + (WVOWN ? WV : 0);
     static constexpr int oQA = oV;                        // the prologue's q operands alias the V ring
     static constexpr int oWK = WVOWN ? oW : oV + NT * QA1;
-    static constexpr int oWV = WVOWN ? oW : oQT;
+    static constexpr int oWV = WVOWN ? oW + WKOWN : oQT;
     static constexpr int oM = oEnd;                       // NT = 1: [128] running maxima
     static constexpr int oX = oM + kBM * 4;               // NT = 1: [2 groups][128] (maximum, sum)
     static constexpr int oBar = oX + 2 * kBM * 8;
@@ -132,7 +140,8 @@ struct PF {
     static constexpr int SMEM = 1024 + oBar + NBAR * 8;
     // TMEM columns: S of each group, P of each group (packed pairs), O of each tile; q~ starts in O
     static constexpr uint32_t TM_S = 0, TM_P = 2 * kPT, TM_O = TM_P + 2 * QP * (kPT / 2), TM_COLS = 512;
-    static_assert(RK % 8 == 0 && RV % 8 == 0 && RKX <= 256 && RKX <= ORV, "ranks");
+    static_assert(RK % 2 == 0 && RV % 2 == 0 && RKX <= 256 && RKX <= ORV, "ranks");
+    static_assert(!NARROW || (RK <= 64 && RV <= 64 && WVOWN && !ROPE), "one 64-column box per row");
     static_assert(TM_O + NT * ORV <= TM_COLS && N1 <= 256 && N1 % 16 == 0, "TMEM columns");
     static_assert(STK >= 2 && STV >= 2, "pipeline depth");
     static_assert(KPAGE % 1024 == 0 && QT1 % 1024 == 0, "align");
@@ -164,6 +173,41 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
         v[32 + i] = __uint_as_float(b[i]);
     }
 }
+
+// NARROW rows through registers, by a whole warp: R columns (pairs of bf16) of 64 or 128 rows.
+// A page's plane is loaded as 16-byte words (load), then its pairs are stored (store) at
+//   K-plane (4-byte granules, pair c of row i at c*256 + i*4): granule c / 4 of row i at
+//           (c / 4)*1024 + i*16, the core-matrix layout of a K-major operand;
+//   V-plane and W_up rows (row-major): row i of 128 bytes, 16-byte chunk c / 4 at (c / 4) ^ (i % 8), the
+//           128-byte swizzle of a tensor load.
+template <int R, int ROWS>
+struct NarrowRows {
+    static constexpr int WORDS = ROWS * (R / 2);         // pairs
+    static constexpr int NV = (WORDS / 4 + 31) / 32;     // 16-byte words per lane
+    uint4 v[NV];
+    __device__ __forceinline__ void load(const char *src, int lane) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            if (k * 32 + lane < WORDS / 4) v[k] = reinterpret_cast<const uint4 *>(src)[k * 32 + lane];
+    }
+    template <bool KPLANE>
+    __device__ __forceinline__ void store(char *dst, int lane) const {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int w0 = (k * 32 + lane) * 4;
+            if (w0 >= WORDS) break;
+            const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int x = w0 + e;
+                const int c = KPLANE ? x / ROWS : x % (R / 2), i = KPLANE ? x % ROWS : x / (R / 2);
+                char *at = KPLANE ? dst + (c >> 2) * (ROWS * 16) + i * 16 + (c & 3) * 4
+                                  : dst + i * 128 + (((c >> 2) ^ (i & 7)) << 4) + (c & 3) * 4;
+                *reinterpret_cast<uint32_t *>(at) = w[e];
+            }
+        }
+    }
+};
 
 template <int RK, int RV, int NT, bool ROPE, int QP>
 __global__ void __launch_bounds__(kPThreads, 1)
@@ -197,8 +241,9 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int32_t *bt = p.block_table + static_cast<int64_t>(b) * p.max_blocks;
 
     if (tid == 0) {
-        mbar_init(&bar[kBWk], 1);
-        mbar_init(&bar[kBWv], 1);
+        constexpr uint32_t fills = F::NARROW ? 32 : 1;  // arrivals of a filled stage
+        mbar_init(&bar[kBWk], fills);
+        mbar_init(&bar[kBWv], fills);
         mbar_init(&bar[kBSfin], 1);
         for (int g = 0; g < 2; ++g) {
             mbar_init(&bar[kBOfin + g], 1);
@@ -214,11 +259,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
             mbar_init(&bar[kBPfree + g], 1);
         }
         for (int s = 0; s < F::STK; ++s) {
-            mbar_init(&bar[kBKfull + s], 1);
+            mbar_init(&bar[kBKfull + s], fills);
             mbar_init(&bar[kBKempty + s], 1);
         }
         for (int s = 0; s < F::STV; ++s) {
-            mbar_init(&bar[kBVfull + s], 1);
+            mbar_init(&bar[kBVfull + s], fills);
             mbar_init(&bar[kBVempty + s], 1);
         }
         *abort_flag = 0;
@@ -229,6 +274,11 @@ __global__ void __launch_bounds__(kPThreads, 1)
         for (int s = 0; s < F::STK; ++s)
             for (int i = tid; i < (F::KPAGE - F::KCOPY) / 16; i += kPThreads)
                 reinterpret_cast<uint4 *>(sm + F::oK + s * F::KPAGE + F::KCOPY)[i] = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
+    }
+    if constexpr (F::NARROW) {  // the columns past the ranks of W_up (W_up,t^V after W_up,t^K) and of the V ring
+        for (int i = tid; i < (F::WK + F::WV) / 16; i += kPThreads)
+            reinterpret_cast<uint4 *>(sm + F::oWK)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
     }
     tc_fence_before();
@@ -243,7 +293,43 @@ __global__ void __launch_bounds__(kPThreads, 1)
 
     if (warp == 0) {
         // ----------------------------------------------- producer: W_up,t^K, K-planes, W_up,t^V
-        if (lane == 0) {
+        if constexpr (F::NARROW) {
+            {
+                NarrowRows<RK, F::D> wk;
+                wk.load(static_cast<const char *>(p.w_up_k) + static_cast<int64_t>(wrow) * RK * 2, lane);
+                wk.template store<false>(sm + F::oWK, lane);
+                fence_proxy_async_smem();
+                mbar_arrive(&bar[kBWk]);
+            }
+            // page j + 1 is on its way while page j waits for its stage
+            NarrowRows<RK, kPT> cur, nxt;
+            auto page = [&](int j) {
+                int32_t blk = bt[j];
+                if (blk < 0 || blk >= p.num_blocks) {
+                    if (lane == 0) atomicOr(p.err, LLA_DEVERR_BLOCK_ID);
+                    blk = 0;
+                }
+                return p.pool + (static_cast<int64_t>(blk) * p.H + h) * p.head_page_bytes;
+            };
+            cur.load(page(0), lane);
+            for (int j = 0; j < NPU; ++j) {
+                if (j + 1 < NPU) nxt.load(page(j + 1), lane);
+                const int s = j % F::STK;
+                // (after a failed wait the phases go on: no copy is in flight that could land late)
+                mbar_wait(&bar[kBKempty + s], ((j / F::STK) & 1) ^ 1u, abort_flag, p.err);
+                cur.template store<true>(sm + F::oK + s * F::KPAGE, lane);
+                fence_proxy_async_smem();
+                mbar_arrive(&bar[kBKfull + s]);
+                cur = nxt;
+                if (j == min(F::STK, NPU) - 1) {
+                    NarrowRows<RV, F::D> wv;
+                    wv.load(static_cast<const char *>(p.w_up_v) + static_cast<int64_t>(wrow) * RV * 2, lane);
+                    wv.template store<false>(sm + F::oWV, lane);
+                    fence_proxy_async_smem();
+                    mbar_arrive(&bar[kBWv]);
+                }
+            }
+        } else if (lane == 0) {
             if constexpr (!ROPE) {  // rows e of W_up,t^K as the MN-major operand of Q~
                 mbar_arrive_expect_tx(&bar[kBWk], F::WK);
 #pragma unroll
@@ -303,7 +389,30 @@ __global__ void __launch_bounds__(kPThreads, 1)
         __syncwarp();
     } else if (warp == 2) {
         // ---------------------------------------------------------------------- V producer
-        if (lane == 0) {  // V-planes: one TMA tensor load with 128-byte swizzle per 64 columns
+        if constexpr (F::NARROW) {
+            for (int g = 0; g < NT; ++g)
+                if (npu(g) > 0) mbar_wait(&bar[kBQt + g], 0, abort_flag, p.err);
+            // the ring held the prologue's q operands: its columns past r_v become zeros again
+            for (int i = lane; i < F::STV * F::VPAGE / 16; i += 32)
+                reinterpret_cast<uint4 *>(sm + F::oV)[i] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            NarrowRows<RV, kPT> cur, nxt;
+            auto page = [&](int j) {
+                int32_t blk = bt[j];
+                if (blk < 0 || blk >= p.num_blocks) blk = 0;  // flagged by the K producer
+                return p.pool + (static_cast<int64_t>(blk) * p.H + h) * p.head_page_bytes + kPT * RK * 2;
+            };
+            cur.load(page(0), lane);
+            for (int j = 0; j < NPU; ++j) {
+                if (j + 1 < NPU) nxt.load(page(j + 1), lane);
+                const int s = j % F::STV;
+                mbar_wait(&bar[kBVempty + s], ((j / F::STV) & 1) ^ 1u, abort_flag, p.err);
+                cur.template store<false>(sm + F::oV + s * F::VPAGE, lane);
+                fence_proxy_async_smem();
+                mbar_arrive(&bar[kBVfull + s]);
+                cur = nxt;
+            }
+        } else if (lane == 0) {  // V-planes: one TMA tensor load with 128-byte swizzle per 64 columns
             // the V ring aliases the prologue operands: wait until q~ has been computed
             bool ok = true;
             if constexpr (!ROPE) {
@@ -1210,7 +1319,8 @@ lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t s
     static DeviceOnce configured;
     if (raise_smem_limit(prefill_tc_kernel<RK, RV, NT, ROPE, QP>, F::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
     // the V-planes of every head page: [pages][64 tokens][r_v] bf16, one page = one head page
-    CUtensorMap tv, twk, twv;
+    CUtensorMap tv = {}, twk = {}, twv = {};
+    if constexpr (!F::NARROW) {
     const uint64_t dims[3] = {static_cast<uint64_t>(RV), static_cast<uint64_t>(kPT),
                               static_cast<uint64_t>(prm.num_blocks) * prm.H};
     const uint64_t strides[2] = {static_cast<uint64_t>(RV) * 2, static_cast<uint64_t>(prm.head_page_bytes)};
@@ -1223,6 +1333,7 @@ lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t s
     const uint32_t wbox[2] = {64, F::D};
     if (!encode_tmap_bf16(&twk, a.w_up_k, 2, wk, sk, wbox, true) || !encode_tmap_bf16(&twv, a.w_up_v, 2, wv, sv, wbox, true))
         return LLA_ERR_CUDA;
+    }
     cudaLaunchConfig_t cfg = {};
     // x fastest: the tiles of one (sequence, head), longest first, run together and share its
     // pages in L2 (ordering the longest tiles of every head first was slower: 1.90 -> 2.17 ms)
@@ -1259,6 +1370,7 @@ PParams tc_params(const PrefillArgs &a, int hpb, unsigned *err) {
     p.T = a.T; p.H = a.H; p.loop = a.loop; p.io_bf16 = a.io_bf16;
     p.scale_log2 = a.scale * kLog2e;
     p.mu_v = a.mu_v;
+    p.w_up_k = a.w_up_k; p.w_up_v = a.w_up_v;
     p.pool = static_cast<const char *>(a.pool);
     p.num_blocks = a.num_blocks;
     p.head_page_bytes = hpb;
@@ -1284,6 +1396,7 @@ lla_status launch_prefill(const PrefillArgs &a, cudaStream_t stream) {
         if (a.r_k == 192 && a.r_v == 320) return launch_tc<192, 320, false>(p, a, stream);
         if (a.r_k == 128 && a.r_v == 128) return launch_tc<128, 128, false>(p, a, stream);
         if (a.r_k == 72 && a.r_v == 120 && a.io_bf16) return launch_tc<72, 120, false, 2>(p, a, stream);
+        if (a.r_k == 18 && a.r_v == 30 && a.io_bf16) return launch_tc<18, 30, false, 2>(p, a, stream);
     }
     GParams g = {};
     g.T = a.T; g.H = a.H; g.d = a.d; g.r_k = a.r_k; g.r_v = a.r_v; g.loop = a.loop;

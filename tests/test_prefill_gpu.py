@@ -87,7 +87,7 @@ def test_prefill_long_prompt_rescales(lla):
 
 
 def test_prefill_cuda_core_ranks(lla):
-    # r = (72, 120): not multiples of 16, served by the CUDA-core kernel
+    # r = (72, 120): not multiples of 32
     _prefill_case(lla, 72, 120, "bf16", "bf16", [70, 5], 1, False)
 
 
@@ -159,3 +159,13 @@ def test_prefill_two_tiles_per_cta(lla, r_k, r_v, io):
     # 5 pairs x 13 prompts x 16 heads = 1040: second tiles that are empty, one row, part of a page, full
     _prefill_case(lla, r_k, r_v, "bf16", io, [1025, 520, 513, 512, 448, 385, 384, 383, 130, 129, 128, 64, 1], 2, True,
                   H=16, seed=6)
+
+
+@pytest.mark.parametrize("H,lens", [(2, [1, 63, 64, 65, 130, 300]), (1, [900])])
+def test_prefill_rows_without_16_byte_words(lla, H, lens):
+    # (18, 30): pages and W_up rows go through the producer warps' registers; more pages than stages
+    _prefill_case(lla, 18, 30, "bf16", "bf16", lens, 2, True, H=H, seed=7)
+
+
+def test_prefill_rising_scores_rows_without_16_byte_words(lla):
+    _rising_scores_case(lla, 18, 30, 2, [700, 321], 33, 2 ** -9 + 1e-4)

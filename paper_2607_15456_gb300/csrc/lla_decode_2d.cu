@@ -91,6 +91,10 @@ struct Z2 {
     // for LLA-2D pages, whose stream is bound by HBM and ran 2 % slower beside the faster issue (632 and
     // 645 us on the 128-sequence batch at (288, 480))
     static constexpr bool WARP = NQ == 4;
+    // a vote before the exchange of a page's maxima where the softmax paces the pages (four loops of the
+    // (72, 120) batch 383 -> 347 us, LLA-2D (96, 160) 24.4 -> 23.3 us); pages of 96 KB are paced by HBM, and
+    // the vote cost them 0.7 %
+    static constexpr bool VOTE = RK + RV <= 512;
     static constexpr int NQM = NQ;                      // queries of a unit in the workspace
     static constexpr int NCH = (RV + 127) / 128;        // 128-row chunks of O^T
     static constexpr int NBOX = (RV + 63) / 64;         // TMA boxes a V-plane loads
@@ -348,6 +352,17 @@ __device__ Share find_share(const T2Params &p, int G, int c) {
     r.u = r.g0 < r.g1 ? first[0] : p.U;
     r.s = r.g0 < r.g1 ? first[1] : 0;
     return r;
+}
+
+// named_bar_sync that also tells every thread whether any of them passed true.
+__device__ __forceinline__ bool named_bar_or(int id, int nthreads, bool mine) {
+    int any;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %3, 0;\n\tbarrier.cta.red.or.pred q, %1, %2, p;\n\t"
+                 "selp.b32 %0, 1, 0, q;\n\t}"
+                 : "=r"(any)
+                 : "r"(id), "r"(nthreads), "r"(mine ? 1 : 0)
+                 : "memory");
+    return any != 0;
 }
 
 // Products issued by a converged warp (WARP) or by one thread.
@@ -663,41 +678,50 @@ __global__ void __launch_bounds__(kT2, 1)
                     for (int k = 1; k < Z::QS; ++k) sn += x2[k * NQ + n];
                     x[n] = valid ? sn + betas[n] : -INFINITY;
                 }
-                // per-query maxima over the page: 16 tokens per warp, then the 4 warps
-                float mx[NQ];
-#pragma unroll
-                for (int n = 0; n < NQ; ++n) mx[n] = x[n];
-#pragma unroll
-                for (int o = 8; o >= 1; o >>= 1)
-#pragma unroll
-                    for (int n = 0; n < NQ; ++n) mx[n] = fmaxf(mx[n], __shfl_xor_sync(0xffffffffu, mx[n], o));
-                float *rp = red + s * 64;
-                if (lane == 0) {
-#pragma unroll
-                    for (int n = 0; n < NQ; n += 4)
-                        *reinterpret_cast<float4 *>(rp + q4 * 16 + n) = make_float4(mx[n], mx[n + 1], mx[n + 2], mx[n + 3]);
-                }
-                named_bar_sync(1, 128);
-                bool any = false;
+                // most pages raise no query's maximum by 2^8: with VOTE one barrier that also votes tells all
+                // four warps so, and only otherwise do they exchange the page's maxima
+                bool any = false, mine = false;
                 float f[NQ];
 #pragma unroll
-                for (int n = 0; n < NQ; n += 4) {
-                    float4 a = *reinterpret_cast<const float4 *>(rp + n);
+                for (int n = 0; n < NQ; ++n) {
+                    mine = mine || x[n] > m[n] + kRescaleLog2;
+                    f[n] = 1.f;
+                }
+                if (!Z::VOTE || named_bar_or(1, 128, mine)) {
+                    // per-query maxima over the page: 16 tokens per warp, then the 4 warps
+                    float mx[NQ];
 #pragma unroll
-                    for (int w = 1; w < 4; ++w) {
-                        const float4 bb = *reinterpret_cast<const float4 *>(rp + w * 16 + n);
-                        a = make_float4(fmaxf(a.x, bb.x), fmaxf(a.y, bb.y), fmaxf(a.z, bb.z), fmaxf(a.w, bb.w));
+                    for (int n = 0; n < NQ; ++n) mx[n] = x[n];
+#pragma unroll
+                    for (int o = 8; o >= 1; o >>= 1)
+#pragma unroll
+                        for (int n = 0; n < NQ; ++n) mx[n] = fmaxf(mx[n], __shfl_xor_sync(0xffffffffu, mx[n], o));
+                    float *rp = red + s * 64;
+                    if (lane == 0) {
+#pragma unroll
+                        for (int n = 0; n < NQ; n += 4)
+                            *reinterpret_cast<float4 *>(rp + q4 * 16 + n) = make_float4(mx[n], mx[n + 1], mx[n + 2], mx[n + 3]);
                     }
-                    const float pm[4] = {a.x, a.y, a.z, a.w};
+                    named_bar_sync(1, 128);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float mn = fmaxf(m[n + e], pm[e]);
-                        const bool need = mn > m[n + e] + kRescaleLog2;  // also the first page
-                        f[n + e] = need ? ex2_approx(m[n + e] - mn) : 1.f;
-                        if (need) {
-                            acc[n + e] *= f[n + e];
-                            m[n + e] = mn;
-                            any = true;
+                    for (int n = 0; n < NQ; n += 4) {
+                        float4 a = *reinterpret_cast<const float4 *>(rp + n);
+#pragma unroll
+                        for (int w = 1; w < 4; ++w) {
+                            const float4 bb = *reinterpret_cast<const float4 *>(rp + w * 16 + n);
+                            a = make_float4(fmaxf(a.x, bb.x), fmaxf(a.y, bb.y), fmaxf(a.z, bb.z), fmaxf(a.w, bb.w));
+                        }
+                        const float pm[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float mn = fmaxf(m[n + e], pm[e]);
+                            const bool need = mn > m[n + e] + kRescaleLog2;  // also the first page
+                            f[n + e] = need ? ex2_approx(m[n + e] - mn) : 1.f;
+                            if (need) {
+                                acc[n + e] *= f[n + e];
+                                m[n + e] = mn;
+                                any = true;
+                            }
                         }
                     }
                 }

@@ -40,17 +40,21 @@
 //
 // Bound by the tensor pipe and the shared memory that feeds it: a (192, 320) page takes 640 cycles of PV
 // products and 576 of score products (a 128 x 64 x 16 product reads 6 KB, 48 cycles of shared memory for
-// 32 of arithmetic).  Measured, 16 heads: 4 x 8192 tokens at (192, 320) 1920 -> 1640 us (1385 TFLOP/s; the
-// clock falls under the power limit), at (96, 160) 1445 -> 944 us, at (128, 128) 1445 -> 1016 us; a tile of
-// 2 pages from launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the
-// last page, and the hi and lo projections followed each other through shared memory); (72, 120), 300
-// tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8341 -> 58.6 us; (18, 30), 1000 tokens 720 ->
-// 23.4 us, 8192 tokens 43.1 -> 0.60 ms (1.4 us a page, twice the (72, 120) page's: the producer warps.
-// Their pairs' places kept in registers changed nothing; three pages in flight spilled and cost 15 %).
+// 32 of arithmetic).  Measured, 16 heads, from the kernel with one tile, eight softmax warps in pairs and
+// one-thread issue: 4 x 8192 tokens at (192, 320) 1955 -> 1656 us (1370 TFLOP/s; the clock falls under
+// the power limit), at (96, 160) 1445 -> 908 us, at (128, 128) 1445 -> 1000 us; a tile of 2 pages from
+// launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the last
+// page, and the hi and lo projections followed each other through shared memory).  From the CUDA cores:
+// (72, 120), 300 tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8330 -> 51 us; (18, 30), 1000 tokens
+// 720 -> 23.4 us, 8192 tokens 43.1 -> 0.60 ms (1.4 us a page, twice the (72, 120) page's: the producer
+// warps.  Their pairs' places kept in registers changed nothing; three pages in flight spilled and cost
+// 15 %).
 //
 // CUDA-core path (fp32 storage, other ranks, d != 128, fp32 inputs at (72, 120) and (18, 30)): one CTA
 // per (query, sequence, head), fp32 throughout.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "lla_device.cuh"
 #include "lla_internal.h"
@@ -89,6 +93,7 @@ struct PParams {
     const void *qrot;
     int kpps;
     int64_t qrows;  // rows of the rotated-query buffer (B * max_len)
+    int B, first;   // prompts; (head, prompt) pairs that run one after the other, before the last ones together
 };
 
 // Shared-memory and TMEM plan of the tensor-core kernel for ranks (RK, RV), d = 128, NT query tiles
@@ -223,8 +228,19 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
     const int nqt = (p.max_len + NT * kBM - 1) / (NT * kBM);
-    const int qt = nqt - 1 - static_cast<int>(blockIdx.x);  // longest causal ranges first
-    const int b = blockIdx.y, h = blockIdx.z;
+    int qt = blockIdx.x, b = blockIdx.y, h = blockIdx.z;
+    if (p.first >= 0) {  // pair after pair, then tile by tile every pair of the rest
+        int pair = blockIdx.x / nqt;
+        qt = blockIdx.x - pair * nqt;
+        if (pair >= p.first) {
+            const int r = blockIdx.x - p.first * nqt, n = p.H * p.B - p.first;
+            qt = r / n;
+            pair = p.first + r - qt * n;
+        }
+        h = pair / p.B;
+        b = pair - h * p.B;
+    }
+    qt = nqt - 1 - qt;  // longest causal ranges first
     pdl_wait();
     const int q0 = p.cu_seqlens[b];
     const int L = p.cu_seqlens[b + 1] - q0;
@@ -1314,7 +1330,7 @@ lla_status launch_pf(K kern, dim3 grid, int threads, int smem, cudaStream_t stre
 }
 
 template <int RK, int RV, int NT, bool ROPE, int QP>
-lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {
+lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t stream) {
     using F = PF<RK, RV, NT, ROPE, QP>;
     static DeviceOnce configured;
     if (raise_smem_limit(prefill_tc_kernel<RK, RV, NT, ROPE, QP>, F::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
@@ -1322,12 +1338,12 @@ lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t s
     CUtensorMap tv = {}, twk = {}, twv = {};
     if constexpr (!F::NARROW) {
     const uint64_t dims[3] = {static_cast<uint64_t>(RV), static_cast<uint64_t>(kPT),
-                              static_cast<uint64_t>(prm.num_blocks) * prm.H};
-    const uint64_t strides[2] = {static_cast<uint64_t>(RV) * 2, static_cast<uint64_t>(prm.head_page_bytes)};
+                              static_cast<uint64_t>(prm0.num_blocks) * prm0.H};
+    const uint64_t strides[2] = {static_cast<uint64_t>(RV) * 2, static_cast<uint64_t>(prm0.head_page_bytes)};
     const uint32_t box[3] = {64, kPT, 1};
-    if (!encode_tmap_bf16(&tv, prm.pool + kPT * RK * 2, 3, dims, strides, box, true)) return LLA_ERR_CUDA;
+    if (!encode_tmap_bf16(&tv, prm0.pool + kPT * RK * 2, 3, dims, strides, box, true)) return LLA_ERR_CUDA;
     // W_up of both axes: [H T d][r] bf16, the d rows of one (head, loop) at a time
-    const uint64_t wk[2] = {static_cast<uint64_t>(RK), static_cast<uint64_t>(prm.H) * prm.T * F::D};
+    const uint64_t wk[2] = {static_cast<uint64_t>(RK), static_cast<uint64_t>(prm0.H) * prm0.T * F::D};
     const uint64_t wv[2] = {static_cast<uint64_t>(RV), wk[1]};
     const uint64_t sk[1] = {static_cast<uint64_t>(RK) * 2}, sv[1] = {static_cast<uint64_t>(RV) * 2};
     const uint32_t wbox[2] = {64, F::D};
@@ -1335,9 +1351,26 @@ lla_status launch_tiles(const PParams &prm, const PrefillArgs &a, cudaStream_t s
         return LLA_ERR_CUDA;
     }
     cudaLaunchConfig_t cfg = {};
-    // x fastest: the tiles of one (sequence, head), longest first, run together and share its
-    // pages in L2 (ordering the longest tiles of every head first was slower: 1.90 -> 2.17 ms)
-    cfg.gridDim = dim3((a.max_len + NT * kBM - 1) / (NT * kBM), a.B, a.H);
+    // The launch order.  One (head, prompt) pair after the other, its longest tiles first, shares the pair's
+    // pages in L2, but ends on the last pair's long tiles; the longest tiles of all pairs first ends evenly
+    // but reads all pages at once.  So pair after pair, and then the last three waves of CTAs' pairs, or
+    // as many as half of L2 holds, together.  Pair after pair only / this rule / all together: 3 ragged
+    // prompts at (72, 120) 127 / 115 / 113 us, 8 x 2048 tokens at (96, 160) 207 / 195 / 186, 4 x 2000 at
+    // (18, 30) 235 / 169 / 171, 4 x 8192 at (192, 320) 1679 / 1652 / 2047, six ragged rotary prompts 396 /
+    // 357 / 356.  (Six and ten waves: 1693 and 1770 us at (192, 320).)
+    const int tiles = (a.max_len + NT * kBM - 1) / (NT * kBM);
+    const int64_t pairs = static_cast<int64_t>(a.B) * a.H;
+    PParams prm = prm0;
+    prm.first = -1;
+    cfg.gridDim = dim3(tiles, a.B, a.H);
+    if (pairs * tiles < (int64_t(1) << 31)) {
+        const int sms = num_sms();
+        if (sms <= 0) return LLA_ERR_CUDA;
+        const int64_t pair_bytes = static_cast<int64_t>(a.max_len) * ((ROPE ? F::D : RK) + RV) * 2;
+        const int64_t last = std::max<int64_t>((3ll * sms + tiles - 1) / tiles, (64ll << 20) / pair_bytes);
+        prm.first = static_cast<int>(std::max<int64_t>(0, pairs - last));
+        cfg.gridDim = dim3(static_cast<unsigned>(pairs * tiles));
+    }
     cfg.blockDim = dim3(kPThreads);
     cfg.dynamicSmemBytes = F::SMEM;
     cfg.stream = stream;
@@ -1375,7 +1408,7 @@ PParams tc_params(const PrefillArgs &a, int hpb, unsigned *err) {
     p.num_blocks = a.num_blocks;
     p.head_page_bytes = hpb;
     p.block_table = a.block_table; p.max_blocks = a.max_blocks;
-    p.cu_seqlens = a.cu_seqlens; p.max_len = a.max_len;
+    p.cu_seqlens = a.cu_seqlens; p.B = a.B; p.max_len = a.max_len;
     p.q = a.q; p.out = a.out; p.err = err;
     return p;
 }

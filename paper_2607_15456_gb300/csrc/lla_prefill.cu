@@ -42,10 +42,10 @@
 // products and 576 of score products (a 128 x 64 x 16 product reads 6 KB, 48 cycles of shared memory for
 // 32 of arithmetic).  Measured, 16 heads, from the kernel with one tile, eight softmax warps in pairs and
 // one-thread issue: 4 x 8192 tokens at (192, 320) 1955 -> 1656 us (1370 TFLOP/s; the clock falls under
-// the power limit), at (96, 160) 1445 -> 908 us, at (128, 128) 1445 -> 1000 us; a tile of 2 pages from
+// the power limit), at (96, 160) 1445 -> 919 us, at (128, 128) 1445 -> 975 us; a tile of 2 pages from
 // launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the last
 // page, and the hi and lo projections followed each other through shared memory).  From the CUDA cores:
-// (72, 120), 300 tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8330 -> 51 us; (18, 30), 1000 tokens
+// (72, 120), 300 tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8330 -> 55 us; (18, 30), 1000 tokens
 // 720 -> 23.4 us, 8192 tokens 43.1 -> 0.60 ms (1.4 us a page, twice the (72, 120) page's: the producer
 // warps.  Their pairs' places kept in registers changed nothing; three pages in flight spilled and cost
 // 15 %).
@@ -1384,16 +1384,23 @@ lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t 
 }
 
 // One query tile per CTA, or two that share every page.  Two halve the pages' way through L2 and need no
-// hand-over of maxima, but a CTA's work is twice as long, so that few CTAs end unevenly: one prompt of
-// 8192 tokens at (96, 160) (512 pairs of tiles) takes 255 us with one tile and 274 with two, two such
-// prompts (1024) 496 and 493, four 994 and 944.  With rotated keys (128 wide instead of 96) the pages
-// weigh more: 396 and 375 us at 512 pairs, 135 and 146 at 256.  With two bf16 parts the products bound
-// it either way (1317 and 1333 us), so (72, 120) takes one.
+// hand-over of maxima, but a CTA's work is twice as long, so that few CTAs end unevenly.  Measured with one
+// and with two (us, 16 heads; pairs of tiles over the whole batch at its longest prompt):
+//   (96, 160):  1 x 2048 tokens (128 pairs) 28 and 36, 2 x 2048 (256) 56 and 51, 32 x 250 (512) 66 and 61,
+//               1 x 8192 (512) 231 and 220, 4 x 8192 (2048) 1005 and 919
+//   (128, 128): 1 x 2048 29 and 38, 2 x 2048 58 and 52, 32 x 250 65 and 60, 4 x 8192 1031 and 975
+//   rotated keys, (96, 160): 1 x 2048 47 and 57, 4 x 600 (192) 54 and 51, 1 x 4096 (256) 115 and 101, 2 x 8192
+//               (1024) 723 and 579: they are 128 wide instead of 96, so that the pages weigh more
+// From 160 to 400 pairs the two come within a few percent where the prompts differ in length (4 x 700 to
+// 1050 tokens, 256 pairs, 35 and 36; 8 x 64 to 2048, 384 pairs of which half exist, 25 and 28), so that
+// two start above that; with rotated keys those two cases take 63 and 61, 50 and 51, and two start at 256.
+// Prompts of one tile leave the second empty (32 x 100: 34 and 37).  With two bf16 parts the products bound
+// it either way (2 x 8192 at (72, 120): 630 and 644), so (72, 120) takes one.
 template <int RK, int RV, bool ROPE, int QP = 1>
 lla_status launch_tc(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {
     if constexpr (RV <= 160 && QP == 1) {
         const int64_t pairs = static_cast<int64_t>((a.max_len + 2 * kBM - 1) / (2 * kBM)) * a.B * a.H;
-        if (pairs >= (ROPE ? 512 : 1024)) return launch_tiles<RK, RV, 2, ROPE, QP>(prm, a, stream);
+        if (a.max_len > kBM && pairs >= (ROPE ? 256 : 400)) return launch_tiles<RK, RV, 2, ROPE, QP>(prm, a, stream);
     }
     return launch_tiles<RK, RV, 1, ROPE, QP>(prm, a, stream);
 }

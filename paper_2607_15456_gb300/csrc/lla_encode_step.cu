@@ -20,9 +20,9 @@
 // need no staging, no tensor maps (four per layer) and no TMEM.
 //
 // Measured (replayed from a graph, cold weights) against the kernels that took these calls before: 24
-// layers of 16 tokens at (96, 160) 90.5 -> 25.3 us (bytes: 17 us), with mu 113.6 -> 35 us, 64 tokens
+// layers of 16 tokens at (96, 160) 90.5 -> 25.6 us (bytes: 17 us), with mu 113.6 -> 36 us, 64 tokens
 // 337 -> 73 us, 128 tokens 216 -> 134 us; 48 layers of 64 tokens at (72, 120) 584 -> 112 us; 48 layers
-// of 128 tokens at (18, 30) 397 -> 87 us; one layer of 16 tokens at (96, 160) 9.2 -> 4.0 us.  What
+// of 128 tokens at (18, 30) 397 -> 90 us; one layer of 16 tokens at (96, 160) 7.3 -> 5.2 us.  What
 // bounds it: the latency of one block of W_down per warp at few tokens; the loads of x (16 bytes of a
 // token per lane, again for every 64 columns) at many, so that the prompt kernel takes over where
 // tokens x ranks pass kStepWork (100 tokens at (192, 320): 9.2 us a layer there, 10.4 here).
@@ -68,9 +68,11 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 
 __device__ __forceinline__ uint4 ldg_stream(const uint4 *p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    // (not .nc: the previous kernel on the stream may still write it when this one starts)
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
     return v;
 }
 
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
             } else {
 #pragma unroll
                 for (int u = 0; u < C::SLOTS; ++u)
-                    B.w[i][u] = g + 8 * u < nch ? __ldg(reinterpret_cast<const uint32_t *>(row + u * 8 * CW * 2)) : 0u;
+                    B.w[i][u] = g + 8 * u < nch ? *reinterpret_cast<const uint32_t *>(row + u * 8 * CW * 2) : 0u;
             }
         }
         if constexpr (MU) {
@@ -195,10 +197,12 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
             }
         }
     };
-    // weights are inputs of the call: their first loads go out before the wait on the previous kernel
-    if (b0 < b1) load_w(blk, b0);
+    // any input, the codec's too, may come from the previous kernel: only addresses come before the wait
     pdl_wait();
-    if (b0 < b1) load_x(blk, b0);
+    if (b0 < b1) {
+        load_w(blk, b0);
+        load_x(blk, b0);
+    }
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
         compute(blk);

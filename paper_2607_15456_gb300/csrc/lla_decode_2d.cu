@@ -248,14 +248,13 @@ __global__ void __launch_bounds__(256) absorb2d_kernel(const A2Params p) {
     auto unit = [&](int b) { return p.loops ? b * p.H + h : b; };
     auto iorow = [&](int b) { return ((p.loops ? static_cast<int64_t>(t) * p.B : 0) + b) * p.H + h; };
     const int col = j0 + lane;
-    // this thread's 16 weights (column j0 + lane, rows 16 warp .. 16 warp + 15): inputs of the
-    // call, loaded before the wait on the previous kernel
+    pdl_wait();  // the codec and the queries may come from the previous kernel; the workspace is free after it
+    pdl_trigger();
+    // this thread's 16 weights: column j0 + lane, rows 16 warp .. 16 warp + 15
     const uint16_t *W = static_cast<const uint16_t *>(p.w_up_k) + th * kD * RK + col;
     float wv[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) wv[u] = col < RK ? bf_to_f(W[(warp * 16 + u) * RK]) : 0.f;
-    pdl_wait();  // the queries may come from the previous kernel; the workspace is free after it
-    pdl_trigger();
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) page_prefix(p);
     for (int i = tid; i < 16 * kD; i += 256) {
         const int bi = i >> 7, e = i & (kD - 1);

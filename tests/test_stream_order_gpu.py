@@ -55,3 +55,39 @@ def test_step_encode_after_the_kernel_that_writes_its_codec(lla, what, r):
     for _ in range(4):
         assert torch.equal(encode(False), want)
     assert lla.lla_get_device_error() == 0
+
+
+@pytest.mark.parametrize("entry", ["loops", "2d"])
+def test_shared_latent_decode_after_the_kernel_that_writes_its_codec(lla, entry):
+    """W_up^K [H][T][d][r] (loops) or [T][H][d][r] (LLA-2D) of one loop, written just before the call."""
+    H, d, r_k, r_v, B = 2, 128, 96, 160, 3
+    write, buf = _writer(lla, H * d * r_k, "bf16")
+    g = torch.Generator(device=DEV).manual_seed(93)
+    rand = lambda *s: torch.randn(s, generator=g, device=DEV).to(torch.bfloat16)
+    geom = lla.Geometry(1, H, d, r_k, r_v)
+    codec = lla.Codec(None, None, buf, rand(H * d * r_v))
+    two_d = entry == "2d"
+    bb = (lla.lla_cache_2d_block_bytes if two_d else lla.lla_cache_block_bytes)(geom)
+    pool = rand(B * bb // 2)
+    cache = lla.Cache(pool, B, torch.arange(B, dtype=torch.int32, device=DEV).view(B, 1), 1)
+    lens = torch.full((B,), 60, dtype=torch.int32, device=DEV)
+    q = rand(1, B, H, d)
+    size = lla.lla_decode_2d_workspace_size if two_d else lla.lla_decode_loops_workspace_size
+    ws = torch.empty(size(geom, B), dtype=torch.uint8, device=DEV)
+
+    def decode(settle):
+        out = torch.empty_like(q)
+        write()
+        if settle:
+            torch.cuda.synchronize()
+        if two_d:
+            lla.lla_decode_attn_2d(geom, codec, cache, lens, 64, 0, q[0], None, None, out[0], ws)
+        else:
+            lla.lla_decode_attn_loops(geom, codec, cache, lens, 64, q, None, None, out, ws)
+        torch.cuda.synchronize()
+        return out
+
+    want = decode(True)
+    for _ in range(4):
+        assert torch.equal(decode(False), want)
+    assert lla.lla_get_device_error() == 0

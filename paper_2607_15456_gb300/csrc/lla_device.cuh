@@ -156,6 +156,31 @@ __device__ __forceinline__ float bf_to_f(uint16_t u) {
     return __uint_as_float(static_cast<uint32_t>(u) << 16);
 }
 
+// x - m of two bf16 pairs as hi + lo, exactly: hi the rounded difference, lo what the rounding left (the
+// error of a rounded sum of two numbers is a number of the same format: Knuth's two-sum).  Where hi is
+// infinite or NaN lo is zero.
+__device__ __forceinline__ void sub_exact_bf16x2(uint32_t x, uint32_t m, uint32_t &hi, uint32_t &lo) {
+    uint32_t b, e, ok;
+    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(hi) : "r"(x), "r"(m));
+    asm("{\n\t.reg .b32 t, u;\n\t"
+        "sub.rn.bf16x2 %0, %2, %3;\n\t"   // b = hi - x, what m took away
+        "sub.rn.bf16x2 t, %2, %0;\n\t"
+        "sub.rn.bf16x2 u, %3, t;\n\t"     // x - (hi - b)
+        "add.rn.bf16x2 t, %4, %0;\n\t"    // m + b
+        "sub.rn.bf16x2 %1, u, t;\n\t}"
+        : "=&r"(b), "=&r"(e)
+        : "r"(hi), "r"(x), "r"(m));
+    const __nv_bfloat162 ev = *reinterpret_cast<const __nv_bfloat162 *>(&e);
+    ok = __heq2_mask(ev, ev);  // 0xffff where e is a number
+    lo = e & ok;
+}
+
+// mu as a bf16 number, which x - mu is formed with, and what that leaves (zero where it is no number).
+__device__ __forceinline__ float bf16_rest(float mu) {
+    const float rest = mu - __bfloat162float(__float2bfloat16_rn(mu));
+    return rest == rest ? rest : 0.f;
+}
+
 // Loads element i of an array of `dtype` (LLA_BF16 / LLA_F32) as float.
 __device__ __forceinline__ float load_elem(const void *base, int64_t i, int is_bf16) {
     if (is_bf16) return bf_to_f(reinterpret_cast<const uint16_t *>(base)[i]);

@@ -13,15 +13,18 @@
 //     (2q, 2q + 1) and (2q + 8, 2q + 9) the rows 8q + 4s + {0, 1} and + {2, 3}, so the words of x
 //     are A registers as loaded, and two rows' words interleave (prmt) into B registers.  Column g
 //     of n-tile j is column 8g + j, so a lane ends with whole 8-column chunks of its tokens.
-//   * mu enters as three more rows of A, the bf16 parts of mu (24 significant bits): mu W_down, in
-//     accumulators of its own, is subtracted at the end.
+//   * with mu, x - m for the bf16 rounding m of mu is formed exactly as two bf16 parts, each an operand A,
+//     and the rest mu - m enters as two more rows of A (its 16 significant bits): (mu - m) W_down, in
+//     accumulators of its own, is subtracted at the end.  (x W_down - mu W_down instead, with mu in three
+//     parts, lost what the two large sums round off where mu is far above the spread of x: with mu 64
+//     times the spread thirty times as many latents were rounded the wrong way.)
 // No shared memory holds operands, so five CTAs fit an SM and about 80 KB of loads are in flight.
 // mma.sync and not tcgen05: with 16 tokens the products are 3 % of the tensor rate, and W_down rows
 // need no staging, no tensor maps (four per layer) and no TMEM.
 //
 // Measured (replayed from a graph, cold weights) against the kernels that took these calls before: 24
-// layers of 16 tokens at (96, 160) 90.5 -> 25.6 us (bytes: 17 us), with mu 113.6 -> 36 us, 64 tokens
-// 337 -> 73 us, 128 tokens 216 -> 134 us; 48 layers of 64 tokens at (72, 120) 584 -> 112 us; 48 layers
+// layers of 16 tokens at (96, 160) 90.5 -> 25.6 us (bytes: 17 us), with mu 113.6 -> 41 us, 64 tokens
+// 337 -> 73 us (with mu 420 -> 119), 128 tokens 216 -> 133 us (1738 -> 227); 48 layers of 64 tokens at (72, 120) 584 -> 112 us; 48 layers
 // of 128 tokens at (18, 30) 397 -> 90 us; one layer of 16 tokens at (96, 160) 7.3 -> 5.2 us.  What
 // bounds it: the latency of one block of W_down per warp at few tokens; the loads of x (16 bytes of a
 // token per lane, again for every 64 columns) at many, so that the prompt kernel takes over where
@@ -92,19 +95,23 @@ template <int MT, bool MU, int CW>
 struct Block {
     uint32_t w[8][Chunks<CW>::SLOTS * Chunks<CW>::WORDS];  // rows 8q .. 8q + 7
     uint4 x[2 * MT];      // tokens g, g + 8 (, g + 16, g + 24)
-    float4 m[MU ? 2 : 1]; // mu of the eight rows
+    float m[MU ? 8 : 1];  // mu of the eight rows
 };
 
 // Resident CTAs per SM the registers are held to.  One block of 32 rows in flight per warp and more
 // warps beat two blocks per warp: 24 layers of 16 tokens at (96, 160) take 25.3 us with five CTAs
 // and one block, 28.2 with four, 30.5 with three and two blocks each.  (64 tokens per CTA, which reads
 // W_down half as often as two CTAs of 32, was slower: 78.8 against 73.3 us for 64 tokens.)
-constexpr int step_ctas(int mt, bool mu) { return mt == 1 ? (mu ? 4 : 5) : 3; }
+// With mu: three and two CTAs, whose registers hold everything (one more each spilled: 24 layers of 16
+// tokens 40.7 and 45.4 us, of 64 tokens 119 and 133; mu - m as constant rows into the tokens' own
+// accumulators instead, 33.5 and 101 us, took four roundings per 16 rows where this takes two, and more
+// latents were rounded the wrong way than with fp32 sums).
+constexpr int step_ctas(int mt, bool mu) { return mt == 1 ? (mu ? 3 : 5) : (mu ? 2 : 3); }
 
 template <int MT, bool MU, int CW>
 __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kernel(const __grid_constant__ StepParams p) {
     using C = Chunks<CW>;
-    constexpr int ROWS = 16 * MT + (MU ? 3 : 0);
+    constexpr int ROWS = 16 * MT + (MU ? 2 : 0);
     constexpr int kRowF = C::COLS + 4;  // floats of a partial row (padded)
     __shared__ __align__(16) float red[kWarps][ROWS][kRowF];
     __shared__ float bias[64];
@@ -124,7 +131,6 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
     const char *x = static_cast<const char *>(axis ? L.x_v : L.x_k) + static_cast<int64_t>(h) * p.d * 2;
     const float *mu = axis ? L.mu_v : L.mu_k;
     const bool use_mu = MU && mu != nullptr;
-    const float row1 = g >= 1 ? 1.f : 0.f, row2 = g >= 2 ? 1.f : 0.f;
 
     Block<MT, MU, CW> blk;
     auto load_w = [&](Block<MT, MU, CW> &B, int b) {
@@ -142,12 +148,9 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
             }
         }
         if constexpr (MU) {
-            B.m[0] = B.m[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (use_mu && g < 3) {
-                const float *s = mu + static_cast<int64_t>(h) * Td + k;
-                B.m[0] = make_float4(s[0], s[1], s[2], s[3]);
-                B.m[1] = make_float4(s[4], s[5], s[6], s[7]);
-            }
+            const float *s = mu + static_cast<int64_t>(h) * Td + k;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) B.m[i] = use_mu ? s[i] : 0.f;
         }
     };
     auto load_x = [&](Block<MT, MU, CW> &B, int b) {
@@ -170,18 +173,31 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             uint32_t am[2] = {0u, 0u};
-            if constexpr (MU) {
-                // row g < 3 of the mu tile: eight of the 24 significant bits of mu at this step's four
-                // k (the upper half-word of what the rows before leave; both steps are exact)
-                const float4 m4 = B.m[s];
-                float v[4] = {m4.x, m4.y, m4.z, m4.w};
+            uint32_t xa[MT][4], xl[MU ? MT : 1][4];  // A of each m-tile: x, or hi and lo of x - m
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    v[i] = fmaf(-row1, __uint_as_float(__float_as_uint(v[i]) & 0xffff0000u), v[i]);
-                    v[i] = fmaf(-row2, __uint_as_float(__float_as_uint(v[i]) & 0xffff0000u), v[i]);
+            for (int m = 0; m < MT; ++m) {
+                const uint4 &u = B.x[2 * m], &v = B.x[2 * m + 1];
+                xa[m][0] = s ? u.z : u.x; xa[m][1] = s ? v.z : v.x; xa[m][2] = s ? u.w : u.y; xa[m][3] = s ? v.w : v.y;
+            }
+            if constexpr (MU) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float m0 = B.m[4 * s + 2 * i], m1 = B.m[4 * s + 2 * i + 1];
+                    const __nv_bfloat162 mb = __floats2bfloat162_rn(m0, m1);
+                    const uint32_t mh = *reinterpret_cast<const uint32_t *>(&mb);
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) {
+                        sub_exact_bf16x2(xa[m][2 * i], mh, xa[m][2 * i], xl[m][2 * i]);
+                        sub_exact_bf16x2(xa[m][2 * i + 1], mh, xa[m][2 * i + 1], xl[m][2 * i + 1]);
+                    }
+                    // rows 0 and 1 of the mu tile: the upper eight bits of mu - m, and the lower (exact)
+                    float r0 = g < 2 ? bf16_rest(m0) : 0.f, r1 = g < 2 ? bf16_rest(m1) : 0.f;
+                    if (g == 1) {
+                        r0 -= __uint_as_float(__float_as_uint(r0) & 0xffff0000u);
+                        r1 -= __uint_as_float(__float_as_uint(r1) & 0xffff0000u);
+                    }
+                    am[i] = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
                 }
-                am[0] = __byte_perm(__float_as_uint(v[0]), __float_as_uint(v[1]), 0x7632);
-                am[1] = __byte_perm(__float_as_uint(v[2]), __float_as_uint(v[3]), 0x7632);
             }
 #pragma unroll
             for (int j = 0; j < C::NT; ++j) {
@@ -190,8 +206,8 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
                 const uint32_t f1 = __byte_perm(B.w[4 * s + 2][j / 2], B.w[4 * s + 3][j / 2], sel);
 #pragma unroll
                 for (int m = 0; m < MT; ++m) {
-                    const uint4 &u = B.x[2 * m], &v = B.x[2 * m + 1];
-                    mma_bf16(acc[m][j], s ? u.z : u.x, s ? v.z : v.x, s ? u.w : u.y, s ? v.w : v.y, f0, f1);
+                    mma_bf16(acc[m][j], xa[m][0], xa[m][1], xa[m][2], xa[m][3], f0, f1);
+                    if constexpr (MU) mma_bf16(acc[m][j], xl[m][0], xl[m][1], xl[m][2], xl[m][3], f0, f1);
                 }
                 if constexpr (MU) mma_bf16(acc[MT][j], am[0], 0u, am[1], 0u, f0, f1);
             }
@@ -235,7 +251,7 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
         put(16 * m + 8 + g, acc[m], 1);
     }
     if constexpr (MU) {
-        if (g < 3) put(16 * MT + g, acc[MT], 0);
+        if (g < 2) put(16 * MT + g, acc[MT], 0);
     }
     __syncthreads();
     if constexpr (MU) {
@@ -244,7 +260,7 @@ __global__ void __launch_bounds__(kThreadsS, step_ctas(MT, MU)) encode_step_kern
 #pragma unroll
             for (int w = 0; w < kWarps; ++w)
 #pragma unroll
-                for (int i = 0; i < 3; ++i) v += red[w][16 * MT + i][tid];
+                for (int i = 0; i < 2; ++i) v += red[w][16 * MT + i][tid];
             bias[tid] = v;
         }
         __syncthreads();

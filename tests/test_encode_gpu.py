@@ -8,11 +8,12 @@ and bf16), ranks whose rows are not a multiple of 16 bytes (4-byte copies), toke
 leave a ragged last tile, x in bf16 and fp32, with and without mu, a decode-step batch, and
 prompts of 128 tokens or more in bf16, which take the tensor-core kernel.
 """
+import numpy as np
 import pytest
 import torch
 
 import oracle
-from helpers import assert_parity, ensure_library, f64, unpack_head
+from helpers import assert_parity, bf16_half_ulp, ensure_library, f64, unpack_head
 
 pytestmark = pytest.mark.gpu
 
@@ -165,3 +166,65 @@ def test_encode_step_tokens_and_rank_edges(lla, N, r_k, r_v, with_mu):
 def test_encode_step_reduction_lengths(lla, T, d):
     # fewer blocks of 32 rows than warps, blocks that do not divide by the warps, a long reduction
     _encode_and_compare(lla, T, 2, d, 40, 72, "bf16", "bf16", [21], True, 14)
+
+
+def _mu_far_above_the_spread(lla, H, d, r_k, r_v, N, two_d=False, T=4):
+    """Half of the stacked coordinates are channels whose mean is thousands of times the spread of the others,
+    and which tokens do not vary in: x - mu is zero there, so those channels may not cost precision.
+    Every latent is within its bf16 rounding of the 64-bit value, but for what a sum in 32 bits of the
+    products (x - mu) w rounds off: less than 2^-23 of the sum of their magnitudes per step of 16."""
+    g = torch.Generator(device=DEV).manual_seed(15)
+    rand = lambda *s: torch.randn(s, generator=g, device=DEV)
+    Hh, Td = (1, T * H * d) if two_d else (H, T * d)
+    geom = lla.Geometry(T, H, d, r_k, r_v)
+    pages = -(-N // 64)
+    bb = (lla.lla_cache_2d_block_bytes if two_d else lla.lla_cache_block_bytes)(geom)
+    pool = torch.zeros(pages * bb, dtype=torch.uint8, device=DEV)
+    x, mu, w = {}, {}, {}
+    for ax, r in (("k", r_k), ("v", r_v)):
+        big = rand(Hh, Td) > 0
+        mu[ax] = torch.where(big, rand(Hh, Td).to(torch.bfloat16).float() * 65536, 0.5 * rand(Hh, Td))
+        s = torch.where(big, mu[ax], 0.5 * rand(N, Hh, Td) + mu[ax]).to(torch.bfloat16)  # stacked x
+        x[ax] = (s.view(N, T, H, d).permute(1, 0, 2, 3) if two_d else s.view(N, H, T, d).permute(2, 0, 1, 3)).contiguous()
+        w[ax] = (rand(Hh, Td, r) * Td ** -0.5).to(torch.bfloat16)
+        y = s.double() - mu[ax].double()
+        x[ax + "64"] = torch.einsum("nhk,hkr->nhr", y, w[ax].double())
+        x[ax + "abs"] = torch.einsum("nhk,hkr->nhr", y.abs(), w[ax].double().abs())
+    sq = (lambda t: t[0].contiguous()) if two_d else (lambda t: t)
+    codec = lla.Codec(sq(w["k"]), sq(w["v"]), None, None, sq(mu["k"]), sq(mu["v"]))
+    (lla.lla_encode_2d if two_d else lla.lla_encode)(geom, codec, lla.Cache(pool, pages, None, 1), x["k"], x["v"],
+                                                      torch.arange(N, device=DEV))
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    pool_cpu, table = pool.cpu(), list(range(pages))
+    for h in range(Hh):
+        for ax, got in zip("kv", unpack_head(pool_cpu, Hh, r_k, r_v, "bf16", table, N, h)):
+            ref, mag = f64(x[ax + "64"][:, h]), f64(x[ax + "abs"][:, h])
+            dev = np.abs(got - ref) - bf16_half_ulp(ref)
+            assert (dev <= (Td / 16 + 8) * 2.0 ** -23 * mag).all(), (ax, h, (dev / mag).max() * 2 ** 23)
+
+
+@pytest.mark.parametrize("N,r_k,r_v", [(1, 96, 160), (16, 18, 30), (33, 72, 120), (64, 24, 70)])
+def test_encode_step_mu_far_above_the_spread(lla, N, r_k, r_v):
+    _mu_far_above_the_spread(lla, 2, 128, r_k, r_v, N)
+
+
+@pytest.mark.parametrize("N,r_k,r_v", [(16, 96, 160), (33, 18, 30)])
+def test_encode_step_infinite_input(lla, N, r_k, r_v):
+    """An infinite coordinate of one token makes its latents infinite with the sign of w, and no other token's."""
+    H, d, T = 2, 128, 2
+    g = torch.Generator(device=DEV).manual_seed(16)
+    rand = lambda *s: torch.randn(s, generator=g, device=DEV)
+    geom = lla.Geometry(T, H, d, r_k, r_v)
+    pages = -(-N // 64)
+    pool = torch.zeros(pages * lla.lla_cache_block_bytes(geom), dtype=torch.uint8, device=DEV)
+    w = [rand(H, T * d, r).to(torch.bfloat16) for r in (r_k, r_v)]
+    x = rand(T, N, H, d).to(torch.bfloat16)
+    x[1, 5, :, 7] = float("inf")
+    codec = lla.Codec(w[0], w[1], None, None, rand(H, T * d), rand(H, T * d))
+    lla.lla_encode(geom, codec, lla.Cache(pool, pages, None, 1), x, x, torch.arange(N, device=DEV))
+    pool_cpu = pool.cpu()
+    for h in range(H):
+        for wa, got in zip(w, unpack_head(pool_cpu, H, r_k, r_v, "bf16", list(range(pages)), N, h)):
+            assert np.isfinite(np.delete(got, 5, 0)).all()
+            assert (got[5] == np.sign(f64(wa[h, d + 7])) * np.inf).all()

@@ -160,19 +160,18 @@ __device__ __forceinline__ float bf_to_f(uint16_t u) {
 // error of a rounded sum of two numbers is a number of the same format: Knuth's two-sum).  Where hi is
 // infinite or NaN lo is zero.
 __device__ __forceinline__ void sub_exact_bf16x2(uint32_t x, uint32_t m, uint32_t &hi, uint32_t &lo) {
-    uint32_t b, e, ok;
+    uint32_t e;
     asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(hi) : "r"(x), "r"(m));
-    asm("{\n\t.reg .b32 t, u;\n\t"
-        "sub.rn.bf16x2 %0, %2, %3;\n\t"   // b = hi - x, what m took away
-        "sub.rn.bf16x2 t, %2, %0;\n\t"
-        "sub.rn.bf16x2 u, %3, t;\n\t"     // x - (hi - b)
-        "add.rn.bf16x2 t, %4, %0;\n\t"    // m + b
-        "sub.rn.bf16x2 %1, u, t;\n\t}"
-        : "=&r"(b), "=&r"(e)
+    asm("{\n\t.reg .b32 b, t, u;\n\t"
+        "sub.rn.bf16x2 b, %1, %2;\n\t"   // b = hi - x, what m took away
+        "sub.rn.bf16x2 t, %1, b;\n\t"
+        "sub.rn.bf16x2 u, %2, t;\n\t"    // x - (hi - b)
+        "add.rn.bf16x2 t, %3, b;\n\t"    // m + b
+        "sub.rn.bf16x2 %0, u, t;\n\t}"
+        : "=r"(e)
         : "r"(hi), "r"(x), "r"(m));
     const __nv_bfloat162 ev = *reinterpret_cast<const __nv_bfloat162 *>(&e);
-    ok = __heq2_mask(ev, ev);  // 0xffff where e is a number
-    lo = e & ok;
+    lo = e & __heq2_mask(ev, ev);  // 0xffff where e is a number
 }
 
 // mu as a bf16 number, which x - mu is formed with, and what that leaves (zero where it is no number).

@@ -2,14 +2,14 @@
 // persistent launch.
 //
 // A unit is (head h, tile of 128 tokens, column group g of one axis):
-//   C[128 x R] = X[128 x T*d] W_down[T*d x R] - mu W_down,
+//   C[128 x R] = (X - m)[128 x T*d] W_down[T*d x R] - (mu - m) W_down,   m: mu rounded to bf16
 // with X the stacked loop vectors of the tile's tokens (row n, column t*d + e = x_t[n][h][e]).
 // LLA-2D is the case of one head of width H*d.  An axis of rank r is cut into ceil(r / 192) column
 // groups of equal width (a multiple of 16; the columns of the last group past r read as zeros and
 // are not stored).  Units are numbered head-major, then tile, then group (K groups first): one CTA
 // per SM takes an equal contiguous range of them, so the groups of a tile follow one another on the
 // same SM and the second read of a tile's x_v hits L2, and a CTA meets few heads (the bias
-// mu W_down of a group is computed once per head the CTA meets).  bf16 operands, fp32 accumulation
+// (mu - m) W_down of a group is computed once per head the CTA meets).  bf16 operands, fp32 accumulation
 // in TMEM, latents rounded to bf16 and scattered to each token's slot.  Warp roles:
 //   warp 0     x producer: per slab of 64 reduction rows, a TMA tensor load with 128-byte swizzle
 //              of the x tile (one box of 128 tokens x 64 elements: a K-major operand) into its
@@ -22,6 +22,10 @@
 //              two accumulator slots, so a unit's epilogue overlaps the next unit's products
 //   warps 2-5  epilogue: one token row per thread, TMEM -> bias -> bf16 -> the paged cache (V-plane
 //              rows pass through a per-warp staging buffer, so a store writes 8 rows of 64 bytes)
+//   warps 7-10 (with mu only) x - m of a slab, exactly, as two bf16 parts in TMEM (one token row per
+//              thread), two slabs deep: the products then take their operand A from there.  x W_down -
+//              mu W_down instead lost what the two large sums round off where mu is far above the spread
+//              of x (mu 64 times the spread: 1.2 % of the latents rounded the wrong way, here 0.007 %)
 // Tokens past N read as zeros (tensor-map fill) and are not stored.
 //
 // Few units with a long reduction (LLA-2D prompts: T*H*d = 8192 rows, N/128 tiles) are split over
@@ -36,10 +40,10 @@
 //
 // Bound: HBM for per-head prompts (x is read once; 41.7 us of bytes for 7208 tokens at (72, 120)),
 // the L2 -> shared memory stream for LLA-2D (a 128 x 192 unit moves 40 KB per 64 rows).  Measured
-// against the CUDA-core kernel, which these shapes took before: 7208 tokens at (72, 120) with mu
-// 1690 -> 60.6 us; 8000 tokens at (18, 30) 516 -> 62 us (150 tokens: 17.4 -> 7.9 us); LLA-2D
-// (288, 480), 1500 tokens 4864 -> 32 us, 16 tokens 63 -> 16 us; and the bias in slices, 8000 tokens
-// at (96, 160) with mu 188 -> 73 us (63 us without).
+// against the CUDA-core kernel, which these shapes took before: 7208 tokens at (72, 120) 1352 -> 52 us,
+// with mu 1690 -> 78 us; 8000 tokens at (18, 30) 516 -> 62 us, with mu 593 -> 85 us (150 tokens 19.7 ->
+// 7.6 us); LLA-2D (288, 480), 1500 tokens 4862 -> 30 us, with mu 5028 -> 64 us.  8000 tokens at (96, 160),
+// here before too: 62 -> 59 us, with mu 191 -> 89 us (the bias in slices; x - m two slabs at a time).
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -52,7 +56,7 @@ namespace {
 
 constexpr int kEM = 128;             // tokens per tile
 constexpr int kES = 64;              // reduction rows per slab
-constexpr int kEThreads = 224;
+constexpr int kEThreads = 224;       // and with mu four more warps
 constexpr int kMaxGroup = 192;       // columns of a group
 constexpr int kMaxGroups = 20;       // groups of both axes (LLA-2D (1152, 1920): 6 + 10)
 constexpr int kMaxSplit = 8;         // CTAs that share one unit's reduction
@@ -62,23 +66,27 @@ constexpr int kResSlabs = 8;         // WRES: most slabs (T*d = 512 rows) kept r
 constexpr int kASlab = kEM * kES * 2;   // x slab (16 KB)
 constexpr int kBAtom = kES * 128;       // one W_down atom of 64 columns (8 KB)
 constexpr int kWStage = 3 * kBAtom;          // 24 KB
-constexpr int kXStages = 5;                 // x slabs in flight (from HBM)
 constexpr int kWStages = 5;                 // W_down slabs in flight (from L2)
-constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kSlotCols = 256;  // accumulator slot s at column s * 256
-constexpr int oW = kXStages * kASlab;
-template <bool WRES>
-struct EL {  // shared-memory plan: x ring, W_down (ring or resident), biases, V staging, barriers
+constexpr uint32_t kTmemCols = 512, kAT = 2 * kMaxGroup;
+template <bool WRES, bool MU>
+struct EL {  // shared-memory plan: x ring, W_down (ring or resident), biases, V staging, mu, barriers
+    static constexpr int THREADS = kEThreads + (MU ? 128 : 0);
+    static constexpr int XST = MU ? 4 : 5;           // x slabs in flight (from HBM)
+    // TMEM: accumulator slot s at s * SLOT; with mu two buffers of x - m as operand A (hi, then lo, 32
+    // columns each) at kAT
+    static constexpr uint32_t SLOT = MU ? kMaxGroup : 256;
+    static constexpr int oW = XST * kASlab;
     static constexpr int GROUPS = WRES ? 2 : kMaxGroups;
     static constexpr int oBias = oW + (WRES ? 2 * kResSlabs * kBAtom : kWStages * kWStage);
     static constexpr int oStg = oBias + GROUPS * kMaxGroup * 4;  // 4 warps x 32 rows x 80 B
-    static constexpr int oBar = oStg + 4 * 32 * 80;
-    static constexpr int NBAR = 2 * kXStages + 2 * kWStages + 4 + 1;
+    static constexpr int oMu = oStg + 4 * 32 * 80;               // 4 warps x 2 buffers x 64 bf16
+    static constexpr int oBar = oMu + (MU ? 4 * 2 * 128 : 0);
+    static constexpr int NBAR = 2 * XST + 2 * kWStages + 4 + 1 + (MU ? 4 : 0);
     static constexpr int SMEM = 1024 + oBar + NBAR * 8 + 16;  // + alignment slack, abort flag, TMEM slot
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 // split units: parts of one column range, [rank][column / 4][row] float4 (over the idle rings)
-static_assert(kMaxSplit * kEM * 32 * 4 <= EL<false>::oBias && 2 * kEM * 96 * 4 <= EL<false>::oBias, "exchange area");
+static_assert(kMaxSplit * kEM * 32 * 4 <= EL<false, true>::oBias && 2 * kEM * 96 * 4 <= EL<false, true>::oBias, "exchange area");
 
 struct ETParams {
     int T, H, d, N;
@@ -136,7 +144,7 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t local_addr, uint32_t rank
         : "memory");
 }
 
-// mu W_down over reduction rows [k0, k1) for the columns of unit U, into bs[0 .. cols): EPL columns
+// (mu - m) W_down over reduction rows [k0, k1) for the columns of unit U, into bs[0 .. cols): EPL columns
 // (8, or 2 when the rows of W_down are not whole 16-byte words) per thread and the rows cut into as
 // many slices as the 128 epilogue threads allow, sixteen rows' loads in flight each (one thread per
 // eight columns over all rows took tens of microseconds).  scr: at least 128 * EPL floats.
@@ -153,7 +161,7 @@ __device__ void group_bias(const uint16_t *W, const float *mu, int r, const Unit
         const uint16_t *Wc = W + U.col0 + ch * EPL;
 #pragma unroll 16
         for (int k = k0 + sl; k < k1; k += nsl) {
-            const float mk = mu[k];
+            const float mk = bf16_rest(mu[k]);
             uint32_t w[EPL / 2];
             if constexpr (EPL == 8) {
                 const uint4 q = *reinterpret_cast<const uint4 *>(Wc + static_cast<int64_t>(k) * r);
@@ -198,25 +206,28 @@ __device__ __forceinline__ char *row_dst(const ETParams &p, const Unit &U, int r
     return U.axis == 0 ? page + r_in * p.gran : page + p.kplane_bytes + static_cast<int64_t>(r_in) * p.r_v * 2;
 }
 
-template <bool WRES>
-__global__ void __launch_bounds__(kEThreads, 1)
+template <bool WRES, bool MU>
+__global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
     encode_tc_kernel(const __grid_constant__ CUtensorMap txk, const __grid_constant__ CUtensorMap txv,
                      const __grid_constant__ CUtensorMap twk, const __grid_constant__ CUtensorMap twv,
                      const ETParams p) {
-    using L = EL<WRES>;
+    using L = EL<WRES, MU>;
+    constexpr int oW = L::oW;
     extern __shared__ __align__(1024) char sm_raw[];
     // 128-byte swizzle atoms need a 1024-byte aligned base
     char *sm = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float *bias = reinterpret_cast<float *>(sm + L::oBias);  // [group][192] of the current head
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + L::oBar);
-    uint64_t *empty = full + kXStages;
-    uint64_t *wfull = empty + kXStages;
+    uint64_t *empty = full + L::XST;
+    uint64_t *wfull = empty + L::XST;
     uint64_t *wempty = wfull + kWStages;
     uint64_t *accfull = wempty + kWStages;  // [2]
     uint64_t *accempty = accfull + 2;     // [2]
     uint64_t *done = accempty + 2;
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(done + 1);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(done + 1) + 1;
+    uint64_t *afull = done + 1, *aempty = afull + 2;  // MU: [2] each
+    uint64_t *after = full + L::NBAR;
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(after);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(after) + 1;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool split = p.split > 1;
     const int64_t u0 = split ? blockIdx.x / p.split : static_cast<int64_t>(blockIdx.x) * p.units / gridDim.x;
@@ -228,9 +239,9 @@ __global__ void __launch_bounds__(kEThreads, 1)
     const int NS = S1 - S0;
 
     if (tid == 0) {
-        for (int s = 0; s < kXStages; ++s) {
+        for (int s = 0; s < L::XST; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&empty[s], MU ? 4 : 1);  // the converting warps, or the products
         }
         for (int s = 0; s < kWStages; ++s) {
             mbar_init(&wfull[s], WRES ? 128 : 1);  // resident: the epilogue warps' copy (one per axis)
@@ -241,12 +252,18 @@ __global__ void __launch_bounds__(kEThreads, 1)
             mbar_init(&accempty[s], 4);  // one arrival per epilogue warp
         }
         mbar_init(done, 1);
+        if constexpr (MU) {
+            for (int s = 0; s < 2; ++s) {
+                mbar_init(&afull[s], 4);
+                mbar_init(&aempty[s], 1);
+            }
+        }
         *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tslot, kTmemCols);
     if constexpr (WRES) {  // the padding columns of the resident W_down
-        for (int i = tid; i < 2 * kResSlabs * kBAtom / 16; i += kEThreads)
+        for (int i = tid; i < 2 * kResSlabs * kBAtom / 16; i += L::THREADS)
             reinterpret_cast<uint4 *>(sm + oW)[i] = make_uint4(0, 0, 0, 0);
     }
     tc_fence_before();
@@ -258,7 +275,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
     if (warp == 0 || (warp == 6 && !WRES)) {
         // ------------------------------------------------------------ producers: x (0), W (6)
         const bool isx = warp == 0;
-        const int NST = isx ? kXStages : kWStages;
+        const int NST = isx ? L::XST : kWStages;
         uint64_t *F = isx ? full : wfull;
         uint64_t *E = isx ? empty : wempty;
         int q = 0;  // slabs issued
@@ -319,23 +336,34 @@ __global__ void __launch_bounds__(kEThreads, 1)
                 // the epilogue has read this slot's previous unit (j - 2)
                 if (!mbar_wait_warp(&accempty[slot], ((j >> 1) & 1) ^ 1u, abort_flag, p.err)) break;
                 tc_fence_after();
-                const uint32_t d = tmem + slot * kSlotCols;
+                const uint32_t d = tmem + slot * L::SLOT;
                 bool ok = true;
 #pragma unroll 1
                 for (int s = 0; s < NS; ++s, ++q) {
-                    const int st = q % kXStages, sw = q % kWStages;
-                    if (!mbar_wait_warp(&full[st], (q / kXStages) & 1, abort_flag, p.err) ||
+                    const int st = q % L::XST, sw = q % kWStages;
+                    if (!(MU ? mbar_wait_warp(&afull[q & 1], (q >> 1) & 1, abort_flag, p.err)
+                             : mbar_wait_warp(&full[st], (q / L::XST) & 1, abort_flag, p.err)) ||
                         (!WRES && !mbar_wait_warp(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err))) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                     const uint32_t a = base + st * kASlab, b = base + oW + (WRES ? (U.axis * kResSlabs + s) * kBAtom : sw * kWStage);
+                    if constexpr (MU) {
 #pragma unroll
-                    for (int ks = 0; ks < kES / 16; ++ks)
-                        umma_bf16_warp(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
-                                  idesc, s > 0 || ks > 0);
-                    umma_commit_warp(&empty[st]);
+                        for (int part = 0; part < 2; ++part)
+#pragma unroll
+                            for (int ks = 0; ks < kES / 16; ++ks)
+                                umma_bf16_ts_warp(d, tmem + kAT + (q & 1) * 64 + part * 32 + ks * 8,
+                                                  umma_desc_sw128_mn(b + ks * 2048, kBAtom), idesc, s > 0 || part > 0 || ks > 0);
+                        umma_commit_warp(&aempty[q & 1]);
+                    } else {
+#pragma unroll
+                        for (int ks = 0; ks < kES / 16; ++ks)
+                            umma_bf16_warp(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
+                                           idesc, s > 0 || ks > 0);
+                        umma_commit_warp(&empty[st]);
+                    }
                     if (!WRES) umma_commit_warp(&wempty[sw]);
                 }
                 if (!ok) break;
@@ -399,7 +427,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
             char *stg = sm + L::oStg + quarter * (32 * 80);
             float *bs = bias + U.g * kMaxGroup;
             const float *mu = U.axis ? p.mu_v : p.mu_k;
-            if (mu && !(have >> U.g & 1u)) {
+            if (MU && mu && !(have >> U.g & 1u)) {
                 have |= 1u << U.g;
                 const int r = U.axis ? p.r_v : p.r_k;
                 const uint16_t *W = static_cast<const uint16_t *>(U.axis ? p.w_down_v : p.w_down_k) +
@@ -407,12 +435,12 @@ __global__ void __launch_bounds__(kEThreads, 1)
                 group_bias<WRES ? 2 : 8>(W, mu + static_cast<int64_t>(U.h) * Td, r, U, S0 * kES, S1 * kES, et,
                                          reinterpret_cast<float *>(sm + L::oStg), bs);
             }
-            const bool use_bias = mu != nullptr;
+            const bool use_bias = MU && mu != nullptr;
             if (split) break;  // the parts meet below
             char *dst = row_dst(p, U, row, U.g == 0);
             mbar_wait(&accfull[slot], (j >> 1) & 1, abort_flag, p.err);
             tc_fence_after();
-            const uint32_t tl = tmem + slot * kSlotCols + (static_cast<uint32_t>(quarter * 32) << 16);
+            const uint32_t tl = tmem + slot * L::SLOT + (static_cast<uint32_t>(quarter * 32) << 16);
 #pragma unroll 1
             for (int c0 = 0; c0 < U.cols; c0 += 32) {
                 float v[32];
@@ -499,6 +527,61 @@ __global__ void __launch_bounds__(kEThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&accempty[slot]);
         }
+    } else if (MU && warp >= 7) {
+        // ------------------------------------------------------- x - m into TMEM (one row per thread)
+        const int quarter = warp & 3, row = quarter * 32 + lane;
+        uint32_t *mws = reinterpret_cast<uint32_t *>(sm + L::oMu) + quarter * 64;  // [2][32] pairs of m
+        const uint32_t ta = tmem + kAT + (static_cast<uint32_t>(quarter * 32) << 16);
+        int q = 0;
+        bool stop = false;
+        for (int64_t u = u0; u < u1 && !stop; ++u) {
+            const Unit U = unit_of(p, u);
+            const float *mu = U.axis ? p.mu_v : p.mu_k;
+            if (mu) mu += static_cast<int64_t>(U.h) * Td + S0 * kES + 2 * lane;
+            float m0 = mu ? mu[0] : 0.f, m1 = mu ? mu[1] : 0.f;  // of the slab to come
+            for (int s = 0; s < NS; ++s, ++q) {
+                const int st = q % L::XST, buf = q & 1;
+                mws[buf * 32 + lane] = pack_bf16(m0, m1);
+                if (mu && s + 1 < NS) {
+                    m0 = mu[(s + 1) * kES];
+                    m1 = mu[(s + 1) * kES + 1];
+                }
+                __syncwarp();
+                if (!mbar_wait_warp(&full[st], (q / L::XST) & 1, abort_flag, p.err)) {
+                    stop = true;
+                    break;
+                }
+                const char *xr = sm + st * kASlab + row * 128;
+                uint32_t hi[32], lo[32];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(xr + ((c ^ (row & 7)) << 4));
+                    hi[4 * c] = x.x; hi[4 * c + 1] = x.y; hi[4 * c + 2] = x.z; hi[4 * c + 3] = x.w;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[st]);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 m = *reinterpret_cast<const uint4 *>(mws + buf * 32 + 4 * c);
+                    sub_exact_bf16x2(hi[4 * c], m.x, hi[4 * c], lo[4 * c]);
+                    sub_exact_bf16x2(hi[4 * c + 1], m.y, hi[4 * c + 1], lo[4 * c + 1]);
+                    sub_exact_bf16x2(hi[4 * c + 2], m.z, hi[4 * c + 2], lo[4 * c + 2]);
+                    sub_exact_bf16x2(hi[4 * c + 3], m.w, hi[4 * c + 3], lo[4 * c + 3]);
+                }
+                // the products of two slabs ago have read this buffer
+                if (!mbar_wait_warp(&aempty[buf], ((q >> 1) & 1) ^ 1u, abort_flag, p.err)) {
+                    stop = true;
+                    break;
+                }
+                tc_fence_after();
+                tmem_st32u_nowait(ta + buf * 64, hi);
+                tmem_st32u_nowait(ta + buf * 64 + 32, lo);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&afull[buf]);
+            }
+        }
     }
     pdl_trigger();
     if (split) {
@@ -510,7 +593,7 @@ __global__ void __launch_bounds__(kEThreads, 1)
         const bool ep = warp >= 2 && warp <= 5;
         const int quarter = warp & 3, row = quarter * 32 + lane;
         const float *bs = bias + U.g * kMaxGroup;
-        const bool use_bias = (U.axis ? p.mu_v : p.mu_k) != nullptr;
+        const bool use_bias = MU && (U.axis ? p.mu_v : p.mu_k) != nullptr;
         if (ep) {
             mbar_wait(&accfull[0], 0, abort_flag, p.err);
             tc_fence_after();
@@ -597,16 +680,16 @@ int groups_of_32(int r) {
 bool wide_rows(const EncodeArgs &a) { return a.r_k % 8 == 0 && a.r_v % 8 == 0; }
 bool fits_resident(const EncodeArgs &a) { return a.r_k <= 64 && a.r_v <= 64 && a.T * a.d <= kResSlabs * kES; }
 
-template <bool WRES>
+template <bool WRES, bool MU>
 lla_status launch_tc(const EncodeArgs &a, const ETParams &p, int grid, cudaStream_t stream) {
     CUtensorMap txk, txv, twk, twv;
     if (!make_maps(a, 0, WRES, &txk, &twk) || !make_maps(a, 1, WRES, &txv, &twv)) return LLA_ERR_CUDA;
     static DeviceOnce configured;
-    if (raise_smem_limit(encode_tc_kernel<WRES>, EL<WRES>::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
+    if (raise_smem_limit(encode_tc_kernel<WRES, MU>, EL<WRES, MU>::SMEM, configured) != LLA_OK) return LLA_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
-    cfg.blockDim = dim3(kEThreads);
-    cfg.dynamicSmemBytes = EL<WRES>::SMEM;
+    cfg.blockDim = dim3(EL<WRES, MU>::THREADS);
+    cfg.dynamicSmemBytes = EL<WRES, MU>::SMEM;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -617,7 +700,7 @@ lla_status launch_tc(const EncodeArgs &a, const ETParams &p, int grid, cudaStrea
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.split > 1 ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, encode_tc_kernel<WRES>, txk, txv, twk, twv, p) != cudaSuccess) return LLA_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, encode_tc_kernel<WRES, MU>, txk, txv, twk, twv, p) != cudaSuccess) return LLA_ERR_CUDA;
     return LLA_OK;
 }
 
@@ -662,7 +745,9 @@ lla_status launch_encode_tc(const EncodeArgs &a, cudaStream_t stream) {
     const int slabs = a.T * a.d / kES;
     while (wide_rows(a) && p.split < kMaxSplit && p.units * p.split * 2 <= sms && slabs / (p.split * 2) >= 8) p.split *= 2;
     const int grid = static_cast<int>(p.split > 1 ? p.units * p.split : p.units < sms ? p.units : sms);
-    return wide_rows(a) ? launch_tc<false>(a, p, grid, stream) : launch_tc<true>(a, p, grid, stream);
+    if (a.mu_k || a.mu_v)
+        return wide_rows(a) ? launch_tc<false, true>(a, p, grid, stream) : launch_tc<true, true>(a, p, grid, stream);
+    return wide_rows(a) ? launch_tc<false, false>(a, p, grid, stream) : launch_tc<true, false>(a, p, grid, stream);
 }
 
 }  // namespace lla

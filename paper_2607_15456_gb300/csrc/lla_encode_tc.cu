@@ -14,18 +14,24 @@
 //   warp 0     x producer: per slab of 64 reduction rows, a TMA tensor load with 128-byte swizzle
 //              of the x tile (one box of 128 tokens x 64 elements: a K-major operand) into its
 //              own ring, which runs on across units
-//   warp 6     W producer: the slab's W_down (boxes of 64 rows x 64 columns: an MN-major
+//   warp 2     W producer: the slab's W_down (boxes of 64 rows x 64 columns: an MN-major
 //              operand) into a second ring; the two rings let the x stream from HBM run ahead
 //              of the W_down stream from L2 (one shared ring of 40 KB stages gave x only 16 of
 //              every 40 bytes in flight)
 //   warp 1     MMA issuer and TMEM owner: 4 MMAs (K = 16) per slab, M = 128, N = R, into one of
-//              two accumulator slots, so a unit's epilogue overlaps the next unit's products
-//   warps 2-5  epilogue: one token row per thread, TMEM -> bias -> bf16 -> the paged cache (V-plane
-//              rows pass through a per-warp staging buffer, so a store writes 8 rows of 64 bytes)
-//   warps 7-10 (with mu only) x - m of a slab, exactly, as two bf16 parts in TMEM (one token row per
-//              thread), two slabs deep: the products then take their operand A from there.  x W_down -
-//              mu W_down instead lost what the two large sums round off where mu is far above the spread
-//              of x (mu 64 times the spread: 1.2 % of the latents rounded the wrong way, here 0.007 %)
+//              two accumulator slots; the next piece of four slabs takes the other
+//   warps 3-10 epilogue: each piece's accumulators are added to the unit's sum, in registers (one token
+//              row and every other chunk of 32 columns per thread); then bias -> bf16 -> the paged cache
+//              (V-plane rows pass through a per-warp staging buffer, so a store writes 8 rows of 64
+//              bytes).  Sums inside the tensor core are cut off, not rounded: over 512 rows and more
+//              they lost up to six times what fp32 sums lose (latents rounded the wrong way, LLA-2D
+//              (1152, 1920): 2.5e-3 in chains of 4096 rows, 2.0e-4 in pieces, 3.9e-4 on the CUDA cores).
+//              Pieces of two slabs, 9.5e-5 and not 1.5e-4 at (72, 120), cost (96, 160) 4 % and LLA-2D 10 %
+//   warps 11-14 (with mu only) x - m of a slab, exactly, as two bf16 parts in TMEM (one token row per
+//              thread), two slabs deep: the products then take their operand A from there, twice as many,
+//              so that a piece is two slabs.  x W_down - mu W_down instead lost what the two large sums
+//              round off where mu is far above the spread of x (mu 64 times the spread: 1.2 % of the
+//              latents rounded the wrong way, here 0.005 %)
 // Tokens past N read as zeros (tensor-map fill) and are not stored.
 //
 // Few units with a long reduction (LLA-2D prompts: T*H*d = 8192 rows, N/128 tiles) are split over
@@ -40,10 +46,11 @@
 //
 // Bound: HBM for per-head prompts (x is read once; 41.7 us of bytes for 7208 tokens at (72, 120)),
 // the L2 -> shared memory stream for LLA-2D (a 128 x 192 unit moves 40 KB per 64 rows).  Measured
-// against the CUDA-core kernel, which these shapes took before: 7208 tokens at (72, 120) 1352 -> 52 us,
-// with mu 1690 -> 78 us; 8000 tokens at (18, 30) 516 -> 62 us, with mu 593 -> 85 us (150 tokens 19.7 ->
-// 7.6 us); LLA-2D (288, 480), 1500 tokens 4862 -> 30 us, with mu 5028 -> 64 us.  8000 tokens at (96, 160),
-// here before too: 62 -> 59 us, with mu 191 -> 89 us (the bias in slices; x - m two slabs at a time).
+// against the CUDA-core kernel, which these shapes took before: 7208 tokens at (72, 120) 1352 -> 53 us,
+// with mu 1690 -> 85 us; 8000 tokens at (18, 30) 516 -> 61 us, with mu 593 -> 92 us (150 tokens 19.7 ->
+// 7.6 us); LLA-2D (288, 480), 1500 tokens 4862 -> 30 us, with mu 5028 -> 82 us.  8000 tokens at (96, 160),
+// here before too: 62 -> 60 us, with mu 191 -> 99 us.  With mu the chain of one slab through a converting
+// warp (about 1500 cycles, from its landing to its products) is the bound.
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"
@@ -56,7 +63,9 @@ namespace {
 
 constexpr int kEM = 128;             // tokens per tile
 constexpr int kES = 64;              // reduction rows per slab
-constexpr int kEThreads = 224;       // and with mu four more warps
+constexpr int kEpi0 = 3;              // x producer, MMA issuer, W producer, then eight epilogue warps
+constexpr int kEpi = 256;
+constexpr int kConv0 = kEpi0 + kEpi / 32;  // and with mu four converting warps
 constexpr int kMaxGroup = 192;       // columns of a group
 constexpr int kMaxGroups = 20;       // groups of both axes (LLA-2D (1152, 1920): 6 + 10)
 constexpr int kMaxSplit = 8;         // CTAs that share one unit's reduction
@@ -70,16 +79,19 @@ constexpr int kWStages = 5;                 // W_down slabs in flight (from L2)
 constexpr uint32_t kTmemCols = 512, kAT = 2 * kMaxGroup;
 template <bool WRES, bool MU>
 struct EL {  // shared-memory plan: x ring, W_down (ring or resident), biases, V staging, mu, barriers
-    static constexpr int THREADS = kEThreads + (MU ? 128 : 0);
-    static constexpr int XST = MU ? 4 : 5;           // x slabs in flight (from HBM)
+    static constexpr int THREADS = kConv0 * 32 + (MU ? 128 : 0);
+    // slabs whose products add up in TMEM (16 sums there either way) before fp32 adds in registers
+    static constexpr int PIECE = MU ? 2 : 4;
+    static constexpr int XST = MU || WRES ? 4 : 5;          // x slabs in flight (from HBM)
     // TMEM: accumulator slot s at s * SLOT; with mu two buffers of x - m as operand A (hi, then lo, 32
     // columns each) at kAT
     static constexpr uint32_t SLOT = MU ? kMaxGroup : 256;
     static constexpr int oW = XST * kASlab;
-    static constexpr int GROUPS = WRES ? 2 : kMaxGroups;
+    static constexpr int GROUPS = !MU ? 0 : WRES ? 2 : kMaxGroups;
+    static constexpr int NC = WRES ? 1 : 3;  // chunks of 32 columns of an epilogue warp
     static constexpr int oBias = oW + (WRES ? 2 * kResSlabs * kBAtom : kWStages * kWStage);
-    static constexpr int oStg = oBias + GROUPS * kMaxGroup * 4;  // 4 warps x 32 rows x 80 B
-    static constexpr int oMu = oStg + 4 * 32 * 80;               // 4 warps x 2 buffers x 64 bf16
+    static constexpr int oStg = oBias + GROUPS * kMaxGroup * 4;  // 8 warps x 32 rows x 80 B
+    static constexpr int oMu = oStg + 8 * 32 * 80;               // 4 warps x 2 buffers x 64 bf16
     static constexpr int oBar = oMu + (MU ? 4 * 2 * 128 : 0);
     static constexpr int NBAR = 2 * XST + 2 * kWStages + 4 + 1 + (MU ? 4 : 0);
     static constexpr int SMEM = 1024 + oBar + NBAR * 8 + 16;  // + alignment slack, abort flag, TMEM slot
@@ -146,20 +158,20 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t local_addr, uint32_t rank
 
 // (mu - m) W_down over reduction rows [k0, k1) for the columns of unit U, into bs[0 .. cols): EPL columns
 // (8, or 2 when the rows of W_down are not whole 16-byte words) per thread and the rows cut into as
-// many slices as the 128 epilogue threads allow, sixteen rows' loads in flight each (one thread per
-// eight columns over all rows took tens of microseconds).  scr: at least 128 * EPL floats.
+// many slices as the 256 epilogue threads allow, eight rows' loads in flight each (one thread per
+// eight columns over all rows took tens of microseconds).  scr: at least 256 * EPL floats.
 template <int EPL>
 __device__ void group_bias(const uint16_t *W, const float *mu, int r, const Unit &U, int k0, int k1, int et,
                            float *scr, float *bs) {
     const int nch = (U.cols + EPL - 1) / EPL;  // at most 24 (EPL = 8), 32 (EPL = 2)
-    const int nsl = 128 / nch;
+    const int nsl = kEpi / nch;
     const int ch = et % nch, sl = et / nch;
     float acc[EPL];
 #pragma unroll
     for (int i = 0; i < EPL; ++i) acc[i] = 0.f;
     if (sl < nsl) {
         const uint16_t *Wc = W + U.col0 + ch * EPL;
-#pragma unroll 16
+#pragma unroll 8
         for (int k = k0 + sl; k < k1; k += nsl) {
             const float mk = bf16_rest(mu[k]);
             uint32_t w[EPL / 2];
@@ -177,16 +189,16 @@ __device__ void group_bias(const uint16_t *W, const float *mu, int r, const Unit
             }
         }
     }
-    named_bar_sync(1, 128);  // scr and bs are free
+    named_bar_sync(1, kEpi);  // scr and bs are free
 #pragma unroll
     for (int i = 0; i < EPL; ++i) scr[et * EPL + i] = acc[i];
-    named_bar_sync(1, 128);
-    for (int c = et; c < U.cols; c += 128) {
+    named_bar_sync(1, kEpi);
+    for (int c = et; c < U.cols; c += kEpi) {
         float v = 0.f;
         for (int q = 0; q < nsl; ++q) v += scr[(q * nch + c / EPL) * EPL + c % EPL];
         bs[c] = v;
     }
-    named_bar_sync(1, 128);
+    named_bar_sync(1, kEpi);
 }
 
 // Where token row `row` of unit U goes: its K-plane row or V-plane row in the page of its slot (NULL:
@@ -244,12 +256,12 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
             mbar_init(&empty[s], MU ? 4 : 1);  // the converting warps, or the products
         }
         for (int s = 0; s < kWStages; ++s) {
-            mbar_init(&wfull[s], WRES ? 128 : 1);  // resident: the epilogue warps' copy (one per axis)
+            mbar_init(&wfull[s], WRES ? kEpi : 1);  // resident: the epilogue warps' copy (one per axis)
             mbar_init(&wempty[s], 1);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(&accfull[s], 1);
-            mbar_init(&accempty[s], 4);  // one arrival per epilogue warp
+            mbar_init(&accempty[s], 8);  // one arrival per epilogue warp
         }
         mbar_init(done, 1);
         if constexpr (MU) {
@@ -270,10 +282,13 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
     __syncthreads();
     tc_fence_after();
     constexpr uint32_t tmem = 0;  // all of TMEM is allocated; a constant keeps the issuing warp's code uniform
+    // epilogue: token row `row` of the tile, and of its columns the even or the odd chunks of 32
+    const int wt = tid - kEpi0 * 32, half = (warp - kEpi0) >> 2, quarter = warp & 3, row = quarter * 32 + lane;
+    float sum[L::NC][32];
     pdl_wait();  // x, slots and the pool may come from the previous kernel
 
-    if (warp == 0 || (warp == 6 && !WRES)) {
-        // ------------------------------------------------------------ producers: x (0), W (6)
+    if (warp == 0 || (warp == 2 && !WRES)) {
+        // ------------------------------------------------------------ producers: x (0), W (2)
         const bool isx = warp == 0;
         const int NST = isx ? L::XST : kWStages;
         uint64_t *F = isx ? full : wfull;
@@ -316,10 +331,11 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
         // ------------------------------------------------------------------------ MMA issuer
         {
             const uint32_t base = smem_addr(sm);
-            int q = 0, j = 0, head = -1;
+            int q = 0, head = -1;
+            uint32_t piece = 0;
             int nres[2] = {0, 0};               // WRES: copies of each axis's W_down seen
             bool wax[2] = {false, false};
-            for (int64_t u = u0; u < u1; ++u, ++j) {
+            for (int64_t u = u0; u < u1; ++u) {
                 const Unit U = unit_of(p, u);
                 if constexpr (WRES) {  // the head's W_down of this axis is in shared memory
                     if (U.h != head) {
@@ -332,15 +348,16 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
                     }
                 }
                 const uint32_t idesc = umma_idesc_bf16(128, U.R, 0, 1);
-                const int slot = j & 1;
-                // the epilogue has read this slot's previous unit (j - 2)
-                if (!mbar_wait_warp(&accempty[slot], ((j >> 1) & 1) ^ 1u, abort_flag, p.err)) break;
-                tc_fence_after();
-                const uint32_t d = tmem + slot * L::SLOT;
                 bool ok = true;
 #pragma unroll 1
                 for (int s = 0; s < NS; ++s, ++q) {
-                    const int st = q % L::XST, sw = q % kWStages;
+                    const int st = q % L::XST, sw = q % kWStages, slot = piece & 1;
+                    const bool fresh = s % L::PIECE == 0;  // the epilogue has read this slot's piece before last
+                    if (fresh && !mbar_wait_warp(&accempty[slot], ((piece >> 1) & 1) ^ 1u, abort_flag, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t d = tmem + slot * L::SLOT;
                     if (!(MU ? mbar_wait_warp(&afull[q & 1], (q >> 1) & 1, abort_flag, p.err)
                              : mbar_wait_warp(&full[st], (q / L::XST) & 1, abort_flag, p.err)) ||
                         (!WRES && !mbar_wait_warp(&wfull[sw], (q / kWStages) & 1, abort_flag, p.err))) {
@@ -355,19 +372,22 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
 #pragma unroll
                             for (int ks = 0; ks < kES / 16; ++ks)
                                 umma_bf16_ts_warp(d, tmem + kAT + (q & 1) * 64 + part * 32 + ks * 8,
-                                                  umma_desc_sw128_mn(b + ks * 2048, kBAtom), idesc, s > 0 || part > 0 || ks > 0);
+                                                  umma_desc_sw128_mn(b + ks * 2048, kBAtom), idesc, !fresh || part > 0 || ks > 0);
                         umma_commit_warp(&aempty[q & 1]);
                     } else {
 #pragma unroll
                         for (int ks = 0; ks < kES / 16; ++ks)
                             umma_bf16_warp(d, umma_desc_sw128_k(a + ks * 32), umma_desc_sw128_mn(b + ks * 2048, kBAtom),
-                                           idesc, s > 0 || ks > 0);
+                                           idesc, !fresh || ks > 0);
                         umma_commit_warp(&empty[st]);
                     }
                     if (!WRES) umma_commit_warp(&wempty[sw]);
+                    if (s % L::PIECE == L::PIECE - 1 || s == NS - 1) {
+                        umma_commit_warp(&accfull[slot]);
+                        ++piece;
+                    }
                 }
                 if (!ok) break;
-                umma_commit_warp(&accfull[slot]);
             }
             // every product has completed before TMEM is released
             umma_commit_warp(done);
@@ -375,18 +395,14 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
             mbar_wait_warp(done, 0, &never, p.err);
         }
         __syncwarp();
-    } else if (warp <= 5) {
+    } else if (warp >= kEpi0 && warp < kConv0) {
         // --------------------------------------------------------------------------- epilogue
-        const int et = tid - 64;  // 0..127
-        const int quarter = warp & 3;
-        const int row = quarter * 32 + lane;
         int head = -1;
-        uint32_t have = 0;  // groups whose bias of this head is in `bias`
+        uint32_t have = 0;             // groups whose bias of this head is in `bias`
         bool wax[2] = {false, false};  // WRES: axes whose W_down of this head is resident
-        int j = 0;
-        for (int64_t u = u0; u < u1; ++u, ++j) {
+        uint32_t piece = 0;
+        for (int64_t u = u0; u < u1; ++u) {
             const Unit U = unit_of(p, u);
-            const int slot = j & 1;
             if (U.h != head) {
                 head = U.h;
                 have = 0;
@@ -398,24 +414,24 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
                 // of the previous head has completed: its last accumulator has been read.
                 wax[U.axis] = true;
                 const int r = U.axis ? p.r_v : p.r_k, hp = r / 2;
-                // 16-byte loads of the contiguous rows, up to sixteen in flight per thread, and four
+                // 16-byte loads of the contiguous rows, up to eight in flight per thread, and four
                 // 4-byte stores each (4-byte loads of padded rows took 8 us a head: 15 -> 8 us a call)
                 const uint4 *W = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(U.axis ? p.w_down_v : p.w_down_k) +
                                                                  static_cast<int64_t>(U.h) * Td * r);
                 char *dst = sm + oW + U.axis * (kResSlabs * kBAtom);
                 const uint32_t inv = (1u << 20) / hp + 1;  // q / hp = q * inv >> 20 below 512 rows of 32 pairs
-                for (int i0 = et; i0 < Td * r / 8; i0 += 128 * 16) {
-                    uint4 v[16];
+                for (int i0 = wt; i0 < Td * r / 8; i0 += kEpi * 8) {
+                    uint4 v[8];
 #pragma unroll
-                    for (int b = 0; b < 16; ++b)
-                        if (i0 + b * 128 < Td * r / 8) v[b] = W[i0 + b * 128];
+                    for (int b = 0; b < 8; ++b)
+                        if (i0 + b * kEpi < Td * r / 8) v[b] = W[i0 + b * kEpi];
 #pragma unroll
-                    for (int b = 0; b < 16; ++b) {
-                        if (i0 + b * 128 >= Td * r / 8) break;
+                    for (int b = 0; b < 8; ++b) {
+                        if (i0 + b * kEpi >= Td * r / 8) break;
                         const uint32_t wd[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const uint32_t q = (i0 + b * 128) * 4 + e;  // pair q: row q / hp
+                            const uint32_t q = (i0 + b * kEpi) * 4 + e;  // pair q: row q / hp
                             const uint32_t k = static_cast<uint32_t>((static_cast<uint64_t>(q) * inv) >> 20), c = q - k * hp;
                             *reinterpret_cast<uint32_t *>(dst + k * 128 + (((c >> 2) ^ (k & 7)) << 4) + (c & 3) * 4) = wd[e];
                         }
@@ -424,27 +440,58 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
                 fence_proxy_async_smem();
                 mbar_arrive(&wfull[U.axis]);
             }
-            char *stg = sm + L::oStg + quarter * (32 * 80);
+            const bool use_bias = MU && (U.axis ? p.mu_v : p.mu_k) != nullptr;
             float *bs = bias + U.g * kMaxGroup;
-            const float *mu = U.axis ? p.mu_v : p.mu_k;
-            if (MU && mu && !(have >> U.g & 1u)) {
+            if (MU && use_bias && !(have >> U.g & 1u)) {
                 have |= 1u << U.g;
                 const int r = U.axis ? p.r_v : p.r_k;
                 const uint16_t *W = static_cast<const uint16_t *>(U.axis ? p.w_down_v : p.w_down_k) +
                                     static_cast<int64_t>(U.h) * Td * r;
-                group_bias<WRES ? 2 : 8>(W, mu + static_cast<int64_t>(U.h) * Td, r, U, S0 * kES, S1 * kES, et,
-                                         reinterpret_cast<float *>(sm + L::oStg), bs);
+                group_bias<WRES ? 2 : 8>(W, (U.axis ? p.mu_v : p.mu_k) + static_cast<int64_t>(U.h) * Td, r, U, S0 * kES,
+                                         S1 * kES, wt, reinterpret_cast<float *>(sm + L::oStg), bs);
             }
-            const bool use_bias = MU && mu != nullptr;
-            if (split) break;  // the parts meet below
-            char *dst = row_dst(p, U, row, U.g == 0);
-            mbar_wait(&accfull[slot], (j >> 1) & 1, abort_flag, p.err);
-            tc_fence_after();
-            const uint32_t tl = tmem + slot * L::SLOT + (static_cast<uint32_t>(quarter * 32) << 16);
+            // the sum of the unit's pieces
+#pragma unroll
+            for (int i = 0; i < L::NC; ++i)
+#pragma unroll
+                for (int k = 0; k < 32; ++k) sum[i][k] = 0.f;
 #pragma unroll 1
-            for (int c0 = 0; c0 < U.cols; c0 += 32) {
-                float v[32];
-                tmem_ld32(tl + c0, v);  // warp-collective: every lane loads, valid rows store
+            for (int s = 0; s < NS; s += L::PIECE, ++piece) {
+                const int slot = piece & 1;
+                mbar_wait_warp(&accfull[slot], (piece >> 1) & 1, abort_flag, p.err);
+                tc_fence_after();
+                const uint32_t tl = tmem + slot * L::SLOT + (static_cast<uint32_t>(quarter * 32) << 16);
+#pragma unroll
+                for (int i = 0; i < L::NC; ++i) {
+                    const int c0 = 64 * i + 32 * half;
+                    if (c0 >= U.cols) break;
+                    if constexpr (MU) {  // fewer registers
+#pragma unroll
+                        for (int k0 = 0; k0 < 32; k0 += 16) {
+                            float v[16];
+                            tmem_ld16(tl + c0 + k0, v);  // warp-collective
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) sum[i][k0 + k] += v[k];
+                        }
+                    } else {
+                        float v[32];
+                        tmem_ld32(tl + c0, v);
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) sum[i][k] += v[k];
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&accempty[slot]);  // this slot may take the piece after next
+            }
+            if (split) break;  // the parts meet below
+            char *stg = sm + L::oStg + (warp - kEpi0) * (32 * 80);
+            char *dst = row_dst(p, U, row, U.g == 0 && half == 0);
+#pragma unroll
+            for (int i = 0; i < L::NC; ++i) {
+                const int c0 = 64 * i + 32 * half;
+                if (c0 >= U.cols) break;
+                const float (&v)[32] = sum[i];
                 if constexpr (WRES) {
                     // rows that are not whole 16-byte words: pairs of columns.  K: consecutive rows
                     // are consecutive granules.  V: the warp's 32 rows through the staging buffer, so
@@ -522,65 +569,66 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
                     }
                 }
             }
-            // this slot may take unit j + 2
+        }
+    } else if (MU && warp >= kConv0) {
+        // ------------------------------------------------------- x - m into TMEM (one row per thread)
+        uint32_t *mws = reinterpret_cast<uint32_t *>(sm + L::oMu) + quarter * 64;  // [2][32] pairs of m
+        const char *xr = sm + row * 128;
+        const uint32_t ta = tmem + kAT + (static_cast<uint32_t>(quarter * 32) << 16);
+        const int total = static_cast<int>(u1 - u0) * NS;
+        int64_t u = u0;
+        int s = 0;
+        const float *mu = nullptr;
+        float m0 = 0.f, m1 = 0.f;  // mu of the slab to come
+        auto next_mu = [&] {       // of slab s of unit u, then on to the next
+            if (s == 0 && u < u1) {
+                const Unit U = unit_of(p, u);
+                mu = U.axis ? p.mu_v : p.mu_k;
+                if (mu) mu += static_cast<int64_t>(U.h) * Td + S0 * kES + 2 * lane;
+                else m0 = m1 = 0.f;
+            }
+            if (u < u1 && mu) {
+                m0 = mu[s * kES];
+                m1 = mu[s * kES + 1];
+            }
+            if (++s == NS) {
+                s = 0;
+                ++u;
+            }
+        };
+        next_mu();
+#pragma unroll 1
+        for (int q = 0; q < total; ++q) {
+            const int st = q % L::XST, buf = q & 1;
+            mws[buf * 32 + lane] = pack_bf16(m0, m1);
+            next_mu();
+            __syncwarp();
+            mbar_wait_warp(&full[st], (q / L::XST) & 1, abort_flag, p.err);
+            uint32_t hi[32], lo[32];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint4 x = *reinterpret_cast<const uint4 *>(xr + st * kASlab + ((c ^ (row & 7)) << 4));
+                hi[4 * c] = x.x; hi[4 * c + 1] = x.y; hi[4 * c + 2] = x.z; hi[4 * c + 3] = x.w;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[st]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint4 m = *reinterpret_cast<const uint4 *>(mws + buf * 32 + 4 * c);
+                sub_exact_bf16x2(hi[4 * c], m.x, hi[4 * c], lo[4 * c]);
+                sub_exact_bf16x2(hi[4 * c + 1], m.y, hi[4 * c + 1], lo[4 * c + 1]);
+                sub_exact_bf16x2(hi[4 * c + 2], m.z, hi[4 * c + 2], lo[4 * c + 2]);
+                sub_exact_bf16x2(hi[4 * c + 3], m.w, hi[4 * c + 3], lo[4 * c + 3]);
+            }
+            // the products of two slabs ago have read this buffer
+            mbar_wait_warp(&aempty[buf], ((q >> 1) & 1) ^ 1u, abort_flag, p.err);
+            tc_fence_after();
+            tmem_st32u_nowait(ta + buf * 64, hi);
+            tmem_st32u_nowait(ta + buf * 64 + 32, lo);
+            tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&accempty[slot]);
-        }
-    } else if (MU && warp >= 7) {
-        // ------------------------------------------------------- x - m into TMEM (one row per thread)
-        const int quarter = warp & 3, row = quarter * 32 + lane;
-        uint32_t *mws = reinterpret_cast<uint32_t *>(sm + L::oMu) + quarter * 64;  // [2][32] pairs of m
-        const uint32_t ta = tmem + kAT + (static_cast<uint32_t>(quarter * 32) << 16);
-        int q = 0;
-        bool stop = false;
-        for (int64_t u = u0; u < u1 && !stop; ++u) {
-            const Unit U = unit_of(p, u);
-            const float *mu = U.axis ? p.mu_v : p.mu_k;
-            if (mu) mu += static_cast<int64_t>(U.h) * Td + S0 * kES + 2 * lane;
-            float m0 = mu ? mu[0] : 0.f, m1 = mu ? mu[1] : 0.f;  // of the slab to come
-            for (int s = 0; s < NS; ++s, ++q) {
-                const int st = q % L::XST, buf = q & 1;
-                mws[buf * 32 + lane] = pack_bf16(m0, m1);
-                if (mu && s + 1 < NS) {
-                    m0 = mu[(s + 1) * kES];
-                    m1 = mu[(s + 1) * kES + 1];
-                }
-                __syncwarp();
-                if (!mbar_wait_warp(&full[st], (q / L::XST) & 1, abort_flag, p.err)) {
-                    stop = true;
-                    break;
-                }
-                const char *xr = sm + st * kASlab + row * 128;
-                uint32_t hi[32], lo[32];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint4 x = *reinterpret_cast<const uint4 *>(xr + ((c ^ (row & 7)) << 4));
-                    hi[4 * c] = x.x; hi[4 * c + 1] = x.y; hi[4 * c + 2] = x.z; hi[4 * c + 3] = x.w;
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[st]);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint4 m = *reinterpret_cast<const uint4 *>(mws + buf * 32 + 4 * c);
-                    sub_exact_bf16x2(hi[4 * c], m.x, hi[4 * c], lo[4 * c]);
-                    sub_exact_bf16x2(hi[4 * c + 1], m.y, hi[4 * c + 1], lo[4 * c + 1]);
-                    sub_exact_bf16x2(hi[4 * c + 2], m.z, hi[4 * c + 2], lo[4 * c + 2]);
-                    sub_exact_bf16x2(hi[4 * c + 3], m.w, hi[4 * c + 3], lo[4 * c + 3]);
-                }
-                // the products of two slabs ago have read this buffer
-                if (!mbar_wait_warp(&aempty[buf], ((q >> 1) & 1) ^ 1u, abort_flag, p.err)) {
-                    stop = true;
-                    break;
-                }
-                tc_fence_after();
-                tmem_st32u_nowait(ta + buf * 64, hi);
-                tmem_st32u_nowait(ta + buf * 64 + 32, lo);
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&afull[buf]);
-            }
+            if (lane == 0) mbar_arrive(&afull[buf]);
         }
     }
     pdl_trigger();
@@ -590,33 +638,29 @@ __global__ void __launch_bounds__(EL<WRES, MU>::THREADS, 1)
         cluster_sync();
         const Unit U = unit_of(p, u0);
         const int own = ((U.cols + p.split - 1) / p.split + 7) & ~7;  // columns each rank stores
-        const bool ep = warp >= 2 && warp <= 5;
-        const int quarter = warp & 3, row = quarter * 32 + lane;
+        const bool ep = warp >= kEpi0 && warp < kConv0;
         const float *bs = bias + U.g * kMaxGroup;
         const bool use_bias = MU && (U.axis ? p.mu_v : p.mu_k) != nullptr;
         if (ep) {
-            mbar_wait(&accfull[0], 0, abort_flag, p.err);
-            tc_fence_after();
-            const uint32_t tl = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-#pragma unroll 1
-            for (int c0 = 0; c0 < U.cols; c0 += 8) {
-                float v[8];
-                tmem_ld8(tl + c0, v);
-                if (use_bias) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) v[i] -= bs[c0 + i];
+            for (int i = 0; i < L::NC; ++i)
+#pragma unroll
+                for (int k = 0; k < 32; k += 8) {
+                    const int c0 = 64 * i + 32 * half + k;
+                    if (c0 >= U.cols) break;
+                    float v[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = use_bias ? sum[i][k + e] - bs[c0 + e] : sum[i][k + e];
+                    const uint32_t to = c0 / own;
+                    const uint32_t at = smem_addr(sm) + ((crank * (own / 4) + (c0 - to * own) / 4) * kEM + row) * 16;
+                    st_cluster_f4(at, to, make_float4(v[0], v[1], v[2], v[3]));
+                    st_cluster_f4(at + kEM * 16, to, make_float4(v[4], v[5], v[6], v[7]));
                 }
-                const uint32_t to = c0 / own;
-                const uint32_t at = smem_addr(sm) + ((crank * (own / 4) + (c0 - to * own) / 4) * kEM + row) * 16;
-                st_cluster_f4(at, to, make_float4(v[0], v[1], v[2], v[3]));
-                st_cluster_f4(at + kEM * 16, to, make_float4(v[4], v[5], v[6], v[7]));
-            }
-            tc_fence_before();
         }
         cluster_sync();
         if (ep) {
-            char *dst = row_dst(p, U, row, U.g == 0 && crank == 0);
-            for (int c0 = crank * own; c0 < min(U.cols, (crank + 1) * own); c0 += 8) {
+            char *dst = row_dst(p, U, row, U.g == 0 && crank == 0 && half == 0);
+            for (int c0 = crank * own + 8 * half; c0 < min(U.cols, (crank + 1) * own); c0 += 16) {
                 float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 for (int q = 0; q < p.split; ++q) {
                     const float4 *src = reinterpret_cast<const float4 *>(sm) + (q * (own / 4) + (c0 - crank * own) / 4) * kEM + row;

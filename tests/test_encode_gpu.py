@@ -239,3 +239,29 @@ def test_encode_infinite_input(lla, N, r_k, r_v):
         for wa, got in zip(w, unpack_head(pool_cpu, H, r_k, r_v, "bf16", list(range(pages)), N, h)):
             assert np.isfinite(np.delete(got, 5, 0)).all()
             assert (got[5] == np.sign(f64(wa[h, d + 7])) * np.inf).all()
+
+
+@pytest.mark.parametrize("with_mu", [False, True])
+def test_encode_2d_long_sums_are_as_exact_as_fp32(lla, with_mu):
+    """8192 products of one sign: sums in the tensor core are cut off, not rounded, so that a long one falls
+    short by half a unit of 2^-23 per step on average.  In chains of 16 steps, added up by fp32 adds, a latent
+    is short by 16 / 4 such units (the partial sums are half as large on average), 4.8e-7 of itself: one in
+    11000 is then rounded to another bf16 number (spacing 2^-8 to 2^-7 of a value).  Chains of 2048 rows would
+    give eight times as many; the bound is three and a half times."""
+    T, H, d, r_k, r_v, N = 4, 16, 128, 288, 480, 500
+    g = torch.Generator(device=DEV).manual_seed(17)
+    rand = lambda *s: torch.rand(s, generator=g, device=DEV) + 0.5
+    geom = lla.Geometry(T, H, d, r_k, r_v)
+    pages = -(-N // 64)
+    pool = torch.zeros(pages * lla.lla_cache_2d_block_bytes(geom), dtype=torch.uint8, device=DEV)
+    x = rand(T, N, H, d).to(torch.bfloat16)
+    w = [rand(T * H * d, r).to(torch.bfloat16) for r in (r_k, r_v)]
+    mu = -rand(T * H * d) if with_mu else None
+    lla.lla_encode_2d(geom, lla.Codec(w[0], w[1], None, None, mu, mu), lla.Cache(pool, pages, None, 1), x, x,
+                      torch.arange(N, device=DEV))
+    s = x.permute(1, 0, 2, 3).reshape(N, -1).double() - (mu.double() if with_mu else 0)
+    wrong = 0
+    for wa, got in zip(w, unpack_head(pool.cpu(), 1, r_k, r_v, "bf16", list(range(pages)), N, 0)):
+        want = (s @ wa.double()).to(torch.bfloat16)
+        wrong += int((torch.from_numpy(got).to(DEV) != want.double()).sum())
+    assert wrong <= 3e-4 * N * (r_k + r_v), wrong

@@ -33,10 +33,12 @@
 // one's softmax (about 1000 cycles from scores to weights) runs beside the other's: the running maximum
 // goes from page to page through shared memory and a named barrier per warp pair, each group keeps its
 // own row sums, and they meet after the last page.
-// Accumulators are fp32 in TMEM; operands are bf16 (q~ carries scale * log2 e).  At (72, 120) q~ and P
-// are sums of two bf16 parts (16 significant bits; twice the products): that shape was served in fp32
-// by the CUDA cores, and its bf16 outputs stay as exact as their rounding.  So at (18, 30), whose rows
-// are not whole 16-byte words: there the producer warps move pages and W_up through registers.
+// Accumulators are fp32 in TMEM; operands are bf16 (q~ carries scale * log2 e).  At (72, 120) q~, P
+// and O / l are sums of three bf16 parts (24 significant bits; three times the products): that shape was
+// served in fp32 by the CUDA cores, and its results stay as exact.  (Two parts, 16 bits, took 56 us instead
+// of 70 for 3 ragged prompts, but with scores in the hundreds five times as many outputs were rounded the
+// wrong way as with fp32 sums.)  So at (18, 30), whose rows are not whole 16-byte words: there the producer
+// warps move pages and W_up through registers.
 //
 // Bound by the tensor pipe and the shared memory that feeds it: a (192, 320) page takes 640 cycles of PV
 // products and 576 of score products (a 128 x 64 x 16 product reads 6 KB, 48 cycles of shared memory for
@@ -45,10 +47,9 @@
 // the power limit), at (96, 160) 1445 -> 919 us, at (128, 128) 1445 -> 975 us; a tile of 2 pages from
 // launch to output 18 -> 10 us (W_up was staged by one warp's cp.async, W_up,t^V only after the last
 // page, and the hi and lo projections followed each other through shared memory).  From the CUDA cores:
-// (72, 120), 300 tokens 265 -> 9.6 us, 3 ragged prompts of 3531 tokens 8330 -> 55 us; (18, 30), 1000 tokens
-// 720 -> 23.4 us, 8192 tokens 43.1 -> 0.60 ms (1.4 us a page, twice the (72, 120) page's: the producer
-// warps.  Their pairs' places kept in registers changed nothing; three pages in flight spilled and cost
-// 15 %).
+// (72, 120), 300 tokens 265 -> 11.2 us, 3 ragged prompts of 3531 tokens 8330 -> 70 us; (18, 30), 1000 tokens
+// 720 -> 25.2 us, 8192 tokens 43.1 -> 0.53 ms (its producer warps bound it: their pairs' places kept in
+// registers changed nothing; three pages in flight spilled and cost 15 %).
 //
 // CUDA-core path (fp32 storage, other ranks, d != 128, fp32 inputs at (72, 120) and (18, 30)): one CTA
 // per (query, sequence, head), fp32 throughout.
@@ -121,6 +122,7 @@ struct PF {
     static constexpr int QA1 = kBM * D * 2;          // q operand of one tile (prologue)
     static constexpr int WK = KATOMS * D * 128;      // W_up,t^K operand (prologue)
     static constexpr int WV = VATOMS * D * 128;      // W_up,t^V operand (epilogue)
+    static constexpr int OP = QP > 1 ? 3 : 2;        // bf16 parts of O / l in the epilogue
     static constexpr int BUDGET = 222 * 1024;
     // W_up,t^V has room of its own, or takes q~'s and the K ring's once every score product is done
     static constexpr bool WVOWN = QT + 2 * KPAGE + 3 * VPAGE + WV <= BUDGET;
@@ -148,6 +150,7 @@ struct PF {
     static_assert(RK % 2 == 0 && RV % 2 == 0 && RKX <= 256 && RKX <= ORV, "ranks");
     static_assert(!NARROW || (RK <= 64 && RV <= 64 && WVOWN && !ROPE), "one 64-column box per row");
     static_assert(TM_O + NT * ORV <= TM_COLS && N1 <= 256 && N1 % 16 == 0, "TMEM columns");
+    static_assert(OP == 2 || (NT == 1 && VATOMS * 32 <= 2 * QP * (kPT / 2)), "the third part over the weights");
     static_assert(STK >= 2 && STV >= 2, "pipeline depth");
     static_assert(KPAGE % 1024 == 0 && QT1 % 1024 == 0, "align");
     static_assert(NT * QA1 <= STV * VPAGE && (WVOWN ? WK <= WV : NT * QA1 + WK <= STV * VPAGE), "prologue operands fit");
@@ -559,11 +562,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
                     constexpr int last = F::ORV - (F::VATOMS - 1) * 64;  // columns of the last chunk
                     const int cols = c == F::VATOMS - 1 ? last : 64;
 #pragma unroll
-                    for (int part = 0; part < 2; ++part)
+                    for (int part = 0; part < F::OP; ++part)
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) {
                             if (ks * 16 >= cols) continue;
-                            umma_bf16_ts_warp(ds, tmem + F::TM_O + tile * F::ORV + c * 64 + part * (cols / 2) + ks * 8,
+                            const uint32_t at = part == 2 ? F::TM_P + c * 32 : F::TM_O + tile * F::ORV + c * 64 + part * (cols / 2);
+                            umma_bf16_ts_warp(ds, tmem + at + ks * 8,
                                          dwv + ((c * (D * 128) + half * (64 * 128) + ks * 32) >> 4), ido, acc);
                             acc = true;
                         }
@@ -788,10 +792,18 @@ __global__ void __launch_bounds__(kPThreads, 1)
                 if (!any) wait_own();
                 tc_fence_after();
                 tmem_st32u_nowait(tp, w);
-                if constexpr (QP > 1) {
 #pragma unroll
-                    for (int c = 0; c < kPT; c += 2) w[c / 2] = pack_bf16x2(x[c], x[c + 1]);
-                    tmem_st32u_nowait(tp + kPT / 2, w);
+                for (int part = 1; part < QP; ++part) {
+#pragma unroll
+                    for (int c = 0; c < kPT; c += 2) {
+                        w[c / 2] = pack_bf16x2(x[c], x[c + 1]);
+                        if (part + 1 < QP) {
+                            const float2 f = bf2_to_f2(w[c / 2]);
+                            x[c] -= f.x;
+                            x[c + 1] -= f.y;
+                        }
+                    }
+                    tmem_st32u_nowait(tp + part * (kPT / 2), w);
                 }
             }
             if (j == NPg - 1 && kb + kPT > L) {
@@ -837,23 +849,32 @@ __global__ void __launch_bounds__(kPThreads, 1)
             float v[32], u[32];
             tmem_ld32(to + c * 64, v);
             if (half == 32) tmem_ld32(to + c * 64 + 32, u);
-            uint32_t hi[16], lo[16];
+            uint32_t hi[16], lo[16], lo2[16];
             auto convert = [&](const float (&v)[32]) {
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
-                    const float a = v[2 * k] * inv, bb = v[2 * k + 1] * inv;
+                    float a = v[2 * k] * inv, bb = v[2 * k + 1] * inv;
                     hi[k] = pack_bf16x2(a, bb);
-                    const float2 f = bf2_to_f2(hi[k]);
-                    lo[k] = pack_bf16x2(a - f.x, bb - f.y);
+                    float2 f = bf2_to_f2(hi[k]);
+                    a -= f.x;
+                    bb -= f.y;
+                    lo[k] = pack_bf16x2(a, bb);
+                    if constexpr (F::OP == 3) {
+                        f = bf2_to_f2(lo[k]);
+                        lo2[k] = pack_bf16x2(a - f.x, bb - f.y);
+                    }
                 }
             };
+            const uint32_t t2 = tl + F::TM_P + c * 32;  // every product has read the weights there
             convert(v);
             tmem_st16u(to + c * 64, hi);
             tmem_st16u(to + c * 64 + half, lo);
+            if constexpr (F::OP == 3) tmem_st16u(t2, lo2);
             if (half == 32) {
                 convert(u);
                 tmem_st16u(to + c * 64 + 16, hi);
                 tmem_st16u(to + c * 64 + 48, lo);
+                if constexpr (F::OP == 3) tmem_st16u(t2 + 16, lo2);
             }
         }
         tmem_wait_st();
@@ -1356,7 +1377,7 @@ lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t 
     // but reads all pages at once.  So pair after pair, and then the last three waves of CTAs' pairs, or
     // as many as half of L2 holds, together.  Pair after pair only / this rule / all together: 3 ragged
     // prompts at (72, 120) 127 / 115 / 113 us, 8 x 2048 tokens at (96, 160) 207 / 195 / 186, 4 x 2000 at
-    // (18, 30) 235 / 169 / 171, 4 x 8192 at (192, 320) 1679 / 1652 / 2047, six ragged rotary prompts 396 /
+    // (18, 30) 235 / 169 / 171 (both with two bf16 parts of q~ and P), 4 x 8192 at (192, 320) 1679 / 1652 / 2047, six ragged rotary prompts 396 /
     // 357 / 356.  (Six and ten waves: 1693 and 1770 us at (192, 320).)
     const int tiles = (a.max_len + NT * kBM - 1) / (NT * kBM);
     const int64_t pairs = static_cast<int64_t>(a.B) * a.H;
@@ -1395,7 +1416,7 @@ lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t 
 // 1050 tokens, 256 pairs, 35 and 36; 8 x 64 to 2048, 384 pairs of which half exist, 25 and 28), so that
 // two start above that; with rotated keys those two cases take 63 and 61, 50 and 51, and two start at 256.
 // Prompts of one tile leave the second empty (32 x 100: 34 and 37).  With two bf16 parts the products bound
-// it either way (2 x 8192 at (72, 120): 630 and 644), so (72, 120) takes one.
+// it either way (2 x 8192 at (72, 120): 630 and 644), and three leave no TMEM for a second O: one tile.
 template <int RK, int RV, bool ROPE, int QP = 1>
 lla_status launch_tc(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {
     if constexpr (RV <= 160 && QP == 1) {
@@ -1435,8 +1456,8 @@ lla_status launch_prefill(const PrefillArgs &a, cudaStream_t stream) {
         if (a.r_k == 96 && a.r_v == 160) return launch_tc<96, 160, false>(p, a, stream);
         if (a.r_k == 192 && a.r_v == 320) return launch_tc<192, 320, false>(p, a, stream);
         if (a.r_k == 128 && a.r_v == 128) return launch_tc<128, 128, false>(p, a, stream);
-        if (a.r_k == 72 && a.r_v == 120 && a.io_bf16) return launch_tc<72, 120, false, 2>(p, a, stream);
-        if (a.r_k == 18 && a.r_v == 30 && a.io_bf16) return launch_tc<18, 30, false, 2>(p, a, stream);
+        if (a.r_k == 72 && a.r_v == 120 && a.io_bf16) return launch_tc<72, 120, false, 3>(p, a, stream);
+        if (a.r_k == 18 && a.r_v == 30 && a.io_bf16) return launch_tc<18, 30, false, 3>(p, a, stream);
     }
     GParams g = {};
     g.T = a.T; g.H = a.H; g.d = a.d; g.r_k = a.r_k; g.r_v = a.r_v; g.loop = a.loop;

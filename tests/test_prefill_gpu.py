@@ -141,7 +141,7 @@ def _rising_scores_case(lla, r_k, r_v, H, lens, seed, tol):
 
 def test_prefill_rising_scores_one_tile_per_cta(lla):
     # the two softmax groups take a tile's pages in turn and hand the running maximum on.  At (72, 120)
-    # q~ and the softmax weights are sums of two bf16 parts: bf16 outputs are then as exact as their
+    # q~ and the softmax weights are sums of three bf16 parts: bf16 outputs are then as exact as their
     # own rounding (2^-9 relative) however large the scores
     _rising_scores_case(lla, 72, 120, 2, [700, 321], 31, 2 ** -9 + 1e-4)
 
@@ -169,3 +169,24 @@ def test_prefill_rows_without_16_byte_words(lla, H, lens):
 
 def test_prefill_rising_scores_rows_without_16_byte_words(lla):
     _rising_scores_case(lla, 18, 30, 2, [700, 321], 33, 2 ** -9 + 1e-4)
+
+
+@pytest.mark.parametrize("r_k,r_v", [(72, 120), (18, 30)])
+def test_prefill_in_parts_is_as_exact_as_the_cuda_cores(lla, r_k, r_v):
+    """bf16 queries take the tensor cores with q~, weights and O / l in bf16 parts, the same queries in fp32 the
+    CUDA cores in fp32.  A sum in the tensor core falls short by 2^-25 of itself per step on average; some 60
+    steps (values and projection) over partial sums twice the result's size make 3.6e-6 of an output, which
+    rounds one in 1500 (a spacing is 2^-8 to 2^-7) to another bf16 number.  Operands of 16 bits instead of 24
+    would move one in 550; the bound is one in 1000."""
+    lens, H = [200, 130, 64, 1], 8
+    sc = Scene(lla, T=4, H=H, d=128, r_k=r_k, r_v=r_v, storage="bf16", io="bf16", lens=lens, seed=34, with_mu=True,
+               extra_tokens=0)
+    q = sc.W.normal((sum(lens), H, 128), 34, 72, device=DEV)
+    cu = torch.tensor(np.cumsum([0] + lens), dtype=torch.int32, device=DEV)
+    out, ref = torch.empty_like(q), torch.empty(q.shape, device=DEV)
+    lla.lla_prefill_attn(sc.geom, sc.codec, sc.cache, cu, max(lens), 1, q, out)
+    lla.lla_prefill_attn(sc.geom, sc.codec, sc.cache, cu, max(lens), 1, q.float(), ref)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    moved = (out != ref.to(torch.bfloat16)).float().mean().item()
+    assert moved <= 1e-3, moved

@@ -4,7 +4,7 @@
 Each translation unit is compiled by nvcc in parallel, then linked into
 paper_2607_15456_gb300/liblla.so with the CUDA runtime linked statically, so the library
 needs nothing but the driver at run time.  The binding is one host translation unit against torch's
-headers, compiled beside them.
+headers, compiled beside them; where it cannot be built, calls are marshalled in Python.
 """
 from __future__ import annotations
 
@@ -39,16 +39,17 @@ def _sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
-        os.path.join(CSRC, "*.h")) + [BINDING, os.path.join(ROOT, "include", "lla.h"), __file__]
+def _newer(target: str, deps) -> bool:
+    return os.path.exists(target) and all(os.path.getmtime(p) <= os.path.getmtime(target) for p in deps)
 
 
-def up_to_date() -> bool:
-    if not (os.path.exists(LIB) and os.path.exists(NATIVE)):
-        return False
-    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
-    return all(os.path.getmtime(p) <= t for p in _deps())
+def library_up_to_date() -> bool:
+    return _newer(LIB, _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
+                  [os.path.join(ROOT, "include", "lla.h"), __file__])
+
+
+def binding_up_to_date() -> bool:
+    return _newer(NATIVE, [BINDING, os.path.join(ROOT, "include", "lla.h"), __file__])
 
 
 def _run(cmd, what: str):
@@ -80,8 +81,10 @@ def link_binding(obj: str) -> None:
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
-    """Compiles every csrc/*.cu for sm_103a and links liblla.so; returns its path."""
-    if not force and up_to_date():
+    """Compiles every csrc/*.cu for sm_103a and links liblla.so, and builds the binding's native
+    marshalling beside it; returns the library's path."""
+    library, binding = force or not library_up_to_date(), force or not binding_up_to_date()
+    if not library and not binding:
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
@@ -99,16 +102,22 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         return obj
 
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 2)) as ex:
-        binding = ex.submit(compile_binding)
-        objs = list(ex.map(compile_one, _sources()))
-        binding = binding.result()
-    tmp = LIB + ".tmp%d" % os.getpid()
-    cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", *objs, "-o", tmp]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
-    os.replace(tmp, LIB)
-    link_binding(binding)
+        obj = ex.submit(compile_binding) if binding else None
+        objs = list(ex.map(compile_one, _sources())) if library else []
+    if library:
+        tmp = LIB + ".tmp%d" % os.getpid()
+        cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", *objs, "-o", tmp]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
+        os.replace(tmp, LIB)
+    if binding:
+        try:
+            link_binding(obj.result())
+        except (RuntimeError, OSError, ImportError) as e:  # no g++, no headers, another torch
+            if os.path.exists(NATIVE):
+                os.remove(NATIVE)  # of an older source
+            sys.stderr.write(f"_lla_native.so was not built, calls will be marshalled in Python: {e}\n")
     return LIB
 
 

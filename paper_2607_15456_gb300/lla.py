@@ -4,20 +4,23 @@ Every function here has the name of the C entry point it calls and does nothing 
 torch tensors into device pointers, fill the ABI structs and raise ``LLAError`` on a non-zero
 status.  The calls of a decode step and of a prompt are marshalled by ``_lla_native``
 (csrc/lla_binding.cpp) when their arguments are the ordinary ones, contiguous CUDA tensors and ints;
-it answers None to anything else, which the Python marshalling below takes or refuses.  All computation happens in the CUDA kernels of liblla.so; there is no fallback: if
-the library is missing or a call fails, an exception is raised.
+it answers None to anything else, which the Python marshalling below takes or refuses, as it does
+every call where that module is missing.  All computation happens in the CUDA kernels of liblla.so;
+there is no fallback: if the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib
 import math
 import os
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
 import torch
 
-from .build import LIB, NATIVE
+from .build import LIB
 
 LLA_BLOCK_TOKENS = 64
 LLA_MAX_BATCH = 1024
@@ -70,16 +73,24 @@ _lib = None
 _native_module = None
 
 
+class _Absent:
+    """In the place of _lla_native where it cannot be loaded: leaves every call to Python."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _native():
     """The native marshalling module, loaded with the library it calls."""
     global _native_module
     if _native_module is None:
         library()
-        if not os.path.exists(NATIVE):
-            raise RuntimeError(f"_lla_native.so not found at {NATIVE}: build it first "
-                               "(python -c 'import __graft_entry__ as g; g.build()')")
-        from . import _lla_native
-        _native_module = _lla_native
+        try:
+            module = importlib.import_module("._lla_native", __package__)
+        except ImportError as e:
+            warnings.warn(f"calls are marshalled in Python (several us each): _lla_native.so is not loaded: {e}")
+            module = _Absent()
+        _native_module = module
     return _native_module
 
 

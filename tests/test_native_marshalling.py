@@ -53,3 +53,34 @@ def test_unusual_geometry_is_left_to_python(lla, field, value):
     args = _args(lla, "decode_attn", None)
     setattr(args[0], field, value)
     assert lla._native().decode_attn(*args) is None
+
+
+def test_a_missing_module_leaves_every_call_to_python(lla, monkeypatch):
+    def missing(name, package=None):
+        raise ImportError("no such module")
+
+    monkeypatch.setattr(lla, "_native_module", None)
+    monkeypatch.setattr(lla.importlib, "import_module", missing)
+    with pytest.warns(UserWarning, match="marshalled in Python"):
+        assert lla._native().encode(1, 2, 3) is None
+    for name in NAMES:
+        args = _args(lla, name, torch.zeros(4, 4, 2, 128))
+        assert getattr(lla._native(), name)(*args) is None
+        with pytest.raises(ValueError, match="CUDA tensors"):
+            getattr(lla, "lla_" + name)(*args)
+
+
+def test_a_binding_that_does_not_compile_does_not_fail_the_build(lla, monkeypatch, tmp_path, capsys):
+    from paper_2607_15456_gb300 import build
+    stale = tmp_path / "_lla_native.so"
+    stale.write_bytes(b"")
+    monkeypatch.setattr(build, "NATIVE", str(stale))
+    monkeypatch.setattr(build, "library_up_to_date", lambda: True)
+    monkeypatch.setattr(build, "binding_up_to_date", lambda: False)
+
+    def fails():
+        raise RuntimeError("g++ on lla_binding.cpp failed")
+
+    monkeypatch.setattr(build, "compile_binding", fails)
+    assert build.build() == build.LIB
+    assert not stale.exists() and "marshalled in Python" in capsys.readouterr().err

@@ -48,8 +48,19 @@ def library_up_to_date() -> bool:
                   [os.path.join(ROOT, "include", "lla.h"), __file__])
 
 
+def binding_abi() -> str:
+    """What _lla_native.so is compiled against: the interpreter's and torch's C++ ABI."""
+    import torch
+    return f"{sysconfig.get_config_var('SOABI')} torch {torch.__version__}"
+
+
 def binding_up_to_date() -> bool:
-    return _newer(NATIVE, [BINDING, os.path.join(ROOT, "include", "lla.h"), __file__])
+    try:
+        with open(NATIVE + ".abi") as f:
+            abi = f.read()
+    except OSError:
+        return False
+    return abi == binding_abi() and _newer(NATIVE, [BINDING, os.path.join(ROOT, "include", "lla.h"), __file__])
 
 
 def _run(cmd, what: str):
@@ -77,7 +88,11 @@ def link_binding(obj: str) -> None:
     tmp = NATIVE + ".tmp%d" % os.getpid()
     _run(["g++", "-shared", obj, "-o", tmp, "-L" + PKG, "-l:liblla.so", "-Wl,-rpath,$ORIGIN", "-L" + lib, "-ltorch_python",
           "-ltorch_cpu", "-lc10", "-lc10_cuda"], "linking _lla_native.so")
+    if os.path.exists(NATIVE + ".abi"):
+        os.remove(NATIVE + ".abi")  # never a new note beside an old module
     os.replace(tmp, NATIVE)
+    with open(NATIVE + ".abi", "w") as f:
+        f.write(binding_abi())
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:

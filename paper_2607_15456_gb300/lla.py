@@ -20,7 +20,7 @@ from typing import Optional
 
 import torch
 
-from .build import LIB
+from .build import LIB, NATIVE, binding_abi
 
 LLA_BLOCK_TOKENS = 64
 LLA_MAX_BATCH = 1024
@@ -86,8 +86,12 @@ def _native():
     if _native_module is None:
         library()
         try:
+            with open(NATIVE + ".abi") as f:
+                abi = f.read()
+            if abi != binding_abi():  # its tensors would be misread
+                raise ImportError(f"built for {abi}, not for {binding_abi()}")
             module = importlib.import_module("._lla_native", __package__)
-        except ImportError as e:
+        except (ImportError, OSError) as e:
             warnings.warn(f"calls are marshalled in Python (several us each): _lla_native.so is not loaded: {e}")
             module = _Absent()
         _native_module = module

@@ -84,3 +84,13 @@ def test_a_binding_that_does_not_compile_does_not_fail_the_build(lla, monkeypatc
     monkeypatch.setattr(build, "compile_binding", fails)
     assert build.build() == build.LIB
     assert not stale.exists() and "marshalled in Python" in capsys.readouterr().err
+
+
+def test_a_binding_of_another_torch_is_neither_loaded_nor_up_to_date(lla, monkeypatch):
+    from paper_2607_15456_gb300 import build
+    assert build.binding_up_to_date()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert not build.binding_up_to_date()
+    monkeypatch.setattr(lla, "_native_module", None)
+    with pytest.warns(UserWarning, match="built for"):
+        assert lla._native().encode(1, 2, 3) is None

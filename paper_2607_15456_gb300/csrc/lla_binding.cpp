@@ -2,8 +2,9 @@
 //
 // Each function takes the arguments of the Python function of the same name (with a stream handle or
 // None for the current stream), fills the structs of include/lla.h straight from the objects and calls
-// liblla with the GIL released.  It handles the ordinary call and nothing else: plain CUDA tensors that
-// are contiguous (or None), Python ints in range, bf16 or fp32 data.  Anything else (integer addresses,
+// liblla with the GIL released.  It handles the ordinary call and nothing else: plain CUDA tensors
+// (torch.nn.Parameter among them) that are contiguous, or None, Python ints in range, bf16 or fp32 data.
+// Anything else (integer addresses,
 // tensor subclasses, host or strided tensors, other types, wrong lengths) returns None, and the caller
 // goes through its Python marshalling, which accepts or refuses it as it always did.  No reference is
 // kept to any argument.

@@ -7,8 +7,8 @@ reconstructed K/V of every key (Eq. decode).  Two comparisons per (sequence, hea
     storage: relative L2 <= 1e-5);
   * against the oracle fed the latents the GPU stored, so that only the attention kernel is
     under test (relative L2 <= 5e-3 with bf16 tensor-core operands, 1e-5 in fp32).
-Cases reach both code paths (tcgen05 for bf16 storage with ranks multiple of 16, CUDA cores
-otherwise), prompts shorter than a page, on page and tile boundaries and across several query
+Cases reach both code paths (tcgen05 for bf16 storage at (96, 160), (192, 320) and (128, 128), and with
+bf16 queries at (72, 120) and (18, 30); CUDA cores otherwise), prompts shorter than a page, on page and tile boundaries and across several query
 tiles, fp32 and bf16 queries, with and without mu.
 """
 import math
@@ -34,7 +34,7 @@ def lla():
     return m
 
 
-def _prefill_case(lla, r_k, r_v, storage, io, lens, loop, with_mu, H=2, seed=0):
+def _prefill_case(lla, r_k, r_v, storage, io, lens, loop, with_mu, H=2, seed=0, tight=None):
     sc = Scene(lla, T=4, H=H, d=128, r_k=r_k, r_v=r_v, storage=storage, io=io, lens=lens,
                seed=seed, with_mu=with_mu, extra_tokens=0)
     W = sc.W
@@ -48,7 +48,7 @@ def _prefill_case(lla, r_k, r_v, storage, io, lens, loop, with_mu, H=2, seed=0):
     assert lla.lla_get_device_error() == 0
     got, q64 = f64(out), f64(q)
     w = sc.w64
-    tight = 1e-5 if storage == "fp32" else 5e-3
+    tight = tight or (1e-5 if storage == "fp32" else 5e-3)
     off = 0
     for b, L in enumerate(lens):
         for h in range(H):
@@ -86,9 +86,16 @@ def test_prefill_long_prompt_rescales(lla):
     _prefill_case(lla, 96, 160, "bf16", "bf16", [1500], 3, False, H=1, seed=5)
 
 
-def test_prefill_cuda_core_ranks(lla):
-    # r = (72, 120): not multiples of 32
+def test_prefill_tensor_core_ranks_in_parts(lla):
+    # r = (72, 120): not multiples of 32, served in three bf16 parts
     _prefill_case(lla, 72, 120, "bf16", "bf16", [70, 5], 1, False)
+
+
+@pytest.mark.parametrize("r_k,r_v,io,tight", [(72, 120, "fp32", 1e-5), (18, 30, "fp32", 1e-5), (40, 56, "fp32", 1e-5),
+                                              (40, 56, "bf16", 2 ** -8)])
+def test_prefill_cuda_core_ranks(lla, r_k, r_v, io, tight):
+    # bf16 storage on the CUDA cores: fp32 queries at the ranks that take parts, and any other ranks
+    _prefill_case(lla, r_k, r_v, "bf16", io, [140, 70, 5], 1, True, tight=tight)
 
 
 def test_prefill_fp32_storage(lla):
@@ -190,3 +197,67 @@ def test_prefill_in_parts_is_as_exact_as_the_cuda_cores(lla, r_k, r_v):
     assert lla.lla_get_device_error() == 0
     moved = (out != ref.to(torch.bfloat16)).float().mean().item()
     assert moved <= 1e-3, moved
+
+
+def _stepped_scores_case(lla, r_k, r_v, H, lens):
+    """Scores that step up every third page and are equal within a step: only coordinate 0 of the K latents is
+    not zero, and it holds the step.  Even rows' steps are 16 in the exp2 domain, past the rescale threshold
+    (8), odd rows' are 4.  A row's output is then the mean of the V latents of its last step, and of those
+    before it by 2^-16 or 2^-4 a step, so that a page that is lost or counted twice moves it by 1 / 3 of a
+    value.  The step itself is off by 2^-9 (q~ in bf16), which moves the weight of the steps before by 3 %
+    of 1 / 16 at most; weights and outputs are rounded by up to 2^-8 each."""
+    g = torch.Generator(device=DEV).manual_seed(35)
+    geom, d, T = lla.Geometry(1, H, 128, r_k, r_v), 128, 1
+    w_k = torch.zeros(H, T, d, r_k, device=DEV, dtype=torch.bfloat16)
+    w_k[..., 0] = 1 / 128  # q~_0 is the mean of q
+    w_v = torch.zeros(H, T, d, r_v, device=DEV, dtype=torch.bfloat16)
+    w_v[:, 0, torch.arange(min(d, r_v)), torch.arange(min(d, r_v))] = 1  # o is the mean of the V latents
+    codec = lla.Codec(None, None, w_k, w_v)
+    pages = [-(-L // 64) for L in lens]
+    table = torch.full((len(lens), max(pages)), -1, dtype=torch.int32, device=DEV)
+    perm = torch.randperm(sum(pages), generator=g, device=DEV).to(torch.int32)
+    e = 8 if r_k % 8 == 0 else 2
+    pool = torch.full((sum(pages), H, 64 * (r_k + r_v)), float("nan"), device=DEV, dtype=torch.bfloat16)
+    cv, o = [], 0
+    for b, n in enumerate(pages):
+        blk = perm[o:o + n]
+        table[b, :n] = blk
+        o += n
+        v = torch.randn(n, H, 64, r_v, generator=g, device=DEV).to(torch.bfloat16)
+        k = torch.zeros(n, H, r_k // e, 64, e, device=DEV, dtype=torch.bfloat16)
+        k[:, :, 0, :, 0] = (torch.arange(n, device=DEV) // 3).view(n, 1, 1).to(torch.bfloat16)
+        pool[blk.long()] = torch.cat([k.reshape(n, H, -1), v.reshape(n, H, -1)], 2)
+        cv.append(v.permute(1, 0, 2, 3).reshape(H, n * 64, r_v)[:, :lens[b]].double())
+    N = sum(lens)
+    step = torch.tensor([16.0, 4.0], device=DEV)[torch.arange(N, device=DEV) % 2]
+    q = (step * math.log(2) * math.sqrt(d)).view(N, 1, 1).expand(N, H, d).to(torch.bfloat16).contiguous()
+    out = torch.full_like(q, float("nan"))
+    cu = torch.tensor(np.cumsum([0] + list(lens)), dtype=torch.int32, device=DEV)
+    lla.lla_prefill_attn(geom, codec, lla.Cache(pool, sum(pages), table, max(pages)), cu, max(lens), 0, q, out)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    off, cols = 0, min(d, r_v)
+    for b, L in enumerate(lens):
+        i = torch.arange(L, device=DEV)
+        s = (i // 192).double()[None] * (q[off:off + L, 0, 0].double() / math.sqrt(d))[:, None]
+        p = torch.softmax(s.masked_fill(i[None] > i[:, None], -math.inf), 1)
+        ref = (p @ cv[b])[..., :cols].permute(1, 0, 2)
+        err = (out[off:off + L, :, :cols].double() - ref).abs()
+        # per output: its own rounding and the weights' (2^-8 each, of the values' weighted size), and 3 % of what
+        # the steps before the last contribute to odd rows (1 / 16 of their size at most)
+        size = (p @ cv[b].abs())[..., :cols].permute(1, 0, 2)
+        bound = size * (2 * 2 ** -8 + 0.03 / 16) + 1e-6
+        assert (err <= bound).all(), (b, (err / bound).max().item())
+        off += L
+
+
+@pytest.mark.parametrize("r_k,r_v,H,lens", [
+    (96, 160, 2, [1000, 577]),                                    # one tile per CTA: the groups take turns
+    (192, 320, 2, [700]),
+    (72, 120, 2, [700, 321]),                                     # three bf16 parts
+    (18, 30, 2, [700, 321]),
+    (96, 160, 16, [1030, 1000, 900, 770, 500, 257, 129, 63]),     # 5 pairs x 8 x 16 = 640: two tiles per CTA
+    (128, 128, 16, [1030, 1000, 900, 770, 500, 257, 129, 63]),
+])
+def test_prefill_stepped_scores(lla, r_k, r_v, H, lens):
+    _stepped_scores_case(lla, r_k, r_v, H, lens)

@@ -16,7 +16,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import assert_parity, ensure_library, f64, rel_l2
+from helpers import assert_parity, bf16_half_ulp, ensure_library, f64, rel_l2
 from test_decode_gpu import Scene
 
 pytestmark = pytest.mark.gpu
@@ -124,4 +124,30 @@ def test_rope_prefill_two_tiles_per_cta(lla, rk, rv):
             ref = oracle.prefill_rope(loop, gk, gv, w["w_up_k"][h], w["w_up_v"][h], w["mu_k"][h], w["mu_v"][h],
                                       q64[off:off + L, h], sc.scale, base, 1)
             assert rel_l2(got[off:off + L, h], ref) <= 5e-3, (b, h)
+        off += L
+
+
+def test_rope_prefill_two_tiles_per_cta_equal_weights(lla):
+    """q = 0: every weight is 1, exactly, and a row's output is the mean of its values up to the bf16 rounding of
+    the output and fp32 sums, so that a page lost from or counted twice in a row of n pages moves it by 1 / n.
+    3 pairs of tiles x 15 prompts x 16 heads take two tiles per CTA."""
+    lens, H = [720, 585, 384, 300, 257, 256, 200, 129, 128, 127, 65, 64, 63, 2, 1], 16
+    sc = Scene(lla, T=4, H=H, d=128, r_k=96, r_v=160, storage="bf16", io="bf16", lens=lens, seed=85, with_mu=True,
+               extra_tokens=0)
+    q = torch.zeros((sum(lens), H, 128), dtype=torch.bfloat16, device=DEV)
+    out = torch.full_like(q, float("nan"))
+    cu = torch.tensor(np.cumsum([0] + lens), dtype=torch.int32, device=DEV)
+    ws = torch.empty(lla.lla_prefill_rope_workspace_size(sc.geom, len(lens), max(lens)), dtype=torch.uint8, device=DEV)
+    lla.lla_prefill_attn_rope(sc.geom, sc.codec, sc.cache, 10000.0, 0, cu, max(lens), 1, q, out, ws)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    got, off = f64(out), 0
+    for b, L in enumerate(lens):
+        for h in range(H):
+            _, cv = sc.gpu_latents(b, h)
+            mean = np.cumsum(cv, 0) / np.arange(1, L + 1)[:, None]
+            ref = mean @ sc.w64["w_up_v"][h][1].T + sc.w64["mu_v"][h].reshape(4, 128)[1]
+            dev = np.abs(got[off:off + L, h] - ref)
+            # the output's rounding; O / l enters the projection as two bf16 parts (2^-17 of each of 160 terms)
+            assert (dev <= bf16_half_ulp(ref) + 2e-4).all(), (b, h, dev.max())
         off += L

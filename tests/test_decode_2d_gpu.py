@@ -327,3 +327,28 @@ def test_encode_2d_on_tensor_cores(lla, H, r_k, r_v, lens, with_mu):
         gk, gv = s.gpu_latents(b)
         assert_parity(gk, s.ck[b], "bf16", f"c_k {b}")
         assert_parity(gv, s.cv[b], "bf16", f"c_v {b}")
+
+
+@pytest.mark.parametrize("rk,rv", [(96, 160), (288, 480)])
+def test_maxima_that_rise_after_the_first_page(lla, rk, rv):
+    """Runs of several pages whose scores grow by the page, heads' queries 0, 0.2, 1 and 4 times N(0, 1) in
+    turn: on most pages some heads pass the rescale threshold (2^8) and others do not.  Against the oracle on
+    the stored latents, relative L2 <= 5e-3 (p is rounded to bf16)."""
+    lens = [1300, 1290, 1217, 1100, 640, 577, 130, 65] * 6
+    sc = Scene2D(lla, H=8, r_k=rk, r_v=rv, io="fp32", lens=lens, seed=78, with_mu=True, oracle_encode=False)
+    N = sum(lens)
+    grow = torch.cat([1 + 2 * torch.arange(L, device=DEV) / 64 for L in lens]).view(1, N, 1, 1)
+    slots = torch.cat([sc.pt.slots(b, range(L)) for b, L in enumerate(lens)]).to(DEV)
+    lla.lla_encode_2d(sc.geom, sc.codec, sc.cache, (sc.x_k * grow).contiguous(), sc.x_v, slots)
+    q = sc.W.normal((sc.B, 8, 128), 78, 95, dtype=torch.float32, device=DEV)
+    q = (q * torch.tensor([0, 0.2, 1, 4] * 2, device=DEV).view(1, 8, 1)).contiguous()
+    out = torch.empty_like(q)
+    lla.lla_decode_attn_2d(sc.geom, sc.codec, sc.cache, torch.tensor(lens, dtype=torch.int32, device=DEV), max(lens), 1, q,
+                           None, None, out, sc.ws)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    for b in (0, 4, 7, 26, 47):
+        ref = sc.oracle_decode(1, q, None, None, b)
+        got = f64(out[b])
+        for h in range(8):
+            assert rel_l2(got[h], ref[h]) <= 5e-3, (b, h, rel_l2(got[h], ref[h]))

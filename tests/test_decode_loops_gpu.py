@@ -113,3 +113,29 @@ def test_pass1_empty_cache_returns_current_values(lla):
     sc = Scene(lla, lens=[0, 0], io="fp32", seed=54)
     q, ck, cv, out, ws = _run_loops(sc, True)
     torch.testing.assert_close(out, cv, rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("rk,rv", [(96, 160), (72, 120), (192, 320)])
+def test_maxima_that_rise_after_the_first_page(lla, rk, rv):
+    """Runs of several pages whose scores grow by the page: loop t's queries are 0, 0.2, 1 and 4 times N(0, 1),
+    so that on most pages some of a unit's queries pass the rescale threshold (2^8) and others do not, and
+    the zero queries never.  Against the oracle on the stored latents, fp32 outputs: relative L2 <= 1e-4."""
+    lens = [1300, 1290, 1217, 1100, 640, 577, 130, 65] * 2
+    sc = Scene(lla, H=4, r_k=rk, r_v=rv, io="fp32", lens=lens, seed=56, with_mu=True)
+    W, N = sc.W, sum(lens)
+    grow = torch.cat([1 + 2 * torch.arange(L, device=DEV) / 64 for L in lens]).view(1, N, 1, 1)
+    lla.lla_encode(sc.geom, sc.codec, sc.cache, (sc.x_k * grow).contiguous(), sc.x_v, sc.slots)
+    shape = (sc.T, sc.B, sc.H, sc.d)
+    q = W.normal(shape, 56, 95, dtype=torch.float32, device=DEV) * torch.tensor([0, 0.2, 1, 4], device=DEV).view(4, 1, 1, 1)
+    out = torch.empty(shape, device=DEV)
+    ws = torch.full((lla.lla_decode_loops_workspace_size(sc.geom, sc.B),), 0xFF, dtype=torch.uint8, device=DEV)
+    lla.lla_decode_attn_loops(sc.geom, sc.codec, sc.cache, torch.tensor(lens, dtype=torch.int32, device=DEV), max(lens), q,
+                              None, None, out, ws)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    for b in (0, 1, 4, 7, 11, 15):
+        for h in range(sc.H):
+            latents = sc.gpu_latents(b, h)
+            for t in range(sc.T):
+                ref = sc.oracle_decode(t, q[t], None, None, b, h, latents=latents)
+                assert rel_l2(f64(out[t, b, h]), ref) <= 1e-4, (b, h, t, rel_l2(f64(out[t, b, h]), ref))

@@ -674,7 +674,7 @@ def run_extras(device):
     enc_flops = 2.0 * N * H * T * d * (w.r_k + w.r_v)
     out["encode_prefill"] = {
         "workload": f"{w.name} prompt encode, {nseq}x{L} tokens, H={H}, (r_k, r_v)=({w.r_k}, {w.r_v})",
-        "kernel": "encode_kernel (lla_encode)", "ms_per_call": enc_ms,
+        "kernel": "encode_tc_kernel (lla_encode)", "ms_per_call": enc_ms,
         "GB_s": enc_bytes / (enc_ms / 1e3) / 1e9, "hbm_frac": enc_bytes / (enc_ms / 1e3) / 1e9 / hbm,
         "TFLOP_s": enc_flops / (enc_ms / 1e3) / 1e12,
         "tensor_frac": enc_flops / (enc_ms / 1e3) / 1e12 / tc_peak,
@@ -1019,7 +1019,7 @@ def run_rho2_as_written(device, steps=None):
         "decode_kernel_hbm_frac": dec_bytes / dec_kernel_s / 1e9 / peak,
         "total_s": (pf_ms + dec_total_ms) / 1e3,
         "kernels": "encode_tc_kernel + prefill_tc_kernel (lla_prefill_two_pass); decode_async_kernel + "
-                   "encode_layers_kernel (decode steps)"}}
+                   "encode_step_kernel (decode steps)"}}
 
 
 def run_long_prompt(device, L=65536, rope=False):

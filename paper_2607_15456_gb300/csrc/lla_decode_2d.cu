@@ -28,8 +28,9 @@
 //                       warp 6     O^T issuer: M = 128 latent rows per chunk, N = 16 (the p
 //                                  parts of the queries, padded with zero rows of P^T), K = 64
 //                                  tokens; the swizzled V-plane is an MN-major A operand.  Two
-//                                  issuing threads, because an MMA takes its issuing thread tens
-//                                  of cycles
+//                                  issuers, so that neither product waits behind the other's
+//                                  barriers; whole warps with one elected thread for the loops,
+//                                  one thread each for LLA-2D
 //                       warps 2-5  per page: the scores of 16 tokens per warp, the maxima over
 //                                  the page per query, P^T as a bf16 operand, the lazy O^T
 //                                  rescale; per run: the partial out to the workspace
@@ -249,6 +250,8 @@ __global__ void __launch_bounds__(256) absorb2d_kernel(const A2Params p) {
     auto iorow = [&](int b) { return ((p.loops ? static_cast<int64_t>(t) * p.B : 0) + b) * p.H + h; };
     const int col = j0 + lane;
     pdl_wait();  // the codec and the queries may come from the previous kernel; the workspace is free after it
+    // The attention kernel may start: once every CTA is here the caller's previous kernel is complete, so its
+    // producers may read any input of the call, and q~, beta and the workspace only after their own wait.
     pdl_trigger();
     // this thread's 16 weights: column j0 + lane, rows 16 warp .. 16 warp + 15
     const uint16_t *W = static_cast<const uint16_t *>(p.w_up_k) + th * kD * RK + col;
@@ -287,11 +290,6 @@ __global__ void __launch_bounds__(256) absorb2d_kernel(const A2Params p) {
             if (lane == 0) p.beta[static_cast<int64_t>(unit(b0 + bi)) * NQ + n] = s * p.scale_log2;
         }
     }
-    // (triggering the attention kernel's launch right after the wait, so that its set-up could
-    // overlap this kernel where their CTAs fit one SM, gained 2 % at rho = 4 and lost 10 % on the
-    // Ouro-2.6B batch)
-    __syncthreads();
-    pdl_trigger();
 }
 
 // ------------------------------------------------------------------------- attention kernel

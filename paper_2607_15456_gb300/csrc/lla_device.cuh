@@ -140,8 +140,8 @@ __device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// Programmatic dependent launch: wait for the previous grid in the stream to complete (or to
-// trigger), and allow the next grid to be scheduled.  Both are no-ops without the attribute.
+// Programmatic dependent launch: wait until the previous grid in the stream is complete and its writes
+// are visible, and allow the next grid to be scheduled.  Both are no-ops without the attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

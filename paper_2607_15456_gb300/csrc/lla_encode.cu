@@ -15,9 +15,11 @@
 // about one memory round trip.  256 threads are 16 column pairs x 4 groups of 4 tokens x 4
 // slices of the reduction axis; the 4 partial sums per output meet in shared memory.
 //
-// bf16 x and storage go to the tensor cores instead: a decode step's tokens to lla_encode_step.cu,
-// prompts and LLA-2D to lla_encode_tc.cu.  This kernel takes fp32 x or storage and head widths that
-// are not multiples of 32.
+// bf16 x and storage go to the tensor cores instead: a decode step's tokens (T*d below 4096, up to 64
+// tokens, or 256 where tokens x ranks stay below 32768) to lla_encode_step.cu, prompts and LLA-2D to
+// lla_encode_tc.cu.  This kernel takes fp32 x or storage, head widths that are not multiples of 32 (64 for
+// prompts), prompts whose ranks are not both multiples of 8 unless both are at most 64 and T*d at most
+// 512, and the stacks and ranks that kernel has no room for.
 #include <cuda_runtime.h>
 
 #include "lla_device.cuh"

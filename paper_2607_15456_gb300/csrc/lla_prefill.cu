@@ -61,6 +61,7 @@
 #include "lla_internal.h"
 #include "lla_tcgen05.cuh"
 #include "lla_tmap.h"
+#include "lla_units.cuh"
 
 namespace lla {
 namespace {
@@ -95,6 +96,7 @@ struct PParams {
     int kpps;
     int64_t qrows;  // rows of the rotated-query buffer (B * max_len)
     int B, first;   // prompts; (head, prompt) pairs that run one after the other, before the last ones together
+    FastDiv by_tiles, by_rest, by_prompts;  // by the tiles of a pair, the pairs that run together, the prompts
 };
 
 // Shared-memory and TMEM plan of the tensor-core kernel for ranks (RK, RV), d = 128, NT query tiles
@@ -233,14 +235,14 @@ __global__ void __launch_bounds__(kPThreads, 1)
     const int nqt = (p.max_len + NT * kBM - 1) / (NT * kBM);
     int qt = blockIdx.x, b = blockIdx.y, h = blockIdx.z;
     if (p.first >= 0) {  // pair after pair, then tile by tile every pair of the rest
-        int pair = blockIdx.x / nqt;
+        int pair = div_by(blockIdx.x, p.by_tiles);
         qt = blockIdx.x - pair * nqt;
         if (pair >= p.first) {
-            const int r = blockIdx.x - p.first * nqt, n = p.H * p.B - p.first;
-            qt = r / n;
-            pair = p.first + r - qt * n;
+            const int r = blockIdx.x - p.first * nqt;
+            qt = div_by(r, p.by_rest);
+            pair = p.first + r - qt * (p.H * p.B - p.first);
         }
-        h = pair / p.B;
+        h = div_by(pair, p.by_prompts);
         b = pair - h * p.B;
     }
     qt = nqt - 1 - qt;  // longest causal ranges first
@@ -1390,6 +1392,11 @@ lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t 
         const int64_t pair_bytes = static_cast<int64_t>(a.max_len) * ((ROPE ? F::D : RK) + RV) * 2;
         const int64_t last = std::max<int64_t>((3ll * sms + tiles - 1) / tiles, (64ll << 20) / pair_bytes);
         prm.first = static_cast<int>(std::max<int64_t>(0, pairs - last));
+        // divisions by multiplication: a tile past its prompt is little else (32 prompts of 100 tokens at
+        // (192, 320), launched for 8192 each: 212 us with divisions, 187 so)
+        prm.by_tiles = fast_div(tiles);
+        prm.by_rest = fast_div(static_cast<uint32_t>(pairs - prm.first));
+        prm.by_prompts = fast_div(a.B);
         cfg.gridDim = dim3(static_cast<unsigned>(pairs * tiles));
     }
     cfg.blockDim = dim3(kPThreads);
@@ -1415,7 +1422,10 @@ lla_status launch_tiles(const PParams &prm0, const PrefillArgs &a, cudaStream_t 
 // From 160 to 400 pairs the two come within a few percent where the prompts differ in length (4 x 700 to
 // 1050 tokens, 256 pairs, 35 and 36; 8 x 64 to 2048, 384 pairs of which half exist, 25 and 28), so that
 // two start above that; with rotated keys those two cases take 63 and 61, 50 and 51, and two start at 256.
-// Prompts of one tile leave the second empty (32 x 100: 34 and 37).  With two bf16 parts the products bound
+// Prompts of one tile leave the second empty (32 x 100: 34 and 37).  The pairs are counted from max_len, an
+// upper bound; where it is far above the prompts, half as many CTAs past their ends weigh more than empty
+// tiles (one and two tiles: 32 x 100 tokens under max_len 1024 47 and 40, 8192 179 and 109; 8 x 500 to 900
+// under 8192 91 and 78; rotated keys, 16 x 100 under 4096 94 and 76).  With two bf16 parts the products bound
 // it either way (2 x 8192 at (72, 120): 630 and 644), and three leave no TMEM for a second O: one tile.
 template <int RK, int RV, bool ROPE, int QP = 1>
 lla_status launch_tc(const PParams &prm, const PrefillArgs &a, cudaStream_t stream) {

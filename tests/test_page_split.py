@@ -77,3 +77,47 @@ def test_page_split_tiles_the_pages_and_cta_of_inverts_it():
         assert r.returncode == 0, r.stderr[-3000:]
         r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
         assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout[-2000:]
+
+
+DIVISIONS = r"""
+#include <cstdio>
+#include "lla_units.cuh"
+
+int main() {
+    int fails = 0;
+    auto check = [&](uint32_t d) {
+        const lla::FastDiv f = lla::fast_div(d);
+        auto one = [&](int64_t x) {
+            if (x < 0 || x > 2147483647 || lla::div_by(static_cast<int>(x), f) == x / d) return;
+            if (fails++ < 10) std::printf("%lld / %u\n", (long long)x, d);
+        };
+        for (int64_t x = 0; x < 3000; ++x) one(x);
+        for (int64_t k = 1; k * d <= 2147483647; k += 1 + k / 64)  // both sides of multiples, over the range
+            for (int e = -1; e <= 1; ++e) one(k * d + e);
+        for (int64_t x = 2147483647; x > 2147483647ll - 300; --x) one(x);
+    };
+    for (uint32_t d = 1; d <= 5000; ++d) check(d);
+    for (uint64_t d = 5001; d < (1ull << 31); d += d / 16) check(static_cast<uint32_t>(d));
+    for (int b = 13; b < 31; ++b)
+        for (int e = -1; e <= 1; ++e) check((1u << b) + e);
+    check(2147483647u);
+    std::printf("%s\n", fails ? "FAILED" : "ok");
+    return fails ? 1 : 0;
+}
+"""
+
+
+def test_division_by_multiplication_is_exact():
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    with tempfile.TemporaryDirectory() as tmp:
+        src, exe = os.path.join(tmp, "div_check.cu"), os.path.join(tmp, "div_check")
+        with open(src, "w") as f:
+            f.write(DIVISIONS)
+        r = subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17",
+                            "-I", CSRC, "-I", os.path.join(ROOT, "include"), src, "-o", exe],
+                           capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr[-3000:]
+        r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout[-2000:]

@@ -6,7 +6,7 @@ L2 <= 5e-3; fp32 storage and fp32 x: relative L2 <= 1e-5).  The cases reach the 
 separate code paths: a reduction axis T*d longer than one shared-memory chunk of W_down (fp32
 and bf16), ranks whose rows are not a multiple of 16 bytes (4-byte copies), token counts that
 leave a ragged last tile, x in bf16 and fp32, with and without mu, a decode-step batch, and
-prompts of 128 tokens or more in bf16, which take the tensor-core kernel.
+prompts of more than 64 tokens (or 256, at small ranks) in bf16, which take the tcgen05 kernel.
 """
 import numpy as np
 import pytest
@@ -265,3 +265,31 @@ def test_encode_2d_long_sums_are_as_exact_as_fp32(lla, with_mu):
         want = (s @ wa.double()).to(torch.bfloat16)
         wrong += int((torch.from_numpy(got).to(DEV) != want.double()).sum())
     assert wrong <= 3e-4 * N * (r_k + r_v), wrong
+
+
+@pytest.mark.parametrize("d,r_k,r_v,lens,with_mu", [(72, 40, 56, [20, 3], True), (128, 100, 100, [300], True),
+                                                    (40, 18, 30, [130], False)])
+def test_encode_bf16_on_the_cuda_cores(lla, d, r_k, r_v, lens, with_mu):
+    # what the tensor-core kernels leave: head widths that are not multiples of 32 (64 for prompts), and prompts
+    # whose ranks are neither multiples of 8 nor small
+    _encode_and_compare(lla, 4, 3, d, r_k, r_v, "bf16", "bf16", lens, with_mu, 19)
+
+
+def test_encode_layers_equals_per_layer_calls_on_the_cuda_cores(lla):
+    T, H, d, r_k, r_v, L, N = 4, 2, 72, 40, 56, 3, 16
+    g = torch.Generator(device=DEV).manual_seed(20)
+    rand = lambda *s: torch.randn(s, generator=g, device=DEV).to(torch.bfloat16)
+    geom = lla.Geometry(T, H, d, r_k, r_v)
+    bb, slots = lla.lla_cache_block_bytes(geom), torch.arange(N, device=DEV)
+    codecs = [lla.Codec(rand(H, T * d, r_k), rand(H, T * d, r_v), None, None, rand(H, T * d).float() if l == 1 else None)
+              for l in range(L)]
+    x = [[rand(T, N, H, d) for _ in range(L)] for _ in range(2)]
+    pools = [[torch.full((bb,), 0xFF, dtype=torch.uint8, device=DEV) for _ in range(L)] for _ in range(2)]
+    caches = [[lla.Cache(p, 1, None, 1) for p in ps] for ps in pools]
+    lla.lla_encode_layers(geom, codecs, caches[0], x[0], x[1], slots)
+    for l in range(L):
+        lla.lla_encode(geom, codecs[l], caches[1][l], x[0][l], x[1][l], slots)
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    for a, b in zip(*pools):
+        assert torch.equal(a, b)

@@ -37,7 +37,7 @@ layer near 1 GB, above L2; the (1152, 1920) workload's 16 sequences take 351 MB 
         python profile_case.py --case 2d --workload2d ouro14_2d_rho533 --batch 16 --calls 6
 
 prefill: encodes `--prompts` prompts of `--len` tokens of a workload's ranks (tensor-core encode,
-one launch per axis), then runs `--calls` causal prefill calls over them:
+both axes in one launch), then runs `--calls` causal prefill calls over them:
 
     ncu --set full --clock-control none -k regex:"encode_tc_kernel|prefill_tc_kernel" -c 3 \\
         python profile_case.py --case prefill --workload ouro14_rho2 \\

@@ -293,3 +293,26 @@ def test_encode_layers_equals_per_layer_calls_on_the_cuda_cores(lla):
     assert lla.lla_get_device_error() == 0
     for a, b in zip(*pools):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("N,r_k,r_v", [(20, 96, 160), (200, 96, 160), (200, 18, 30)])
+@pytest.mark.parametrize("axis", ["k", "v"])
+def test_encode_with_mu_of_one_axis(lla, axis, N, r_k, r_v):
+    H, d, T = 2, 128, 4
+    g = torch.Generator(device=DEV).manual_seed(21)
+    rand = lambda *s: torch.randn(s, generator=g, device=DEV)
+    geom = lla.Geometry(T, H, d, r_k, r_v)
+    pages = -(-N // 64)
+    pool = torch.zeros(pages * lla.lla_cache_block_bytes(geom), dtype=torch.uint8, device=DEV)
+    w = {a: (rand(H, T * d, r) * (T * d) ** -0.5).to(torch.bfloat16) for a, r in (("k", r_k), ("v", r_v))}
+    x = {a: rand(T, N, H, d).to(torch.bfloat16) for a in "kv"}
+    mu = rand(H, T * d)
+    codec = lla.Codec(w["k"], w["v"], None, None, mu if axis == "k" else None, mu if axis == "v" else None)
+    lla.lla_encode(geom, codec, lla.Cache(pool, pages, None, 1), x["k"], x["v"], torch.arange(N, device=DEV))
+    torch.cuda.synchronize()
+    assert lla.lla_get_device_error() == 0
+    pool_cpu = pool.cpu()
+    for h in range(H):
+        for a, got in zip("kv", unpack_head(pool_cpu, H, r_k, r_v, "bf16", list(range(pages)), N, h)):
+            want = oracle.encode(f64(x[a])[:, :, h], f64(mu[h]) if a == axis else None, f64(w[a][h]))
+            assert_parity(got, want, "bf16", f"{a} head {h}", io="bf16")
